@@ -522,7 +522,7 @@ int flood_ensemble_init(flood_grid* g, int M, const float* h0, int h0_per_member
         (rc = dalloc(g, &g->w_post, M)) || (rc = dalloc(g, &g->ms, (size_t)3 * M)) ||
         (rc = dalloc(g, &g->vacc, (size_t)M * g->nslot * 2)) || (rc = dalloc(g, &g->rain_acc, M)) ||
         (rc = dalloc(g, &g->inflow_acc, M)) ||
-        (rc = dalloc(g, &g->beta, M)) || (rc = dalloc(g, &g->pfi, (size_t)5 * M)) ||
+        (rc = dalloc(g, &g->beta, M)) || (rc = dalloc(g, &g->pfi, (size_t)4 * M)) ||
         (rc = dalloc(g, &g->pf_small, 4)) || (rc = dalloc(g, &g->neff, 1)) ||
         (rc = dalloc(g, &g->part, (size_t)M * g->part_cap)) || (rc = dalloc(g, &g->storage, M)) ||
         (rc = dalloc(g, &g->plan, M))) {
@@ -691,9 +691,8 @@ int pf_assimilate(flood_grid* g, int G, const float* y, const double* d, const d
     a.status = g->pf_small + 2;
     a.idx = g->pfi;
     a.src = g->pfi + M;
-    a.cnt = g->pfi + 2 * M;
-    a.copy_dst = g->pfi + 3 * M;
-    a.copy_src = g->pfi + 4 * M;
+    a.copy_dst = g->pfi + 2 * M;
+    a.copy_src = g->pfi + 3 * M;
     a.rain_mult = g->rain_mult;
     a.scale = g->scale;
     a.ms = g->ms + (g->k % 3) * M;

@@ -50,7 +50,7 @@ struct flood_grid {
     double* d = nullptr;          // [G_cap]
     double* sigma = nullptr;      // [G_cap]
     float* beta = nullptr;        // [M]
-    int32_t* pfi = nullptr;       // idx, src, cnt, copy_dst, copy_src: 5 x [M]
+    int32_t* pfi = nullptr;       // idx, src, copy_dst, copy_src: 4 x [M]
     int32_t* pf_small = nullptr;  // n_copy, resampled, status
     double* neff = nullptr;       // [1]
     double* part = nullptr;       // storage partials

@@ -21,7 +21,6 @@ struct PfArgs {
     int32_t* status;       // [1] 1: every posterior weight was zero
     int32_t* idx;          // [M] resampled indices
     int32_t* src;          // [M] particle held by each slot afterwards
-    int32_t* cnt;          // [M] scratch: duplicates per particle
     int32_t* copy_dst;     // [M] slots to overwrite
     int32_t* copy_src;     // [M] their sources
     int32_t* n_copy;       // [1]

@@ -250,3 +250,45 @@ def test_resume_at_a_window_boundary_is_bit_exact(capi):
             assert np.array_equal(got[m][k], want[m][k]), (m, k)
     assert np.array_equal(got_mem["t"], want_mem["t"])
     assert np.array_equal(got_mem["weights"], want_mem["weights"])
+
+
+@pytest.mark.parametrize("M", [1, 2, 31, 32, 33, 64, 65, 255, 256, 257, 3072])
+def test_filter_block_at_the_edges_of_its_warps(capi, M):
+    """The one-block filter over member counts around its warp and block
+    sizes and at its largest: weights against the oracle, indices the
+    sequential definition's on those weights (bit for bit), slots and
+    parameters exact; more members than its shared memory holds are refused."""
+    ny, nx, G = 3, 5, 3
+    rng = np.random.default_rng(M)
+    z = np.zeros((ny, nx), np.float32)
+    n = np.full((ny, nx), 0.05, np.float32)
+    h0 = rng.uniform(0.05, 0.15, (M, ny, nx)).astype(np.float32)
+    rm, sc = synth.ensemble_prior(M, M)
+    with capi.Grid(z, n) as g:
+        g.ensemble_init(M, rm, sc, np.zeros(1, np.float32), h0=h0)
+        y = rng.uniform(0.0, 0.3, (M, G)).astype(np.float32)
+        d = rng.uniform(0.1, 0.2, G)
+        u, beta = synth.pf_draws(M, 1, M)
+        pf = g.pf_assimilate(d, 0.05, u, beta, y=y, force=True)
+        mem = g.members()
+        after = [g.get_state(m)[0] for m in (0, M // 2, M - 1)]
+    w_o, neff_o = oracle.pf_weights(y.astype(np.float64), d, np.full(G, 0.05), np.full(M, 1 / M))
+    assert np.allclose(pf["weights"], w_o, rtol=1e-6, atol=1e-300)
+    assert abs(pf["neff"] - neff_o) <= 1e-6 * neff_o and pf["resampled"]
+    assert np.array_equal(pf["idx"], oracle.resample_systematic(pf["weights"], u))
+    src = oracle.assign_slots(pf["idx"])
+    for s, h in zip((0, M // 2, M - 1), after):
+        assert np.array_equal(h, h0[src[s]])
+    assert np.array_equal(mem["rain_mult"], (rm[src] * beta).astype(np.float32))
+    assert np.array_equal(mem["scale"], sc[src])
+    assert np.array_equal(mem["hmax"], h0.max((1, 2))[src])
+
+
+def test_filter_refuses_more_members_than_its_block_holds(capi):
+    M = 3073
+    with capi.Grid(np.zeros((1, 2), np.float32), np.full((1, 2), 0.05, np.float32)) as g:
+        one = np.ones(M, np.float32)
+        g.ensemble_init(M, one, one, np.zeros(1, np.float32))
+        with pytest.raises(capi.FloodError) as e:
+            g.pf_assimilate(np.array([0.1]), 0.05, 0.5, one, y=np.zeros((M, 1), np.float32))
+        assert e.value.code == -2
