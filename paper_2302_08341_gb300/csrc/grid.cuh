@@ -116,7 +116,8 @@ struct flood_grid {
                                   // the drainage flag
     double* gdpart = nullptr;     // [M][nslot] drainage-rate gradient partials
     std::vector<double> adj_gdrain;  // [M] dL/d(drainage rate) of the last adjoint
-    double* lc_cgrad = nullptr;   // [M][4] per-class Manning gradients of the last adjoint
+    double* lc_cgrad = nullptr;   // [M][4] per-class Manning gradients of the last adjoint,
+                                  // then the parts they are summed from
     double* lc_dgrad = nullptr;   // [M] drainage-rate gradients (device copy, calibration)
     // inflow hydrograph (inflow.cu)
     float* inflow = nullptr;      // [inflow_blocks] discharge per rain block (m^3/s)

@@ -63,25 +63,41 @@ __global__ void land_adjoint_fields_kernel(float* __restrict__ out, const float*
     }
 }
 
-// dL_m/dn of each class for member m (one CTA per member): the per-cell
-// Manning gradients of the member summed over the cells of each class, in
-// FP64 and a fixed order (deterministic).
+// dL_m/dn of each class for member m: the per-cell Manning gradients of the
+// member summed over the cells of each class, in FP64 and a fixed order
+// (deterministic): kGradParts CTAs per member sum a share of its rows each, a
+// warp per member then adds the CTAs' sums.  Bound by the narrow FP64 pipe
+// (an addition per cell and class present among a warp's 128 cells), so a
+// class that no lane holds is skipped and the sum is spread over the whole
+// chip; the padding's gradients are zero, so whole padded rows are read as
+// float4.  600 x 707 cells x 8 members: 1210 us with one CTA per member.
 constexpr int kGradThreads = 256;
+constexpr int kGradParts = 128;
 
-__global__ void __launch_bounds__(kGradThreads) land_class_grad_kernel(
-    const float* __restrict__ gnm, const uint8_t* __restrict__ cls, int ny, int nx, int ld,
-    size_t plane, double* __restrict__ out)
+__global__ void __launch_bounds__(kGradThreads) land_class_part_kernel(
+    const float* __restrict__ gnm, const uint8_t* __restrict__ cls, size_t plane,
+    double* __restrict__ part)
 {
-    const int m = blockIdx.x;
+    const int m = blockIdx.y, b = blockIdx.x;
     const float* g = gnm + (size_t)m * plane;
     double acc[kMaxClasses] = {0.0, 0.0, 0.0, 0.0};
-    const size_t cells = (size_t)ny * nx;
-    for (size_t i = threadIdx.x; i < cells; i += kGradThreads) {
-        const size_t o = (i / nx) * ld + i % nx;
-        const double v = g[o];
-        const int k = cls[o];
+    const size_t n4 = plane / 4, lo = n4 * b / kGradParts, hi = n4 * (b + 1) / kGradParts;
+    for (size_t i0 = lo; i0 < hi; i0 += kGradThreads) {  // whole warps: the votes below
+        const size_t i = i0 + threadIdx.x;
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        uint32_t w = 0;
+        if (i < hi) {
+            v = __ldg(reinterpret_cast<const float4*>(g) + i);
+            w = __ldg(reinterpret_cast<const uint32_t*>(cls) + i);
+        }
+        const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-        for (int q = 0; q < kMaxClasses; ++q) acc[q] += (k == q) ? v : 0.0;
+        for (int j = 0; j < 4; ++j) {
+            const int k = (w >> (8 * j)) & 0xff;
+#pragma unroll
+            for (int q = 0; q < kMaxClasses; ++q)
+                if (__any_sync(0xffffffffu, k == q)) acc[q] += (k == q) ? (double)vv[j] : 0.0;
+        }
     }
     __shared__ double red[kMaxClasses][kGradThreads];
 #pragma unroll
@@ -93,7 +109,23 @@ __global__ void __launch_bounds__(kGradThreads) land_class_grad_kernel(
             for (int q = 0; q < kMaxClasses; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + w];
         __syncthreads();
     }
-    if (threadIdx.x < kMaxClasses) out[(size_t)m * kMaxClasses + threadIdx.x] = red[threadIdx.x][0];
+    if (threadIdx.x < kMaxClasses)
+        part[((size_t)m * kGradParts + b) * kMaxClasses + threadIdx.x] = red[threadIdx.x][0];
+}
+
+__global__ void land_class_sum_kernel(const double* __restrict__ part, double* __restrict__ out)
+{
+    const int m = blockIdx.x, lane = threadIdx.x;
+    const double* p = part + (size_t)m * kGradParts * kMaxClasses;
+#pragma unroll
+    for (int q = 0; q < kMaxClasses; ++q) {
+        double acc = 0.0;
+#pragma unroll
+        for (int b = 0; b < kGradParts; b += 32) acc += p[(b + lane) * kMaxClasses + q];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (lane == 0) out[(size_t)m * kMaxClasses + q] = acc;
+    }
 }
 
 // Cells of the classes in `mask` (outside the domain) hold no water and no
@@ -116,6 +148,29 @@ __global__ void zero_outside_kernel(float* __restrict__ state, const uint8_t* __
 }
 
 }  // namespace
+
+// Per-class Manning gradients of the last adjoint into g->lc_cgrad.
+static int launch_class_grad(flood_grid* g, cudaStream_t s)
+{
+    const int M = g->M;
+    if (!g->lc_cgrad) {  // the sums, then the CTAs' parts
+        const int rc = flood::dalloc(g, &g->lc_cgrad, (size_t)M * kMaxClasses * (1 + kGradParts));
+        if (rc) return rc;
+    }
+    double* part = g->lc_cgrad + (size_t)M * kMaxClasses;
+    // members along y: at most 65535 a launch
+    for (int m0 = 0; m0 < M; m0 += 65535) {
+        const int n = std::min(M - m0, 65535);
+        land_class_part_kernel<<<dim3(kGradParts, n), kGradThreads, 0, s>>>(
+            g->gnm + (size_t)m0 * g->plane, g->cls8, g->plane,
+            part + (size_t)m0 * kGradParts * kMaxClasses);
+        g->launches++;
+    }
+    land_class_sum_kernel<<<M, 32, 0, s>>>(part, g->lc_cgrad);
+    g->launches++;
+    CK(g, cudaGetLastError());
+    return FLOOD_OK;
+}
 
 namespace flood {
 
@@ -190,18 +245,13 @@ int land_calibration_step(flood_grid* g, const double* loss, const double* rain_
 {
     const int M = g->M;
     const bool classes = g->adj_gn && g->gnm;
-    if (classes && !g->lc_cgrad) {
-        const int rc = dalloc(g, &g->lc_cgrad, (size_t)M * kMaxClasses);
-        if (rc) return rc;
-    }
     if (!g->lc_dgrad) {
         const int rc = dalloc(g, &g->lc_dgrad, (size_t)M);
         if (rc) return rc;
     }
     if (classes) {
-        land_class_grad_kernel<<<M, kGradThreads, 0, s>>>(g->gnm, g->cls8, g->ny, g->nx, g->ld,
-                                                          g->plane, g->lc_cgrad);
-        g->launches++;
+        const int rc = launch_class_grad(g, s);
+        if (rc) return rc;
     }
     CK(g, cudaMemcpyAsync(g->lc_dgrad, g->adj_gdrain.data(), sizeof(double) * M,
                           cudaMemcpyHostToDevice, s));
@@ -437,14 +487,8 @@ extern "C" int flood_adjoint_land_grad(flood_grid* g, double* grad_n_class, doub
     if (!g->adj_gn || !g->gnm)
         return flood::fail(g, FLOOD_ERR_STATE, "the last flood_adjoint was not given grad_n");
     cudaStream_t s = S(stream);
-    if (!g->lc_cgrad) {
-        const int rc = flood::dalloc(g, &g->lc_cgrad, (size_t)M * kMaxClasses);
-        if (rc) return rc;
-    }
-    land_class_grad_kernel<<<M, kGradThreads, 0, s>>>(g->gnm, g->cls8, g->ny, g->nx, g->ld, g->plane,
-                                                      g->lc_cgrad);
-    g->launches++;
-    CK(g, cudaGetLastError());
+    const int rc = launch_class_grad(g, s);
+    if (rc) return rc;
     std::vector<double> h((size_t)M * kMaxClasses);
     CK(g, cudaMemcpyAsync(h.data(), g->lc_cgrad, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, s));
     CK(g, cudaStreamSynchronize(s));

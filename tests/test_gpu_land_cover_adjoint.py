@@ -320,3 +320,27 @@ def test_calibration_step_without_manning_gradients_moves_rain_and_drainage(capi
     assert np.array_equal(n1, n0)
     assert np.allclose(d1, d_or, rtol=2e-7) and np.allclose(rm1, m_or, rtol=2e-7)
     assert np.all(d1 != d0) and np.all(rm1 != rm0)
+
+
+@pytest.mark.parametrize("ny,nx,M", [(1, 2, 1), (3, 5, 2), (17, 129, 1), (40, 300, 1), (33, 1000, 3)])
+def test_class_gradients_are_the_sums_of_the_field(capi, ny, nx, M):
+    """The per-class sums on planes smaller and larger than the number of
+    CTAs that share them: every member's sums against its field (one member's
+    field is grad_n itself; of more members the sums over the members), to
+    FP32's rounding of the field's member sum."""
+    rng = np.random.default_rng(ny * nx)
+    terr = synth.make_terrain(ny, nx, seed=ny, building_frac=0.0)
+    cls = rng.integers(0, 3, (ny, nx)).astype(np.uint8)
+    rm, sc = synth.ensemble_prior(3, M)
+    h0 = rng.uniform(0.1, 0.2, (M, ny, nx)).astype(np.float32)
+    cells = np.array([0, ny * nx - 1], np.int32)
+    with capi.Grid(terr.z, terr.n) as g:
+        g.set_land_cover(cls, synth.LAND_CLASSES)
+        g.ensemble_init(M, rm, np.ones(M, np.float32), synth.hyetograph_constant(30.0, 300.0), h0=h0)
+        out = g.adjoint(cells, np.full((2, 2), 0.1), 4.0, grad_h0=False)
+        gn, _ = g.adjoint_land_grad()
+    f = out["grad_n"].astype(np.float64)
+    for k in range(len(synth.LAND_CLASSES)):
+        tol = 1e-15 * f.size if M == 1 else 2.0 ** -24 * M
+        scale = np.abs(f[cls == k]).sum() + np.abs(gn[:, k]).sum()
+        assert abs(gn[:, k].sum() - f[cls == k].sum()) <= tol * scale + 1e-300
