@@ -51,8 +51,8 @@ __device__ __forceinline__ void finish_task(const BatchArgs& a, MemberClock* ms_
 {
     if (mo.bad) atomicOr(a.err, 1);
     const unsigned hb = __reduce_max_sync(0xffffffffu, mo.bad ? 0u : __float_as_uint(mo.hmax) & 0x7fffffffu);
-    double out_acc = (double)mo.out_s - (double)mo.out_c, clamp_acc = (double)mo.clamp;
-    double drn_acc = LC ? (double)mo.drn_s - (double)mo.drn_c : 0.0;
+    double out_acc = mo.out, clamp_acc = mo.clamp;
+    double drn_acc = LC ? mo.drn : 0.0;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         out_acc += __shfl_xor_sync(0xffffffffu, out_acc, off);
@@ -136,14 +136,12 @@ __global__ void __launch_bounds__(32 * W, 20 / W) batch_tma_kernel(const BatchAr
     k.limiter = a.limiter;
     k.q_in = 0.0f;  // no inflow boundary here
     k.in_r0 = k.in_r1 = 0;
-    uint32_t bar0;
-    unsigned char* my_stages;
-    tma_march_smem(smem_raw, W, w, bar0, my_stages);
+    const TmaSmem sm = tma_march_smem(smem_raw, W, w);
     float* dst = sd.state + (size_t)(1 - p.cur) * 3 * sd.plane;
     LandK lk;
     if (LC) lk = batch_land_k(a.scen + i, p.dr, p.dt, lane);
     MarchOut mo;
-    if (!tma_march<false, LC, LIM>(a.maps + 2 * i, a.maps + 2 * i + 1, p.cur * 3, bar0, my_stages,
+    if (!tma_march<false, LC, LIM>(a.maps + 2 * i, a.maps + 2 * i + 1, p.cur * 3, sm,
                                    dst, nullptr, nullptr, a.err, sd.plane, sd.ny, sd.nx, sd.ld, tk.c0,
                                    tk.r0, tk.r1, lane, k, p.dt_dx, sd.scale, p.dr, a.east_out,
                                    a.south_out, mo, &lk))
@@ -292,7 +290,7 @@ __device__ __forceinline__ bool grid_barrier_plan(const PersistArgs& q, int j, d
 // further task: its barriers may still have a copy in flight).
 template <int LIM, bool LC>
 __device__ __forceinline__ bool persistent_task(const PersistArgs& q, int j, int t, MemberClock* ms_out,
-                                                int lane, uint32_t bar0, unsigned char* my_stages)
+                                                int lane, const TmaSmem& sm)
 {
     const BatchArgs& a = q.a;
     const WarpTask tk = a.tasks[t];
@@ -313,8 +311,8 @@ __device__ __forceinline__ bool persistent_task(const PersistArgs& q, int j, int
     LandK lk;
     if (LC) lk = batch_land_k(a.scen + i, p.dr, p.dt, lane);
     MarchOut mo;
-    const bool ok = tma_march<false, LC, LIM>(a.maps + 2 * i, a.maps + 2 * i + 1, p.cur * 3, bar0,
-                                              my_stages, dst, nullptr, nullptr, a.err, sd.plane,
+    const bool ok = tma_march<false, LC, LIM>(a.maps + 2 * i, a.maps + 2 * i + 1, p.cur * 3, sm,
+                                              dst, nullptr, nullptr, a.err, sd.plane,
                                               sd.ny, sd.nx, sd.ld, tk.c0, tk.r0, tk.r1, lane, k,
                                               p.dt_dx, sd.scale, p.dr, a.east_out, a.south_out, mo,
                                               &lk);
@@ -328,7 +326,7 @@ __device__ __forceinline__ bool persistent_task(const PersistArgs& q, int j, int
     __syncwarp();
     if (lane == 0) {
         fence_proxy_async_smem();
-        for (int s = 0; s < kTmaNS; ++s) mbar_inval(bar0 + 8u * s);
+        for (int s = 0; s < kTmaNS; ++s) mbar_inval(sm.bar0 + 8u * s);
     }
     __syncwarp();
     finish_task<LC, true>(a, ms_out, tk, p, mo, lane);
@@ -344,9 +342,7 @@ __global__ void __launch_bounds__(32 * W, 20 / W) batch_persistent_kernel(const 
     const int lane = threadIdx.x;
     const int w = threadIdx.y;
     const bool first_thread = blockIdx.x == 0 && w == 0 && lane == 0;
-    uint32_t bar0;
-    unsigned char* my_stages;
-    tma_march_smem(smem_raw, W, w, bar0, my_stages);
+    const TmaSmem sm = tma_march_smem(smem_raw, W, w);
     const double t_stop = *a.t_stop;
     int done = 0;
     if (grid_barrier_plan(q, 0, t_stop, &flag_s)) {  // plans step 0
@@ -363,7 +359,7 @@ __global__ void __launch_bounds__(32 * W, 20 / W) batch_persistent_kernel(const 
             const unsigned nw = gridDim.x * W;
             unsigned t = blockIdx.x * W + w;
             while (t < (unsigned)a.ntasks) {
-                if (!persistent_task<LIM, LC>(q, j, (int)t, ms_out, lane, bar0, my_stages)) break;
+                if (!persistent_task<LIM, LC>(q, j, (int)t, ms_out, lane, sm)) break;
                 if (nw >= (unsigned)a.ntasks) break;
                 unsigned d = 0;
                 if (lane == 0) d = atomicAdd(q.task_next + (j & 1), 1u);

@@ -269,6 +269,65 @@ __device__ __forceinline__ float link_q(float h1, float z1, float h2, float z2, 
     return hf > k.h_eps ? qn : 0.0f;
 }
 
+// Two links at once, with the two-wide FP32 instructions (one issue slot for
+// an add, multiply or fused multiply-add on a register pair; each half is
+// rounded as the scalar one): the same operations in the same order as
+// link_q, so the same values bit for bit.  A difference is a fused
+// multiply-add by -1 (exact product), and |q| is taken after the products it
+// enters (their factors are not negative).  up, dn: h1 and h2 times
+// dx / (4 dt), the limiter's bounds, which a cell shares among its links.
+struct Link2K {
+    float2 m1;        // -1, -1
+    float2 ngdt_dx;   // -g dt / dx
+    float2 gdt;
+    float2 sh;        // half the Manning scale
+    float2 p73;       // -7/3
+    float h_eps;
+};
+
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+
+__device__ __forceinline__ Link2K link2_k(const FaceK& k, float s_half)
+{
+    return Link2K{dup2(-1.0f), dup2(-k.gdt_dx), dup2(k.gdt), dup2(s_half), dup2(-2.33333333f), k.h_eps};
+}
+
+template <int LIM>
+__device__ __forceinline__ float2 link2_q(float2 h1, float2 z1, float2 h2, float2 z2, float2 q,
+                                          float2 nsum, float2 up, float2 dn, const Link2K& k)
+{
+    const float2 dz = __ffma2_rn(z1, k.m1, z2);
+    const float2 a1 = __ffma2_rn(make_float2(fmaxf(dz.x, 0.0f), fmaxf(dz.y, 0.0f)), k.m1, h1);
+    const float2 a2 = __fadd2_rn(h2, make_float2(fminf(dz.x, 0.0f), fminf(dz.y, 0.0f)));
+    const float2 hf = make_float2(fmaxf(a1.x, a2.x), fmaxf(a1.y, a2.y));
+    const float2 dS = __fadd2_rn(dz, __ffma2_rn(h1, k.m1, h2));
+    const float2 num = __ffma2_rn(__fmul2_rn(k.ngdt_dx, hf), dS, q);
+    const float2 nl = __fmul2_rn(k.sh, nsum);
+    const float2 c = __fmul2_rn(__fmul2_rn(k.gdt, __fmul2_rn(nl, nl)), q);
+    const float2 e = __fmul2_rn(k.p73, make_float2(lg2_approx(hf.x), lg2_approx(hf.y)));
+    const float2 fr = __fmul2_rn(
+        c, make_float2(fminf(ex2_approx(e.x), 1.0e30f), fminf(ex2_approx(e.y), 1.0e30f)));
+    float2 qn = __fmul2_rn(num, make_float2(rcp_approx(__fadd_rn(1.0f, fabsf(fr.x))),
+                                            rcp_approx(__fadd_rn(1.0f, fabsf(fr.y)))));
+    if (LIM)
+        qn = make_float2(fmaxf(fminf(qn.x, up.x), -dn.x), fmaxf(fminf(qn.y, up.y), -dn.y));
+    return make_float2(hf.x > k.h_eps ? qn.x : 0.0f, hf.y > k.h_eps ? qn.y : 0.0f);
+}
+
+// min of three, max of three that keeps a NaN operand (one instruction each)
+__device__ __forceinline__ float fmin3(float a, float b, float c)
+{
+    float y;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+    return y;
+}
+__device__ __forceinline__ float fmax3_nan(float a, float b, float c)
+{
+    float y;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+    return y;
+}
+
 // Free-outflow edge link: a ghost cell continuing the bed at the edge slope
 // with the edge cell's depth, so h_flow = h and dx * S = -edge_slope * dx;
 // only outward flow passes.

@@ -13,9 +13,9 @@ namespace flood {
 struct MarchOut {
     float hmax;
     bool bad;
-    float out_s, out_c;   // outflow sum of q over the warp's edge links (Kahan pair)
-    float clamp;          // sum of the negative depths reset to zero
-    float drn_s, drn_c;   // drained depth (land cover; Kahan pair)
+    double out;     // this lane's outflow sum of q over the warp's edge links
+    double clamp;   // sum of the negative depths reset to zero
+    double drn;     // drained depth (land cover)
 };
 
 __device__ __forceinline__ void m_load4(float (&v)[4], const float* p)
@@ -298,11 +298,9 @@ __device__ __forceinline__ MarchOut march_rows(const float* __restrict__ src, fl
     MarchOut out;
     out.hmax = hmax;
     out.bad = !(hmax <= 3.0e38f);  // a NaN or an overflow anywhere
-    out.out_s = out_s;
-    out.out_c = out_c;
-    out.clamp = clamp;
-    out.drn_s = drn_s;
-    out.drn_c = drn_c;
+    out.out = (double)out_s - (double)out_c;
+    out.clamp = (double)clamp;
+    out.drn = (double)drn_s - (double)drn_c;
     return out;
 }
 

@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(32 * WM * WC, (LC ? 4 : FLOOD_STEP_MIN_BLOCKS)
     // warp reductions: max depth (order-free); volume partials widened to
     // FP64 once per warp and reduced in a fixed order
     const unsigned hb = __reduce_max_sync(0xffffffffu, mo.bad ? 0u : __float_as_uint(mo.hmax) & 0x7fffffffu);
-    double out_acc = (double)mo.out_s - (double)mo.out_c, clamp_acc = (double)mo.clamp;
-    double drn_acc = LC ? (double)mo.drn_s - (double)mo.drn_c : 0.0;
+    double out_acc = mo.out, clamp_acc = mo.clamp;
+    double drn_acc = LC ? mo.drn : 0.0;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         out_acc += __shfl_xor_sync(0xffffffffu, out_acc, off);

@@ -12,12 +12,15 @@ namespace {
 
 constexpr int kSpan = kTmaSpan;
 
-// The land-cover form holds its class tables in registers: it gets more of
-// them (four CTAs of four warps per SM instead of five) rather than spill.
+// Warps per SM: what the rings leave room for (20 rings of four 2.8 KB
+// stages, 16 with the running maxima's 512 bytes more).
+__host__ __device__ constexpr int tma_warps_per_sm(bool track) { return track ? 16 : 20; }
+
 // CK: the step may write checkpoints (the adjoint's logged forward); the
 // ordinary step is compiled without that path.
 template <int WM, bool TRACK_MAX, bool LC, int LIM, bool CK, bool HOOK = false>
-__global__ void __launch_bounds__(32 * WM, (TRACK_MAX ? 16 : 20) / WM) step_tma_kernel(const __grid_constant__ TmaArgs t)
+__global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
+    step_tma_kernel(const __grid_constant__ TmaArgs t)
 {
     extern __shared__ unsigned char smem_raw[];
     const StepArgs& a = t.a;
@@ -34,9 +37,7 @@ __global__ void __launch_bounds__(32 * WM, (TRACK_MAX ? 16 : 20) / WM) step_tma_
     if (m >= a.M || c0 >= a.nx) return;  // whole warps; no block-wide barriers below
     if (*reinterpret_cast<volatile const int*>(a.err) & 2) return;  // an earlier wait gave up
 
-    uint32_t bar0;
-    unsigned char* my_stages;
-    tma_march_smem(smem_raw, WM, w, bar0, my_stages, tma_stage_bytes(TRACK_MAX, LC));
+    const TmaSmem sm = tma_march_smem(smem_raw, WM, w, TRACK_MAX);
 
     const size_t mstride = 3 * a.plane;
     // each warp is its own member here: the warp at the first span and strip owns its clock
@@ -62,16 +63,16 @@ __global__ void __launch_bounds__(32 * WM, (TRACK_MAX ? 16 : 20) / WM) step_tma_
     float* hm = TRACK_MAX ? a.hmax_field + (size_t)m * a.plane : nullptr;
     LandK lk;
     if (LC) lk = land_k(a, m, pl.dr, pl.dt, lane);
-    if (!tma_march<TRACK_MAX, LC, LIM, HOOK>(&t.state_map, &t.static_map, (pl.cur * a.M + m) * 3, bar0,
-                                  my_stages, dst, ck, hm, a.err, a.plane, a.ny, a.nx, a.ld, c0, r0,
+    if (!tma_march<TRACK_MAX, LC, LIM, HOOK>(&t.state_map, &t.static_map, (pl.cur * a.M + m) * 3, sm,
+                                  dst, ck, hm, a.err, a.plane, a.ny, a.nx, a.ld, c0, r0,
                                   r1, lane, k, pl.dt_dx, a.scale[m], pl.dr, a.east_out, a.south_out,
                                   mo, &lk, a.wait_budget, &t.hm_map, m))
         return;
 
     if (mo.bad) atomicOr(a.err, 1);
     const unsigned hb = __reduce_max_sync(0xffffffffu, mo.bad ? 0u : __float_as_uint(mo.hmax) & 0x7fffffffu);
-    double out_acc = (double)mo.out_s - (double)mo.out_c, clamp_acc = (double)mo.clamp;
-    double drn_acc = LC ? (double)mo.drn_s - (double)mo.drn_c : 0.0;
+    double out_acc = mo.out, clamp_acc = mo.clamp;
+    double drn_acc = LC ? mo.drn : 0.0;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         out_acc += __shfl_xor_sync(0xffffffffu, out_acc, off);
@@ -96,7 +97,7 @@ __global__ void __launch_bounds__(32 * WM, (TRACK_MAX ? 16 : 20) / WM) step_tma_
 // replay_i + 1, with the member's plan taken from the step log.  LC: with
 // land cover (the class bytes ride in the stage, as in the step).
 template <int WM, int LIM, bool LC = false>
-__global__ void __launch_bounds__(32 * WM, 20 / WM) replay_tma_kernel(const __grid_constant__ TmaArgs t)
+__global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(false) / WM) replay_tma_kernel(const __grid_constant__ TmaArgs t)
 {
     extern __shared__ unsigned char smem_raw[];
     const StepArgs& a = t.a;
@@ -109,9 +110,7 @@ __global__ void __launch_bounds__(32 * WM, 20 / WM) replay_tma_kernel(const __gr
     const int j = a.seg_first + a.replay_i;
     if (j >= a.seg_end[m]) return;
 
-    uint32_t bar0;
-    unsigned char* my_stages;
-    tma_march_smem(smem_raw, WM, w, bar0, my_stages, tma_stage_bytes(false, LC));
+    const TmaSmem sm = tma_march_smem(smem_raw, WM, w);
 
     const size_t mstride = 3 * a.plane;
     const MemberPlan pl = a.log[(size_t)m * a.dt_log_cap + j];
@@ -131,18 +130,12 @@ __global__ void __launch_bounds__(32 * WM, 20 / WM) replay_tma_kernel(const __gr
     MarchOut mo;
     LandK lk;
     if (LC) lk = land_k(a, m, pl.dr, pl.dt, lane);
-    if (!tma_march<false, LC, LIM>(&t.state_map, &t.static_map, (a.replay_i * a.M + m) * 3, bar0,
-                                   my_stages, dst, nullptr, nullptr, a.err, a.plane, a.ny, a.nx,
+    if (!tma_march<false, LC, LIM>(&t.state_map, &t.static_map, (a.replay_i * a.M + m) * 3, sm,
+                                   dst, nullptr, nullptr, a.err, a.plane, a.ny, a.nx,
                                    a.ld, c0, r0, r1, lane, k, pl.dt_dx, a.scale[m], pl.dr,
                                    a.east_out, a.south_out, mo, &lk, kTmaWaitBudget, nullptr, 0))
         return;
     if (mo.bad) atomicOr(a.err, 1);
-}
-
-template <int WM, bool TRACK = false, bool LC = false>
-size_t tma_smem_bytes()
-{
-    return tma_march_smem_bytes(WM, tma_stage_bytes(TRACK, LC));
 }
 
 }  // namespace
@@ -196,18 +189,22 @@ int tma_box_cols() { return kTmaBox; }
 
 namespace {
 
+int spans_of(const StepArgs& a) { return (a.nx + kSpan - 1) / kSpan; }
+int strips_of(const StepArgs& a) { return (a.ny + a.rows_per_strip - 1) / a.rows_per_strip; }
+
 template <int WM, bool TRACK_MAX, bool LC, int LIM, bool CK, bool HOOK>
-void launch_tma_wm(const TmaArgs& t, int spans, int strips, cudaStream_t s)
+void launch_tma_wm(const TmaArgs& t, cudaStream_t s)
 {
     static bool attr = false;
-    const size_t shm = tma_smem_bytes<WM, TRACK_MAX, LC>();
+    const size_t shm = tma_march_smem_bytes(WM, TRACK_MAX);
+    const auto f = step_tma_kernel<WM, TRACK_MAX, LC, LIM, CK, HOOK>;
     if (!attr) {
-        cudaFuncSetAttribute(step_tma_kernel<WM, TRACK_MAX, LC, LIM, CK, HOOK>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
         attr = true;
     }
-    dim3 grid((t.a.M + WM - 1) / WM, spans, strips), block(32, WM);
-    step_tma_kernel<WM, TRACK_MAX, LC, LIM, CK, HOOK><<<grid, block, shm, s>>>(t);
+    const StepArgs& a = t.a;
+    const dim3 grid((a.M + WM - 1) / WM, a.tiles ? a.n_tiles : spans_of(a), a.tiles ? 1 : strips_of(a));
+    f<<<grid, dim3(32, WM), shm, s>>>(t);
 }
 
 // Members per CTA: 4 or 1 for every variant; the plain step also has 2 and 8
@@ -215,41 +212,38 @@ void launch_tma_wm(const TmaArgs& t, int spans, int strips, cudaStream_t s)
 template <bool TRACK_MAX, bool LC, int LIM, bool CK, bool HOOK = false>
 void launch_tma(const TmaArgs& t, int members_per_cta, cudaStream_t s)
 {
-    const StepArgs& a = t.a;
-    const int spans = a.tiles ? a.n_tiles : (a.nx + kSpan - 1) / kSpan;
-    const int strips = a.tiles ? 1 : (a.ny + a.rows_per_strip - 1) / a.rows_per_strip;
     constexpr bool kPlain = !TRACK_MAX && !LC && !CK && !HOOK;
     if (kPlain && members_per_cta == 8)
-        launch_tma_wm<kPlain ? 8 : 4, TRACK_MAX, LC, LIM, CK, HOOK>(t, spans, strips, s);
+        launch_tma_wm<kPlain ? 8 : 4, TRACK_MAX, LC, LIM, CK, HOOK>(t, s);
     else if (members_per_cta >= 4)
-        launch_tma_wm<4, TRACK_MAX, LC, LIM, CK, HOOK>(t, spans, strips, s);
+        launch_tma_wm<4, TRACK_MAX, LC, LIM, CK, HOOK>(t, s);
     else if (kPlain && members_per_cta == 2)
-        launch_tma_wm<kPlain ? 2 : 1, TRACK_MAX, LC, LIM, CK, HOOK>(t, spans, strips, s);
+        launch_tma_wm<kPlain ? 2 : 1, TRACK_MAX, LC, LIM, CK, HOOK>(t, s);
     else
-        launch_tma_wm<1, TRACK_MAX, LC, LIM, CK, HOOK>(t, spans, strips, s);
+        launch_tma_wm<1, TRACK_MAX, LC, LIM, CK, HOOK>(t, s);
+}
+
+template <int WM, int LIM, bool LC>
+void launch_replay_wm(const TmaArgs& t, cudaStream_t s)
+{
+    static bool attr = false;
+    const size_t shm = tma_march_smem_bytes(WM);
+    const auto f = replay_tma_kernel<WM, LIM, LC>;
+    if (!attr) {
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+        attr = true;
+    }
+    const StepArgs& a = t.a;
+    f<<<dim3((a.M + WM - 1) / WM, spans_of(a), strips_of(a)), dim3(32, WM), shm, s>>>(t);
 }
 
 template <int LIM, bool LC>
 void launch_replay_lim(const TmaArgs& t, int members_per_cta, cudaStream_t s)
 {
-    const StepArgs& a = t.a;
-    const int spans = (a.nx + kSpan - 1) / kSpan;
-    const int strips = (a.ny + a.rows_per_strip - 1) / a.rows_per_strip;
-    if (members_per_cta >= 4) {
-        static bool attr = false;
-        const size_t shm = tma_smem_bytes<4, false, LC>();
-        if (!attr) {
-            cudaFuncSetAttribute(replay_tma_kernel<4, LIM, LC>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-            attr = true;
-        }
-        dim3 grid((a.M + 3) / 4, spans, strips), block(32, 4);
-        replay_tma_kernel<4, LIM, LC><<<grid, block, shm, s>>>(t);
-    } else {
-        const size_t shm = tma_smem_bytes<1, false, LC>();
-        dim3 grid(a.M, spans, strips), block(32, 1);
-        replay_tma_kernel<1, LIM, LC><<<grid, block, shm, s>>>(t);
-    }
+    if (members_per_cta >= 4)
+        launch_replay_wm<4, LIM, LC>(t, s);
+    else
+        launch_replay_wm<1, LIM, LC>(t, s);
 }
 
 }  // namespace

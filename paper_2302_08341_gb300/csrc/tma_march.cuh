@@ -5,12 +5,27 @@
 // The warp's rows arrive through a ring of kTmaNS shared-memory stages filled
 // by the tensor memory accelerator: one 3-D tiled copy brings a row of h, qx
 // and qy (136 columns: the span plus 4 halo columns each side, zero-filled
-// past the grid's edges), another the same row of z and n.  Lane 0 keeps
-// kTmaNS - 1 rows in flight ahead of the row being computed, so the memory
+// past the grid's edges), another the same row of z and n.  Lane 0 keeps the
+// ring's rows in flight ahead of the row being computed, so the memory
 // latency is covered by the warp's own pipeline; the halo comes with the
 // tile, so no scalar edge loads remain.  Every mbarrier wait is bounded: on
 // timeout the march records FLOOD_ERR_TIMEOUT in the error word, waits
 // (bounded) for its own copies in flight, and returns false.
+//
+// What bounds it: the issue slots, before memory.  A row of 128 cells took 545
+// warp instructions, of which the arithmetic of its 256 links and 128 depths
+// is about 290; the rest was bookkeeping, edge tests and the link west of the
+// span, which lane 0 computed in a branch of its own.  So links are computed
+// in pairs with the two-wide FP32 instructions (link2_q); the link west of
+// the span is computed by every lane from one broadcast address, in line with
+// the others; cells past the grid's edge are masked in a branch that only the
+// spans holding the edge take (the edge spans ran both forms of every link);
+// the row's four depths share one test for negative values; a row's depth,
+// bed and roughness are read again from its stage rather than carried over,
+// so the row loop needs no unrolling to stay free of moves.  2000 x 2000
+// cells x 96 members: 1.63 -> 1.42 ms per step; 1000 x 1000 x 16: 105 -> 83 us.
+// Two spans a warp (one wait and one link west for 256 cells, 12 warps per SM
+// instead of 20) measured the same or slower at every size but one.
 #pragma once
 
 #include "march.cuh"
@@ -25,60 +40,82 @@ constexpr int kTmaStaticOff = 1664;                // bytes: z, n after h, qx, q
 constexpr int kTmaStageBytes = 2816;               // 128-aligned stage size
 constexpr uint32_t kTmaTx = kTmaBox * 3 * 4 + kTmaBox * 2 * 4;  // bytes landing per stage
 constexpr long long kTmaWaitBudget = kTmaWaitBudgetDefault;  // clock cycles before giving up
+constexpr int kTmaHmOff = kTmaStageBytes;          // running maxima: 128 floats after z, n
 static_assert((kTmaNS & (kTmaNS - 1)) == 0, "ring index arithmetic needs a power of two");
 
-// Dynamic shared memory of a CTA of `warps` warps: barriers, then each warp's
-// stages.
-__host__ __device__ constexpr size_t tma_march_smem_bytes(int warps, int stage_bytes = kTmaStageBytes)
+// With land cover the static planes are the bed and each cell's class code (a
+// uint32 where the roughness would be): the stage keeps its size.
+__host__ __device__ constexpr int tma_stage_bytes(bool track) { return kTmaStageBytes + (track ? 512 : 0); }
+
+// Dynamic shared memory of a CTA of `warps` warps: barriers and the land-cover
+// class tables (64 bytes a warp), then each warp's stages.
+__host__ __device__ constexpr int tma_head_bytes(int warps)
 {
-    return 128 + 128 * ((8 * kTmaNS * warps + 127) / 128) + (size_t)kTmaNS * stage_bytes * warps;
+    return 128 * ((8 * kTmaNS * warps + 127) / 128) + 128 * ((64 * warps + 127) / 128);
 }
-constexpr int kTmaHmOff = kTmaStageBytes;              // running maxima: 128 floats after z, n
-// With land cover the static planes are the bed and each cell's class code
-// (a uint32 where the roughness would be): the stage keeps its size.
-__host__ __device__ constexpr int tma_stage_bytes(bool track, bool lc)
+__host__ __device__ constexpr size_t tma_march_smem_bytes(int warps, bool track = false)
 {
-    return kTmaStageBytes + (track ? 512 : 0) + (lc ? 0 : 0);
+    return 128 + tma_head_bytes(warps) + (size_t)kTmaNS * tma_stage_bytes(track) * warps;
 }
 
-// This warp's barriers and stages inside the CTA's dynamic shared memory.
-__device__ __forceinline__ void tma_march_smem(unsigned char* smem_raw, int warps, int w,
-                                               uint32_t& bar0, unsigned char*& my_stages,
-                                               int stage_bytes = kTmaStageBytes)
+// This warp's share of the CTA's dynamic shared memory.
+struct TmaSmem {
+    uint32_t bar0;            // barriers, 8 bytes each
+    float4* tab;              // [4] class table: rain depth, drainage depth, Manning n
+    unsigned char* stages;
+};
+
+__device__ __forceinline__ TmaSmem tma_march_smem(unsigned char* smem_raw, int warps, int w,
+                                                  bool track = false)
 {
     unsigned char* base = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
-    bar0 = smem_u32(base) + 8u * kTmaNS * w;
-    my_stages = base + 128 * ((8 * kTmaNS * warps + 127) / 128) + kTmaNS * stage_bytes * w;
+    TmaSmem m;
+    m.bar0 = smem_u32(base) + 8u * kTmaNS * w;
+    m.tab = reinterpret_cast<float4*>(base + 128 * ((8 * kTmaNS * warps + 127) / 128)) + 4 * w;
+    m.stages = base + tma_head_bytes(warps) + kTmaNS * tma_stage_bytes(track) * w;
+    return m;
 }
 
-__device__ __forceinline__ void tma_lds4(float (&v)[4], const float* p)
+// Four cells as two pairs.
+struct Quad {
+    float2 a, b;
+};
+__device__ __forceinline__ Quad lds_quad(const float* p)
 {
     const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    return Quad{make_float2(t.x, t.y), make_float2(t.z, t.w)};
 }
-
-__device__ __forceinline__ void tma_store4(float* p, const float (&v)[4])
+__device__ __forceinline__ void st_quad(float* p, const Quad& v)
 {
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(p) = make_float4(v.a.x, v.a.y, v.b.x, v.b.y);
+}
+__device__ __forceinline__ float& quad_at(Quad& v, int j)
+{
+    return j == 0 ? v.a.x : j == 1 ? v.a.y : j == 2 ? v.b.x : v.b.y;
+}
+__device__ __forceinline__ const float& quad_at(const Quad& v, int j)
+{
+    return j == 0 ? v.a.x : j == 1 ? v.a.y : j == 2 ? v.b.x : v.b.y;
 }
 
 // state_map: (ld, ny, planes) with the source h, qx, qy at planes
 // [plane0, plane0 + 3); static_map: (ld, ny, 2) with z then n.  Writes the
 // new state to dst (and ck when non-null); TRACK_MAX: also raises the
 // running maximum depth at hm, whose old values arrive with each row through
-// hm_map (member plane hm_plane, 128 columns from c0; a 3.3 KB stage, so four
-// CTAs of four warps per SM); LC: land cover (roughness by class from lk,
-// the class's share of the rain and its drainage; static_map then holds the
-// bed and each cell's class code, so the codes arrive with the row where
-// the roughness would, halo included).  Each is a separate
-// instantiation, so the plain step carries no trace of them.  Returns false
-// if a wait gave up.  WAIT_HOOK: each row wait may take wait_budget clock
-// cycles instead of kTmaWaitBudget (a failure-detection hook; the copies
-// still in flight are always drained with the full kTmaWaitBudget).
-template <bool TRACK_MAX, bool LC = false, int LIM = -1, bool WAIT_HOOK = false>
+// hm_map (member plane hm_plane, 128 columns from c0); LC: land cover
+// (roughness by class from lk, the class's share of the rain and its
+// drainage; static_map then holds the bed and each cell's class code, so the
+// codes arrive with the row where the roughness would, halo included; the
+// class table sits in shared memory, one word of it per lookup).  Each is a
+// separate instantiation, so the plain step carries no trace of them.
+// Returns false if a wait gave up.  WAIT_HOOK: each row wait may take
+// wait_budget clock cycles instead of kTmaWaitBudget (a failure-detection
+// hook; the copies still in flight are always drained with the full
+// kTmaWaitBudget).
+template <bool TRACK_MAX, bool LC, int LIM, bool WAIT_HOOK = false>
 __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CUtensorMap* static_map,
-                                          int plane0, uint32_t bar0, unsigned char* my_stages,
+                                          int plane0, const TmaSmem& sm,
                                           float* __restrict__ dst, float* ck, float* hm, int* err,
                                           size_t plane,
                                           int ny, int nx, int ld, int c0, int r0, int r1, int lane,
@@ -89,239 +126,263 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
                                           const CUtensorMap* hm_map = nullptr, int hm_plane = 0)
 {
     constexpr int kNS = kTmaNS;
-    constexpr int kBox = kTmaBox;
-    constexpr int kStaticOff = kTmaStaticOff;
-    constexpr int kStageBytes = tma_stage_bytes(TRACK_MAX, LC);
+    constexpr int kStage = tma_stage_bytes(TRACK_MAX);
     constexpr uint32_t kTx = kTmaTx + (TRACK_MAX ? 512u : 0u);
-    constexpr int kZ = kStaticOff / 4;
-    constexpr int kN = kZ + kBox;
-    constexpr long long kWaitBudget = kTmaWaitBudget;
-    const uint32_t stage0 = smem_u32(my_stages);
+    constexpr int kZ = kTmaStaticOff / 4;
+    constexpr int kN = kZ + kTmaBox;
+    constexpr int kQx = kTmaBox, kQy = 2 * kTmaBox;
+    const uint32_t stage0 = smem_u32(sm.stages);
     const float s_half = 0.5f * s;
+    const Link2K lk2 = link2_k(k, s_half);
+    const float2 lim2 = dup2(k.dx_4dt), dtdx2 = dup2(dt_dx), dr2 = dup2(dr);
 
     const int c = c0 + 4 * lane;
-    const bool act = c < nx;
-    const bool interior = (c + 4 < nx);
-    const bool edge_warp = c0 + kTmaSpan >= nx;  // the span holds the grid's last column
+    const bool full = c0 + kTmaSpan < nx;  // every cell and its east neighbour inside
     const int ra = r0 > 0 ? r0 - 1 : r0;   // first row loaded
     const int rb = min(r1 + 1, ny);        // one past the last row loaded
 
+    if (LC && lane < 4) sm.tab[lane] = make_float4(lk->dr, lk->dd, lk->n, 0.0f);
     if (lane == 0) {
-        for (int i = 0; i < kNS; ++i) mbar_init(bar0 + 8u * i, 1);
+        for (int i = 0; i < kNS; ++i) mbar_init(sm.bar0 + 8u * i, 1);
         fence_mbar_init();
     }
     __syncwarp();
-    int issued = ra;  // rows [ra, issued) have been requested
-    auto issue = [&](int row) {
-        const unsigned sidx = (unsigned)(row - ra) & (kNS - 1);
-        const uint32_t bar = bar0 + 8u * sidx;
-        const uint32_t dsts = stage0 + kStageBytes * sidx;
+    auto issue = [&](int row, int slot) {
+        const uint32_t bar = sm.bar0 + 8u * slot;
         mbar_arrive_expect_tx(bar, kTx);
-        tma_load_3d(dsts, state_map, c0 - 4, row, plane0, bar);
-        tma_load_3d(dsts + kStaticOff, static_map, c0 - 4, row, 0, bar);
-        if (TRACK_MAX) tma_load_3d(dsts + kTmaHmOff, hm_map, c0, row, hm_plane, bar);
+        const uint32_t d = stage0 + kStage * slot;
+        tma_load_3d(d, state_map, c0 - 4, row, plane0, bar);
+        tma_load_3d(d + kTmaStaticOff, static_map, c0 - 4, row, 0, bar);
+        if (TRACK_MAX) tma_load_3d(d + kTmaHmOff, hm_map, c0, row, hm_plane, bar);
     };
-    // land classes of a staged row (LC: the class-code plane): the lane's
-    // four cells as one byte each of a word
-    auto cls_of = [&](const float* P) -> uint32_t {
-        const uint4 q = *reinterpret_cast<const uint4*>(P + kN + 4 + 4 * lane);
-        return __byte_perm(__byte_perm(q.x, q.y, 0x0040u), __byte_perm(q.z, q.w, 0x0040u), 0x5410u);
+    if (lane == 0)
+        for (int i = 0; i < kNS && ra + i < rb; ++i) issue(ra + i, i);
+    auto wait_slot = [&](int slot, uint32_t parity, long long budget) -> bool {
+        return mbar_wait_bounded(sm.bar0 + 8u * slot, parity, budget);
     };
-    for (; issued < rb && issued < ra + kNS; ++issued)
-        if (lane == 0) issue(issued);
-    auto wait_row_for = [&](int row, long long budget) -> bool {
-        const int kk = row - ra;
-        return mbar_wait_bounded(bar0 + 8u * ((unsigned)kk & (kNS - 1)), ((unsigned)kk / kNS) & 1,
-                                 budget);
-    };
-    auto wait_row = [&](int row) -> bool {
-        return wait_row_for(row, WAIT_HOOK ? wait_budget : kWaitBudget);
-    };
-    auto row_ptr = [&](int row) -> const float* {
-        return reinterpret_cast<const float*>(my_stages +
-                                              kStageBytes * ((unsigned)(row - ra) & (kNS - 1)));
-    };
-    // recycle the stage of `row` for the next row in line
-    auto release = [&](int row) {
+    const long long budget = WAIT_HOOK ? wait_budget : kTmaWaitBudget;
+    // a row's stage takes the row kNS further on, once the whole warp has read it
+    auto release = [&](int row, int slot) {
         __syncwarp();
-        if (issued < rb) {
-            if (lane == 0) {
-                fence_proxy_async_smem();
-                issue(issued);
-            }
-            ++issued;
+        if (row + kNS < rb && lane == 0) {
+            fence_proxy_async_smem();
+            issue(row + kNS, slot);
         }
-        (void)row;
     };
-    int waited = ra;  // rows [ra, waited) have landed
-    bool ok = true;
-    auto drain_and_fail = [&]() {
+    // rows [from, to) are still in flight: every copy lands before the warp
+    // leaves (bounded each)
+    auto drain_and_fail = [&](int from, int to) {
         if (lane == 0) atomicOr(err, 2);
-        // every copy still in flight lands before the warp leaves (bounded each)
-        for (int row = waited; row < issued; ++row) wait_row_for(row, kWaitBudget);
+        for (int row = from; row < to; ++row)
+            wait_slot((row - ra) % kNS, ((row - ra) / kNS) & 1, kTmaWaitBudget);
+    };
+    auto row_ptr = [&](int slot) -> const float* {
+        return reinterpret_cast<const float*>(sm.stages + kStage * slot);
+    };
+    // Manning n of the class of a staged cell (LC)
+    auto class_n = [&](const float* code) -> float {
+        return reinterpret_cast<const float*>(sm.tab + *reinterpret_cast<const uint32_t*>(code))[2];
+    };
+    auto quad_n = [&](const float* p) -> Quad {  // roughness of four staged cells
+        if (!LC) return lds_quad(p);
+        const uint4 q = *reinterpret_cast<const uint4*>(p);
+        const float* t = reinterpret_cast<const float*>(sm.tab) + 2;
+        return Quad{make_float2(t[4 * q.x], t[4 * q.y]), make_float2(t[4 * q.z], t[4 * q.w])};
+    };
+    // links of four cells with the four south of them (or the row above with this one)
+    auto south_links = [&](const Quad& h1, const Quad& z1, const Quad& n1, const Quad& u1, const Quad& h2,
+                           const Quad& z2, const Quad& n2, const Quad& u2, const Quad& q) -> Quad {
+        return Quad{link2_q<LIM>(h1.a, z1.a, h2.a, z2.a, q.a, __fadd2_rn(n1.a, n2.a), u1.a, u2.a, lk2),
+                    link2_q<LIM>(h1.b, z1.b, h2.b, z2.b, q.b, __fadd2_rn(n1.b, n2.b), u1.b, u2.b, lk2)};
+    };
+    auto bounds = [&](const Quad& h) -> Quad {  // the limiter's bounds of four cells
+        return Quad{__fmul2_rn(h.a, lim2), __fmul2_rn(h.b, lim2)};
     };
 
     const int x0 = 4 + 4 * lane;  // this lane's first cell in a tile row
-    float hC[4] = {0, 0, 0, 0}, zC[4] = {0, 0, 0, 0}, nC[4] = {0, 0, 0, 0};
-    float qyN[4] = {0, 0, 0, 0};
+    int sC = 0;                   // slot of row r, of row r + 1 and that row's phase
     if (r0 > 0) {
-        ok = wait_row(r0 - 1);
-        if (ok) waited = r0;
+        if (!wait_slot(0, 0, budget)) {
+            drain_and_fail(ra, min(rb, ra + kNS));
+            return false;
+        }
+        sC = 1;
     }
-    if (ok) {
-        ok = wait_row(r0);
-        if (ok) waited = r0 + 1;
-    }
-    if (!ok) {
-        drain_and_fail();
+    if (!wait_slot(sC, 0, budget)) {
+        drain_and_fail(r0, min(rb, ra + kNS));
         return false;
     }
-    // land classes (LC): they come with each staged row (zeros past the
-    // grid's edges, where no link uses them)
-    uint32_t clsC = 0;
-    {
-        const float* P = row_ptr(r0);
-        if (LC) clsC = cls_of(P);
-        tma_lds4(hC, P + x0);
-        tma_lds4(zC, P + kZ + x0);
-        if (LC)
-            land_n4(nC, clsC, *lk);
-        else
-            tma_lds4(nC, P + kN + x0);
-        if (r0 > 0) {
-            const float* U = row_ptr(r0 - 1);
-            float hU[4], zU[4], nU[4], qU[4];
-            tma_lds4(hU, U + x0);
-            tma_lds4(zU, U + kZ + x0);
-            if (LC)  // whole warp: the lookups are shuffles
-                land_n4(nU, cls_of(U), *lk);
-            else
-                tma_lds4(nU, U + kN + x0);
-            tma_lds4(qU, U + 2 * kBox + x0);
+    const float* F = row_ptr(sC) + x0;
+    Quad nC = quad_n(F + kN);
+    Quad qN{dup2(0.0f), dup2(0.0f)};
+    if (r0 > 0) {
+        const float* U = row_ptr(0) + x0;
+        const Quad hU = lds_quad(U), hF = lds_quad(F);
+        qN = south_links(hU, lds_quad(U + kZ), quad_n(U + kN), bounds(hU), hF, lds_quad(F + kZ), nC,
+                         bounds(hF), lds_quad(U + kQy));
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                qyN[j] = (c + j < nx)
-                             ? link_q<LIM>(hU[j], zU[j], hC[j], zC[j], qU[j],
-                                      __fmul_rn(s_half, __fadd_rn(nU[j], nC[j])), k)
-                             : 0.0f;
-            release(r0 - 1);
-        }
+        for (int j = 0; j < 4; ++j)
+            if (!full && c + j >= nx) quad_at(qN, j) = 0.0f;
+        release(ra, 0);
     }
 
     float hmax = 0.0f;
     float out_s = 0.0f, out_c = 0.0f, clamp = 0.0f, drn_s = 0.0f, drn_c = 0.0f;
+    int sN = sC + 1;
+    uint32_t phN = 0;
+    float* pd = dst + (size_t)r0 * ld + c;
+    float* pc = ck ? ck + (size_t)r0 * ld + c : nullptr;
+    float* ph = TRACK_MAX ? hm + (size_t)r0 * ld + c : nullptr;
 
-#pragma unroll 2
+#pragma unroll 1
     for (int r = r0; r < r1; ++r) {
-        const size_t o = (size_t)r * ld + c;
         const bool has_s = (r + 1 < ny);
+        if (has_s && !wait_slot(sN, phN, budget)) {
+            drain_and_fail(r + 1, min(rb, r + kNS));
+            return false;
+        }
+        const float* R = row_ptr(sC);
+        const float* P = R + x0;
+        const Quad hC = lds_quad(P), zC = lds_quad(P + kZ), uC = bounds(hC);
+        if (!LC) nC = lds_quad(P + kN);
+        // east links: cells 0 1 2 3 with 1 2 3 and the next lane's first,
+        // straight from the tile
+        const Quad qx = lds_quad(P + kQx);
+        const float hE = P[4], zE = P[kZ + 4], nE = LC ? class_n(P + kN + 4) : P[kN + 4];
+        Quad qE, qS, nS;
+        qE.a = link2_q<LIM>(hC.a, zC.a, make_float2(hC.a.y, hC.b.x), make_float2(zC.a.y, zC.b.x), qx.a,
+                            make_float2(__fadd_rn(nC.a.x, nC.a.y), __fadd_rn(nC.a.y, nC.b.x)), uC.a,
+                            make_float2(uC.a.y, uC.b.x), lk2);
+        qE.b = link2_q<LIM>(hC.b, zC.b, make_float2(hC.b.y, hE), make_float2(zC.b.y, zE), qx.b,
+                            make_float2(__fadd_rn(nC.b.x, nC.b.y), __fadd_rn(nC.b.y, nE)), uC.b,
+                            make_float2(uC.b.y, __fmul_rn(hE, k.dx_4dt)), lk2);
+        // the link west of the span, from the tile's halo: every lane computes
+        // it from lane 0's addresses, lane 0 keeps it
+        float qH = (r >= k.in_r0 && r < k.in_r1) ? k.q_in : 0.0f;  // west edge: wall or inflow
+        if (c0 > 0)
+            qH = link_q<LIM>(R[3], R[kZ + 3], hC.a.x, zC.a.x, R[kQx + 3],
+                             __fmul_rn(s_half, __fadd_rn(LC ? class_n(R + kN + 3) : R[kN + 3], nC.a.x)), k);
         if (has_s) {
-            if (!wait_row(r + 1)) {
-                drain_and_fail();
-                return false;
-            }
-            waited = r + 2;
-        }
-        const float* P = row_ptr(r);
-        float hS[4] = {0, 0, 0, 0}, zS[4] = {0, 0, 0, 0}, nS[4] = {0, 0, 0, 0};
-        float qxo[4], qyo[4];
-        float4 hmo = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (TRACK_MAX) hmo = *reinterpret_cast<const float4*>(P + kTmaHmOff / 4 + 4 * lane);
-        tma_lds4(qxo, P + kBox + x0);
-        tma_lds4(qyo, P + 2 * kBox + x0);
-        uint32_t clsS = 0;
-        if (LC) {
-            // the whole warp, outside any branch (the lookups are shuffles);
-            // past the grid's last row the stage holds an earlier row, whose
-            // classes go unused
-            clsS = cls_of(row_ptr(r + 1));
-            land_n4(nS, clsS, *lk);
-        }
-        if (has_s) {
-            const float* Q = row_ptr(r + 1);
-            tma_lds4(hS, Q + x0);
-            tma_lds4(zS, Q + kZ + x0);
-            if (!LC) tma_lds4(nS, Q + kN + x0);
-        }
-        // east neighbour of the lane's last cell, straight from the tile
-        const float hE = P[x0 + 4], zE = P[kZ + x0 + 4];
-        float nE;
-        float nWl = 0.0f, drv[4], ddv[4];
-        if (LC) {
-            // the east neighbour's and the west halo cell's classes come
-            // with the tile (the codes sit where the roughness would)
-            nE = land_get(lk->n, __float_as_uint(P[kN + x0 + 4]));
-            nWl = land_get(lk->n, __float_as_uint(P[kN + 3]));
-            land_src4(drv, ddv, clsC, *lk);
+            const float* Q = row_ptr(sN) + x0;
+            const Quad hS = lds_quad(Q);
+            nS = quad_n(Q + kN);
+            qS = south_links(hC, zC, nC, uC, hS, lds_quad(Q + kZ), nS, bounds(hS), lds_quad(P + kQy));
         } else {
-            nE = P[kN + x0 + 4];
+            nS = nC;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                quad_at(qS, j) =
+                    south_out ? outflow_q<LIM>(quad_at(hC, j), P[kQy + j], __fmul_rn(s, quad_at(nC, j)), k)
+                              : 0.0f;
         }
-        float qxE[4], qyS[4];
-        if (interior)
-            row_links<true, LIM>(hC, zC, nC, hS, zS, nS, qxo, qyo, hE, zE, nE, has_s, c, nx, s, s_half, k,
-                            east_out, south_out, qxE, qyS);
-        else
-            row_links<false, LIM>(hC, zC, nC, hS, zS, nS, qxo, qyo, hE, zE, nE, has_s, c, nx, s, s_half, k,
-                             east_out, south_out, qxE, qyS);
-        float qW0 = __shfl_up_sync(0xffffffffu, qxE[3], 1);
-        if (lane == 0) {
-            qW0 = (r >= k.in_r0 && r < k.in_r1) ? k.q_in : 0.0f;  // west edge: wall or inflow
-            if (c0 > 0) {  // the neighbouring span's last link, from the tile's halo
-                const float nW = LC ? nWl : P[kN + 3];
-                qW0 = link_q<LIM>(P[3], P[kZ + 3], hC[0], zC[0], P[kBox + 3],
-                             __fmul_rn(s_half, __fadd_rn(nW, nC[0])), k);
+        if (!full) {  // the span holds the grid's last column: its east link, and nothing past it
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int cj = c + j;
+                if (cj >= nx - 1) {
+                    quad_at(qE, j) =
+                        (east_out && cj == nx - 1)
+                            ? outflow_q<LIM>(quad_at(hC, j), P[kQx + j], __fmul_rn(s, quad_at(nC, j)), k)
+                            : 0.0f;
+                    if (cj >= nx) quad_at(qS, j) = 0.0f;
+                }
             }
         }
-        float hN[4];
-        if (interior)
-            row_depths<true, LC>(hC, qxE, qyN, qyS, qW0, c, nx, dt_dx, dr, clamp, hmax, hN,
-                                 drv, ddv, &drn_s, &drn_c);
-        else
-            row_depths<false, LC>(hC, qxE, qyN, qyS, qW0, c, nx, dt_dx, dr, clamp, hmax, hN,
-                                  drv, ddv, &drn_s, &drn_c);
-        if ((edge_warp && east_out) || (!has_s && south_out)) {  // the same for the whole warp
+        // west links: the east links of the cells before, the first from the lane before
+        float qW0 = __shfl_up_sync(0xffffffffu, qE.b.y, 1);
+        if (lane == 0) qW0 = qH;
+        const float2 wa = make_float2(__fsub_rn(qW0, qE.a.x), __fsub_rn(qE.a.x, qE.a.y));
+        const float2 wb = make_float2(__fsub_rn(qE.a.y, qE.b.x), __fsub_rn(qE.b.x, qE.b.y));
+        const float2 na = __fadd2_rn(wa, __ffma2_rn(qS.a, lk2.m1, qN.a));
+        const float2 nb = __fadd2_rn(wb, __ffma2_rn(qS.b, lk2.m1, qN.b));
+        // the step's increment (fluxes and rain) is formed first and added
+        // to the depth once: adding the same rain depth to every cell on its
+        // own rounds every cell of a binade the same way, a bias that builds
+        // up in the stored volume
+        Quad hN;
+        if (!LC) {
+            hN.a = __fadd2_rn(hC.a, __ffma2_rn(dtdx2, na, dr2));
+            hN.b = __fadd2_rn(hC.b, __ffma2_rn(dtdx2, nb, dr2));
+            if (!full) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (c + j >= nx) quad_at(hN, j) = 0.0f;
+            }
+        } else {
+            const uint4 q = *reinterpret_cast<const uint4*>(P + kN);
+            const uint32_t code[4] = {q.x, q.y, q.z, q.w};
+            const float net[4] = {na.x, na.y, nb.x, nb.y};
+            float row_sink = 0.0f;  // the row's drained depth, compensated once per row
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 sd = *reinterpret_cast<const float2*>(sm.tab + code[j]);
+                const bool in = full || c + j < nx;
+                const float hp = in ? __fadd_rn(quad_at(hC, j), __fmaf_rn(dt_dx, net[j], sd.x)) : 0.0f;
+                const float sink = fminf(sd.y, fmaxf(hp, 0.0f));
+                // drainage that took all the water present leaves a depth
+                // that does not depend on the one before: marked like a
+                // clamped cell
+                quad_at(hN, j) = (hp > 0.0f && sink == hp) ? -0.0f : __fsub_rn(hp, sink);
+                row_sink = __fadd_rn(row_sink, sink);
+            }
+            kahan_add(drn_s, drn_c, row_sink);
+        }
+        // wet/dry clamp: a negative depth is rare (the limiter leaves only
+        // rounding), so the four cells share one test.  Clamped cells keep a
+        // negative zero: the adjoint reads the sign bit to know the branch
+        if (fminf(fmin3(hN.a.x, hN.a.y, hN.b.x), hN.b.y) < 0.0f) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (quad_at(hN, j) < 0.0f) {
+                    clamp = __fsub_rn(clamp, quad_at(hN, j));
+                    quad_at(hN, j) = -0.0f;
+                }
+        }
+        // a NaN anywhere stays in the maximum
+        hmax = fmax3_nan(fmax3_nan(hmax, hN.a.x, hN.a.y), hN.b.x, hN.b.y);
+        if ((!full && east_out) || (!has_s && south_out)) {  // the same for the whole warp
             // links leaving the domain this row: the east edge link (one lane)
             // and, on the last row, the south edge links
             float ev = 0.0f;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (c + j == nx - 1 && east_out) ev = qxE[j];
+                if (c + j == nx - 1 && east_out) ev = quad_at(qE, j);
             if (!has_s && south_out)
-                ev = __fadd_rn(ev, __fadd_rn(__fadd_rn(qyS[0], qyS[1]), __fadd_rn(qyS[2], qyS[3])));
+                ev = __fadd_rn(ev, __fadd_rn(__fadd_rn(qS.a.x, qS.a.y), __fadd_rn(qS.b.x, qS.b.y)));
             kahan_add(out_s, out_c, ev);
         }
-        if (act) {
-            tma_store4(dst + o, hN);
-            tma_store4(dst + plane + o, qxE);
-            tma_store4(dst + 2 * plane + o, qyS);
+        if (full || c < nx) {
+            st_quad(pd, hN);
+            st_quad(pd + plane, qE);
+            st_quad(pd + 2 * plane, qS);
             if (ck) {
-                tma_store4(ck + o, hN);
-                tma_store4(ck + plane + o, qxE);
-                tma_store4(ck + 2 * plane + o, qyS);
+                st_quad(pc, hN);
+                st_quad(pc + plane, qE);
+                st_quad(pc + 2 * plane, qS);
             }
-            if (TRACK_MAX)
-                *reinterpret_cast<float4*>(hm + o) =
-                    make_float4(fmaxf(hmo.x, hN[0]), fmaxf(hmo.y, hN[1]), fmaxf(hmo.z, hN[2]),
-                                fmaxf(hmo.w, hN[3]));
+            if (TRACK_MAX) {
+                const Quad o = lds_quad(R + kTmaHmOff / 4 + 4 * lane);
+                *reinterpret_cast<float4*>(ph) = make_float4(fmaxf(o.a.x, hN.a.x), fmaxf(o.a.y, hN.a.y),
+                                                             fmaxf(o.b.x, hN.b.x), fmaxf(o.b.y, hN.b.y));
+            }
         }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            qyN[j] = qyS[j];
-            hC[j] = hS[j];
-            zC[j] = zS[j];
-            nC[j] = nS[j];
-        }
-        clsC = clsS;
-        release(r);
+        pd += ld;
+        if (ck) pc += ld;
+        if (TRACK_MAX) ph += ld;
+        // march: this row's south links are the next row's north links
+        qN = qS;
+        if (LC) nC = nS;
+        release(r, sC);
+        sC = sN;
+        sN = (sN + 1) & (kNS - 1);
+        if (sN == 0) phN ^= 1u;
     }
 
     out.hmax = hmax;
     out.bad = !(hmax <= 3.0e38f);  // a NaN or an overflow anywhere
-    out.out_s = out_s;
-    out.out_c = out_c;
-    out.clamp = clamp;
-    out.drn_s = drn_s;
-    out.drn_c = drn_c;
+    out.out = (double)out_s - (double)out_c;
+    out.clamp = (double)clamp;
+    out.drn = (double)drn_s - (double)drn_c;
     return true;
 }
 
