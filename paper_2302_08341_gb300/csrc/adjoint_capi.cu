@@ -31,6 +31,15 @@ int grow(flood_grid* g, T** p, size_t& have, size_t count)
     return flood::dalloc(g, p, count);
 }
 
+// The reverse stencil's automatic strip height (12 warps per SM).
+int reverse_rows(int ny, int nx, int M, int n_sm)
+{
+    const int spans = (nx + 127) / 128;
+    int rh = 64;
+    while (rh > 4 && (int64_t)M * spans * ((ny + rh - 1) / rh) < (int64_t)n_sm * 32) rh /= 2;
+    return rh;
+}
+
 // Put the state saved in ckpt slot 0 back into each member's current buffer
 // and restore the saved clocks and volume counters (a forward that overflowed
 // the step log is redone).
@@ -189,8 +198,10 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     }
     have = 0;
     if ((rc = grow(g, &g->lam, have, 2 * (size_t)M * ms))) return rc;
+    const int rrows = g->launch_fixed ? g->rows_per_strip : reverse_rows(g->ny, g->nx, M, g->n_sm);
+    const int nslot = flood::step_nslot(g->ny, g->nx, rrows);
     have = 0;
-    if ((rc = grow(g, &g->gpart, have, (size_t)M * g->nslot * 2))) return rc;
+    if ((rc = grow(g, &g->gpart, have, (size_t)M * nslot * 2))) return rc;
     have = 0;
     if ((rc = grow(g, &g->seg_end, have, M))) return rc;
     have = 0;
@@ -205,11 +216,11 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         CK(g, cudaMemsetAsync(g->gnm, 0, sizeof(float) * M * g->plane, s));
     }
     CK(g, cudaMemsetAsync(g->lam, 0, sizeof(float) * 2 * M * ms, s));
-    CK(g, cudaMemsetAsync(g->gpart, 0, sizeof(double) * M * g->nslot * 2, s));
+    CK(g, cudaMemsetAsync(g->gpart, 0, sizeof(double) * M * nslot * 2, s));
     if (g->lc_on) {
         have = 0;
-        if ((rc = grow(g, &g->gdpart, have, (size_t)M * g->nslot))) return rc;
-        CK(g, cudaMemsetAsync(g->gdpart, 0, sizeof(double) * M * g->nslot, s));
+        if ((rc = grow(g, &g->gdpart, have, (size_t)M * nslot))) return rc;
+        CK(g, cudaMemsetAsync(g->gdpart, 0, sizeof(double) * M * nslot, s));
     }
     CK(g, cudaMemcpyAsync(g->samp_step, samp_step.data(), sizeof(int32_t) * ns * M,
                           cudaMemcpyHostToDevice, s));
@@ -241,7 +252,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         tma.static_map = g->lc_on ? g->static_map_lc : g->static_map;
     }
     const bool tma_replay = use_tma;
-    const bool tma_reverse = use_tma && g->rows_per_strip >= 16;
+    const bool tma_reverse = use_tma && rrows >= 16;
 
     const int kmax = *std::max_element(K_m.begin(), K_m.end());
     const int n_seg = (kmax + K - 1) / K;
@@ -305,8 +316,8 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         b.seg_first = first;
         b.plane = g->plane;
         b.ny = g->ny; b.nx = g->nx; b.ld = g->ld; b.M = M;
-        b.rows_per_strip = g->rows_per_strip;
-        b.nslot = g->nslot;
+        b.rows_per_strip = rrows;
+        b.nslot = nslot;
         b.g = g->p.g;
         b.dxd = g->p.dx;
         b.h_eps = (float)g->p.h_eps;
@@ -353,14 +364,14 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         CK(g, cudaMemcpyAsync(grad_n, g->gn_out, sizeof(float) * g->ny * g->nx, cudaMemcpyDefault, s));
     }
     if (grad_rain || grad_scale) {
-        std::vector<double> gp((size_t)M * g->nslot * 2);
+        std::vector<double> gp((size_t)M * nslot * 2);
         CK(g, cudaMemcpyAsync(gp.data(), g->gpart, sizeof(double) * gp.size(), cudaMemcpyDeviceToHost, s));
         CK(g, cudaStreamSynchronize(s));
         for (int m = 0; m < M; ++m) {
             double gr = 0.0, gs = 0.0;
-            for (int k = 0; k < g->nslot; ++k) {
-                gr += gp[((size_t)m * g->nslot + k) * 2];
-                gs += gp[((size_t)m * g->nslot + k) * 2 + 1];
+            for (int k = 0; k < nslot; ++k) {
+                gr += gp[((size_t)m * nslot + k) * 2];
+                gs += gp[((size_t)m * nslot + k) * 2 + 1];
             }
             if (grad_rain) grad_rain[m] = gr;
             if (grad_scale) grad_scale[m] = gs;
@@ -368,11 +379,11 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     }
     g->adj_gdrain.assign(M, 0.0);
     if (g->lc_on) {
-        std::vector<double> gp((size_t)M * g->nslot);
+        std::vector<double> gp((size_t)M * nslot);
         CK(g, cudaMemcpyAsync(gp.data(), g->gdpart, sizeof(double) * gp.size(), cudaMemcpyDeviceToHost, s));
         CK(g, cudaStreamSynchronize(s));
         for (int m = 0; m < M; ++m)
-            for (int k = 0; k < g->nslot; ++k) g->adj_gdrain[m] += gp[(size_t)m * g->nslot + k];
+            for (int k = 0; k < nslot; ++k) g->adj_gdrain[m] += gp[(size_t)m * nslot + k];
     }
     // clocks keep counting from where they were
     std::vector<MemberClock> ce;
@@ -386,7 +397,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     g->adj_gn = grad_n != nullptr;
     g->adj_ns = ns;
     g->adj_G = G;
-    g->adj_nslot = g->nslot;
+    g->adj_nslot = nslot;
     return FLOOD_OK;
 }
 

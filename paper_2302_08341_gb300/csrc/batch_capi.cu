@@ -18,7 +18,10 @@ using flood::MemberClock;
 
 namespace {
 
-constexpr int kGraphSteps = 96;  // a multiple of 3: clock slots line up across replays
+// a multiple of 3: clock slots line up across replays.  Steps past a window's
+// end still launch (idle), so runs are short: 96 steps a run left 36 idle in a
+// 60 s window
+constexpr int kGraphSteps = 24;
 constexpr int kSpan = 128;
 
 thread_local std::string g_batch_msg;
@@ -56,6 +59,8 @@ struct flood_batch {
     double* t_stop = nullptr;         // device scalar
     flood::MemberPlan* plan = nullptr; // [S]
     int rows_per_strip = 64, warps_per_cta = 4;
+    bool launch_fixed = false;        // set by flood_batch_set_launch
+    int n_sm = 0;
     int engine = 0;                   // 0: direct loads, 1: TMA-staged rows, 2: persistent
     unsigned* pbar = nullptr;         // persistent form: barrier words [2], task counters [2]
     int* pact = nullptr;              // [2] some scenario steps, by step parity
@@ -114,6 +119,11 @@ void drop_graph(flood_batch* b)
 // definitive data, as in the ensemble kernel).
 int build_tasks(flood_batch* b)
 {
+    if (!b->launch_fixed) {  // as the ensemble's automatic strip height
+        int64_t rows = 0;
+        for (int e = 0; e < b->S; ++e) rows += (int64_t)b->ny[e] * ((b->nx[e] + kSpan - 1) / kSpan);
+        b->rows_per_strip = flood::strip_rows(rows, b->n_sm * 20);
+    }
     b->tasks.clear();
     b->slot0.assign(b->S, 0);
     std::vector<std::vector<int>> slots(b->S);
@@ -365,6 +375,10 @@ int flood_batch_create(flood_batch** out, int n, const int32_t* ny, const int32_
     flood_batch* b = new flood_batch();
     b->n_scen = n;
     b->p = *p;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&b->n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (b->n_sm <= 0) b->n_sm = 1;
     b->sny.assign(ny, ny + n);
     b->snx.assign(nx, nx + n);
     b->sld.resize(n);
@@ -566,6 +580,7 @@ int flood_batch_set_launch(flood_batch* b, int rows_per_strip, int warps_per_cta
     }
     b->rows_per_strip = rows_per_strip;
     b->warps_per_cta = warps_per_cta;
+    b->launch_fixed = true;
     int rc = build_tasks(b);
     if (rc) return rc;
     return put_entry_sums(b, per, dper);

@@ -287,6 +287,12 @@ struct Link2K {
 
 __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 
+// a - b (m1: -1, -1)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b, float2 m1)
+{
+    return __ffma2_rn(b, m1, a);
+}
+
 __device__ __forceinline__ Link2K link2_k(const FaceK& k, float s_half)
 {
     return Link2K{dup2(-1.0f), dup2(-k.gdt_dx), dup2(k.gdt), dup2(s_half), dup2(-2.33333333f), k.h_eps};
@@ -296,11 +302,12 @@ template <int LIM>
 __device__ __forceinline__ float2 link2_q(float2 h1, float2 z1, float2 h2, float2 z2, float2 q,
                                           float2 nsum, float2 up, float2 dn, const Link2K& k)
 {
-    const float2 dz = __ffma2_rn(z1, k.m1, z2);
-    const float2 a1 = __ffma2_rn(make_float2(fmaxf(dz.x, 0.0f), fmaxf(dz.y, 0.0f)), k.m1, h1);
+    const float2 dz = sub2(z2, z1, k.m1);
+    const float2 dh = sub2(h2, h1, k.m1);
     const float2 a2 = __fadd2_rn(h2, make_float2(fminf(dz.x, 0.0f), fminf(dz.y, 0.0f)));
+    const float2 a1 = sub2(h1, make_float2(fmaxf(dz.x, 0.0f), fmaxf(dz.y, 0.0f)), k.m1);
     const float2 hf = make_float2(fmaxf(a1.x, a2.x), fmaxf(a1.y, a2.y));
-    const float2 dS = __fadd2_rn(dz, __ffma2_rn(h1, k.m1, h2));
+    const float2 dS = __fadd2_rn(dz, dh);
     const float2 num = __ffma2_rn(__fmul2_rn(k.ngdt_dx, hf), dS, q);
     const float2 nl = __fmul2_rn(k.sh, nsum);
     const float2 c = __fmul2_rn(__fmul2_rn(k.gdt, __fmul2_rn(nl, nl)), q);
@@ -410,5 +417,8 @@ int encode_map_3d_u8(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d
                      uint64_t stride1_bytes, uint64_t stride2_bytes, uint32_t b0, uint32_t b1,
                      uint32_t b2);
 int step_nslot(int ny, int nx, int rows_per_strip);
+// Rows per strip for a step over `warp_rows` rows of 128-column spans (of all
+// members) on a GPU that holds `warps` of the kernel's warps at a time.
+int strip_rows(int64_t warp_rows, int warps);
 
 }  // namespace flood

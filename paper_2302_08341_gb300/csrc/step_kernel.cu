@@ -158,6 +158,26 @@ int step_nslot(int ny, int nx, int rows_per_strip)
     return ((ny + rows_per_strip - 1) / rows_per_strip) * ((nx + kSpan - 1) / kSpan);
 }
 
+// A warp's cost is its rows plus about four rows' time of start-up (the first
+// copies' latency) and halo, so strips should be long; but a warp's rows run
+// one after the other (1.1 us each at low occupancy), so as long as every
+// strip finds a place at once, shorter ones finish sooner.  Measured (us per
+// step):
+//  - all strips resident at once with at most 12 rows: the shortest such
+//    strips (1024 x 1024 x 1: 3 rows 14, 8 rows 16.5; 2000 x 2000 x 1: 12 rows
+//    32, 4 rows 34; 600 x 707 x 8: 12 rows 28, 8 rows (1.2 rounds) 33);
+//  - a few rounds of strips: 12 rows (1000 x 1000 x 16: 12 rows 83, 32 rows 96,
+//    4 rows 100; 2000 x 2000 x 8: 145, 148, 179);
+//  - from about eight rounds of 24 rows on, 24 (2000 x 2000 x 96: 24 rows 1420,
+//    64 rows 1533, 12 rows 1486; neighbouring strips' halo rows then still
+//    meet in L2).
+int strip_rows(int64_t warp_rows, int warps)
+{
+    const int64_t one = (warp_rows + warps - 1) / warps;  // rows a warp when all are resident
+    if (one <= 12) return (int)(one < 1 ? 1 : one);
+    return warp_rows >= (int64_t)warps * 24 * 8 ? 24 : 12;
+}
+
 // members_per_cta: warps of one CTA hold this many members of the same span
 // (1: one member over 4 spans, for single members; 2: 2 members x 2 spans;
 // 4 or 8: 4 or 8 members of one span).

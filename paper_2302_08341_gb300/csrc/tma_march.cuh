@@ -22,11 +22,16 @@
 // spans holding the edge take (the edge spans ran both forms of every link);
 // the row's four depths share one test for negative values; a row's depth,
 // bed and roughness are read again from its stage rather than carried over,
-// so the row loop needs no unrolling to stay free of moves.  2000 x 2000
-// cells x 96 members: 1.63 -> 1.42 ms per step; 1000 x 1000 x 16: 105 -> 83 us.
+// so the row loop needs no unrolling to stay free of moves; the row is
+// compiled apart for spans without the grid's last column and for its last
+// row: 350 instructions a row.  2000 x 2000 cells x 96 members: 1.63 -> 1.42 ms
+// per step, where memory binds (96 % of the measured copy rate); 1000 x 1000 x
+// 16: 105 -> 83 us.
 // Two spans a warp (one wait and one link west for 256 cells, 12 warps per SM
 // instead of 20) measured the same or slower at every size but one.
 #pragma once
+
+#include <type_traits>
 
 #include "march.cuh"
 #include "tma.cuh"
@@ -234,9 +239,10 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
     float* pc = ck ? ck + (size_t)r0 * ld + c : nullptr;
     float* ph = TRACK_MAX ? hm + (size_t)r0 * ld + c : nullptr;
 
-#pragma unroll 1
-    for (int r = r0; r < r1; ++r) {
-        const bool has_s = (r + 1 < ny);
+    // One row.  HAS_S: not the grid's last row; FULL: a span without the grid's
+    // last column.  False if the wait for the row below gave up.
+    auto row = [&](int r, auto has_s_t, auto full_t) -> bool {
+        constexpr bool has_s = decltype(has_s_t)::value, full = decltype(full_t)::value;
         if (has_s && !wait_slot(sN, phN, budget)) {
             drain_and_fail(r + 1, min(rb, r + kNS));
             return false;
@@ -293,8 +299,8 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         if (lane == 0) qW0 = qH;
         const float2 wa = make_float2(__fsub_rn(qW0, qE.a.x), __fsub_rn(qE.a.x, qE.a.y));
         const float2 wb = make_float2(__fsub_rn(qE.a.y, qE.b.x), __fsub_rn(qE.b.x, qE.b.y));
-        const float2 na = __fadd2_rn(wa, __ffma2_rn(qS.a, lk2.m1, qN.a));
-        const float2 nb = __fadd2_rn(wb, __ffma2_rn(qS.b, lk2.m1, qN.b));
+        const float2 na = __fadd2_rn(wa, sub2(qN.a, qS.a, lk2.m1));
+        const float2 nb = __fadd2_rn(wb, sub2(qN.b, qS.b, lk2.m1));
         // the step's increment (fluxes and rain) is formed first and added
         // to the depth once: adding the same rain depth to every cell on its
         // own rounds every cell of a binade the same way, a bias that builds
@@ -376,7 +382,20 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         sC = sN;
         sN = (sN + 1) & (kNS - 1);
         if (sN == 0) phN ^= 1u;
+        return true;
+    };
+    const int rS = min(r1, ny - 1);  // rows with a row below them
+    int r = r0;
+    if (full) {
+#pragma unroll 1
+        for (; r < rS; ++r)
+            if (!row(r, std::true_type{}, std::true_type{})) return false;
+    } else {
+#pragma unroll 1
+        for (; r < rS; ++r)
+            if (!row(r, std::true_type{}, std::false_type{})) return false;
     }
+    if (r < r1) row(r, std::false_type{}, std::false_type{});
 
     out.hmax = hmax;
     out.bad = !(hmax <= 3.0e38f);  // a NaN or an overflow anywhere
