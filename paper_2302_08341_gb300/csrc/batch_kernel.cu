@@ -5,6 +5,7 @@
 // march as the ensemble kernel.  Scenarios that reached min(window end, own
 // end time) are idle.
 #include "batch.cuh"
+#include "launch.cuh"
 #include "march.cuh"
 #include "tma_march.cuh"
 
@@ -17,6 +18,8 @@ namespace {
 // toward min(window end, own end time), clock, rain volume.
 __global__ void batch_plan_kernel(const BatchArgs a, int n_scen)
 {
+    pdl_launch();
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_scen) return;
     const ScenDesc sd = a.scen[i];
@@ -123,6 +126,8 @@ __global__ void __launch_bounds__(32 * W, 20 / W) batch_tma_kernel(const BatchAr
     const int lane = threadIdx.x;
     const int w = threadIdx.y;
     const int tid = blockIdx.x * W + w;
+    pdl_launch();
+    pdl_wait();
     if (tid >= a.ntasks) return;  // whole warps; no block-wide barriers below
     const WarpTask tk = a.tasks[tid];
     const int i = tk.scen;
@@ -402,9 +407,9 @@ void launch_tma_w(const BatchArgs& a, cudaStream_t s)
 {
     const unsigned g = (a.ntasks + W - 1) / W;
     if (a.limiter)
-        batch_tma_kernel<W, 1, LC><<<g, dim3(32, W), tma_march_smem_bytes(W), s>>>(a);
+        launch_pdl(batch_tma_kernel<W, 1, LC>, g, dim3(32, W), tma_march_smem_bytes(W), s, a);
     else
-        batch_tma_kernel<W, 0, LC><<<g, dim3(32, W), tma_march_smem_bytes(W), s>>>(a);
+        launch_pdl(batch_tma_kernel<W, 0, LC>, g, dim3(32, W), tma_march_smem_bytes(W), s, a);
 }
 
 }  // namespace
@@ -440,7 +445,7 @@ cudaError_t launch_batch_persistent(const PersistArgs& q, cudaStream_t s)
 
 void launch_batch_plan(const BatchArgs& a, int n_scen, cudaStream_t s)
 {
-    batch_plan_kernel<<<(n_scen + 127) / 128, 128, 0, s>>>(a, n_scen);
+    launch_pdl(batch_plan_kernel, (n_scen + 127) / 128, 128, 0, s, a, n_scen);
 }
 
 void launch_batch_step(const BatchArgs& a, int warps_per_cta, cudaStream_t s)

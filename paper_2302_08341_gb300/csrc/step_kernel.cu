@@ -18,6 +18,7 @@
 //
 // HBM traffic per member-cell-step: read h, qx, qy (12 B), write h, qx, qy
 // (12 B); z and n (8 B) once per tile for the WM members.
+#include "launch.cuh"
 #include "march.cuh"
 
 namespace flood {
@@ -35,6 +36,8 @@ constexpr int kSpan = 128;  // columns per warp
 // (when logging) the step record and checkpoint slot.
 __global__ void plan_kernel(const StepArgs a)
 {
+    pdl_launch();
+    pdl_wait();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= a.M) return;
     const MemberClock in = a.ms_in[m];
@@ -150,7 +153,7 @@ __global__ void __launch_bounds__(32 * WM * WC, (LC ? 4 : FLOOD_STEP_MIN_BLOCKS)
 
 void launch_plan(const StepArgs& a, cudaStream_t s)
 {
-    plan_kernel<<<(a.M + 127) / 128, 128, 0, s>>>(a);
+    launch_pdl(plan_kernel, (a.M + 127) / 128, 128, 0, s, a);
 }
 
 int step_nslot(int ny, int nx, int rows_per_strip)

@@ -4,6 +4,7 @@
 // streams its rows through shared memory (tma_march.cuh).
 #include <cudaTypedefs.h>
 
+#include "launch.cuh"
 #include "tma_march.cuh"
 
 namespace flood {
@@ -28,6 +29,8 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
     const int w = threadIdx.y;
     const int m = blockIdx.x * WM + w;
     int span = blockIdx.y, strip = blockIdx.z;
+    pdl_launch();
+    pdl_wait();
     if (a.tiles) {  // only the tiles that hold a cell of the domain are launched
         const int2 tl = a.tiles[blockIdx.y];
         span = tl.x;
@@ -108,6 +111,8 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(false) / WM) replay_
     const int w = threadIdx.y;
     const int m = blockIdx.x * WM + w;
     const int c0 = blockIdx.y * kSpan;
+    pdl_launch();
+    pdl_wait();
     if (m >= a.M || c0 >= a.nx) return;  // whole warps; no block-wide barriers below
     if (*reinterpret_cast<volatile const int*>(a.err) & 2) return;
     const int j = a.seg_first + a.replay_i;
@@ -207,7 +212,7 @@ void launch_tma_wm(const TmaArgs& t, cudaStream_t s)
     }
     const StepArgs& a = t.a;
     const dim3 grid((a.M + WM - 1) / WM, a.tiles ? a.n_tiles : spans_of(a), a.tiles ? 1 : strips_of(a));
-    f<<<grid, dim3(32, WM), shm, s>>>(t);
+    launch_pdl(f, grid, dim3(32, WM), shm, s, t);
 }
 
 // Members per CTA: 4 or 1 for every variant; the plain step also has 2 and 8
@@ -237,7 +242,7 @@ void launch_replay_wm(const TmaArgs& t, cudaStream_t s)
         attr = true;
     }
     const StepArgs& a = t.a;
-    f<<<dim3((a.M + WM - 1) / WM, spans_of(a), strips_of(a)), dim3(32, WM), shm, s>>>(t);
+    launch_pdl(f, dim3((a.M + WM - 1) / WM, spans_of(a), strips_of(a)), dim3(32, WM), shm, s, t);
 }
 
 template <int LIM, bool LC>
