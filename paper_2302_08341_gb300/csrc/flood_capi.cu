@@ -565,6 +565,7 @@ int flood_ensemble_init(flood_grid* g, int M, const float* h0, int h0_per_member
     CK(g, cudaMemsetAsync(g->vacc, 0, sizeof(double) * M * g->nslot * 2, s));
     CK(g, cudaMemsetAsync(g->rain_acc, 0, sizeof(double) * M, s));
     CK(g, cudaMemsetAsync(g->inflow_acc, 0, sizeof(double) * M, s));
+    CK(g, cudaMemsetAsync(g->pf_small, 0, sizeof(int32_t) * 4, s));
     CK(g, cudaMemsetAsync(g->err, 0, sizeof(int), s));
     g->k = 0;
     flood::launch_hmax(g->state, g->ms, M, g->ny, g->nx, g->ld, g->plane, g->n_sm, s);
@@ -710,7 +711,7 @@ int pf_assimilate(flood_grid* g, int G, const float* y, const double* d, const d
     a.ms = g->ms + (g->k % 3) * M;
     a.M = M;
     a.G = G;
-    flood::launch_pf(a, s);
+    CK(g, flood::launch_pf(a, s));
     flood::launch_copy(g->state, a.ms, a.n_copy, a.copy_dst, a.copy_src, M, g->plane, g->n_sm, s);
     g->launches += 2;
     if (g->lc_on) {  // land-cover parameters follow their particle

@@ -296,13 +296,16 @@ void launch_gauge(const float* state, const MemberClock* ms, const int32_t* cell
     gauge_kernel<<<(n + 127) / 128, 128, 0, s>>>(state, ms, cells, G, M, ld, nx, plane, y);
 }
 
-void launch_pf(const PfArgs& a, cudaStream_t s)
+cudaError_t launch_pf(const PfArgs& a, cudaStream_t s)
 {
-    // the shared memory that more members would need is refused at the launch
+    // the shared memory of more members is refused here, before anything is
+    // launched that would read what the filter did not write
+    if (a.M > kPfMaxMembers) return cudaErrorInvalidValue;
     static const bool attr = cudaFuncSetAttribute(pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                   (int)pf_smem(kPfMaxMembers)) == cudaSuccess;
     (void)attr;
     pf_kernel<<<1, kPfThreads, pf_smem(a.M), s>>>(a);
+    return cudaGetLastError();
 }
 
 void launch_copy(float* state, const MemberClock* ms, const int32_t* n_copy, const int32_t* dsts,
