@@ -68,6 +68,8 @@ void free_ensemble(flood_grid* g)
     dfree(g->gnm); dfree(g->gn_out); dfree(g->gpart); dfree(g->seg_end); dfree(g->samp_step);
     dfree(g->samp_y); dfree(g->samp_d); dfree(g->samp_cells); dfree(g->closs);
     dfree(g->hmax_field); dfree(g->lc_n); dfree(g->lc_drain); dfree(g->dacc);
+    dfree(g->rs_words); dfree(g->rs_xch); dfree(g->rs_seq);
+    g->rs_words = nullptr; g->rs_xch = nullptr; g->rs_seq = nullptr; g->rs_shape = {0, 0, 0};
     dfree(g->inflow_acc); dfree(g->lc_adj); dfree(g->lc_cgrad); dfree(g->gdpart); dfree(g->lc_dgrad);
     g->inflow_acc = nullptr; g->lc_adj = nullptr; g->lc_cgrad = nullptr; g->gdpart = nullptr;
     g->lc_dgrad = nullptr;
@@ -228,6 +230,51 @@ static int launch_one(flood_grid* g, double t_end, cudaStream_t s)
     return FLOOD_OK;
 }
 
+// Whether the next steps stay on the chip: the default engine with its
+// automatic launch shape, members that fit (resident_shape), and nothing asked
+// for that times or limits single step kernels.
+static bool resident_now(const flood_grid* g, ResidentShape* sh)
+{
+    if (g->engine != 1 || !g->maps_ok || g->profile || g->launch_fixed || g->wait_budget >= 0) return false;
+    *sh = resident_shape(g->ny, g->nx, g->M, g->n_sm, g->smem_max, g->track_max, g->lc_on);
+    return sh->bands > 0;
+}
+
+// The buffers of steps in that shape (allocates: not while capturing).
+static int resident_buffers(flood_grid* g, const ResidentShape& sh)
+{
+    if (g->rs_words && g->rs_shape.bands >= sh.bands) return FLOOD_OK;
+    const size_t n = (size_t)2 * g->M * sh.bands;
+    int rc;
+    if ((rc = dalloc(g, &g->rs_words, n)) || (rc = dalloc(g, &g->rs_xch, n * 2 * g->ld)) ||
+        (rc = dalloc(g, &g->rs_seq, g->M)))
+        return rc;
+    CK(g, cudaMemset(g->rs_words, 0, sizeof(unsigned long long) * n));
+    CK(g, cudaMemset(g->rs_xch, 0, sizeof(unsigned long long) * n * 2 * g->ld));
+    CK(g, cudaMemset(g->rs_seq, 0, sizeof(uint32_t) * g->M));
+    g->rs_shape = sh;
+    return FLOOD_OK;
+}
+
+// n steps of every member in one launch.
+static int launch_resident_run(flood_grid* g, const ResidentShape& sh, int n, double t_end, cudaStream_t s)
+{
+    ResidentArgs t{};
+    t.a = step_args(g, t_end);
+    t.ms_end = g->ms + ((g->k + n) % 3) * g->M;
+    t.ms_next = g->ms + ((g->k + n + 1) % 3) * g->M;
+    t.words = g->rs_words;
+    t.xch = g->rs_xch;
+    t.seq = g->rs_seq;
+    t.bands = sh.bands;
+    t.rows = sh.rows;
+    t.n_steps = n;
+    CK(g, launch_resident(t, sh, s));
+    g->k += n;
+    g->launches++;
+    return FLOOD_OK;
+}
+
 // Steps per captured run: a multiple of the member-clock ring's period (3),
 // so that a run captured at ring phase 0 replays at every later phase 0.
 static constexpr int kGraphSteps = 24;
@@ -247,6 +294,13 @@ static std::vector<unsigned char> graph_key(const flood_grid* g, double t_end)
     const int v[4] = {g->engine, g->members_per_cta, g->maps_ok ? 1 : 0, g->n_tiles};
     put(v, sizeof v);
     put(&g->tiles, sizeof g->tiles);
+    ResidentShape sh{0, 0, 0};
+    const bool res = resident_now(g, &sh);
+    const int w[3] = {res ? 1 : 0, sh.bands, sh.rows};
+    put(w, sizeof w);
+    put(&g->rs_words, sizeof g->rs_words);
+    put(&g->rs_xch, sizeof g->rs_xch);
+    put(&g->rs_seq, sizeof g->rs_seq);
     if (g->engine == 1 && g->maps_ok) {
         put(&g->state_map, sizeof g->state_map);
         put(a.lc_on ? &g->static_map_lc : &g->static_map, sizeof(CUtensorMap));
@@ -276,7 +330,11 @@ static int ensure_graph(flood_grid* g, double t_end)
     const int64_t k0 = g->k, l0 = g->launches;
     CK(g, cudaStreamBeginCapture(g->cap_stream, cudaStreamCaptureModeRelaxed));
     int rc = FLOOD_OK;
-    for (int i = 0; i < kGraphSteps && rc == FLOOD_OK; ++i) rc = launch_one(g, t_end, g->cap_stream);
+    ResidentShape sh;
+    if (resident_now(g, &sh))
+        rc = launch_resident_run(g, sh, kGraphSteps, t_end, g->cap_stream);
+    else
+        for (int i = 0; i < kGraphSteps && rc == FLOOD_OK; ++i) rc = launch_one(g, t_end, g->cap_stream);
     cudaGraph_t graph = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(g->cap_stream, &graph);
     g->graph_launch_delta = g->launches - l0;
@@ -305,25 +363,51 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
 {
     g->epoch++;
     int64_t i = 0;
-    // runs of kGraphSteps steps from a captured graph (steps timed one by one
-    // and the adjoint's logged steps launch plainly); the steps before ring
-    // phase 0 and the remainder launch plainly
-    if (g->graphs && !g->profile && !g->logging && count >= kGraphSteps + 2) {
-        for (; g->k % 3 != 0; ++i) {
+    ResidentShape sh;
+    const bool res = resident_now(g, &sh);
+    if (res) {
+        const int rc = resident_buffers(g, sh);
+        if (rc) return rc;
+    }
+    // up to `n` steps, however they run
+    auto some = [&](int n) -> int {
+        i += n;
+        if (res) return launch_resident_run(g, sh, n, t_end, s);
+        for (int q = 0; q < n; ++q) {
             const int rc = launch_one(g, t_end, s);
             if (rc) return rc;
         }
-        const int rc = ensure_graph(g, t_end);
-        if (rc) return rc;
-        for (; count - i >= kGraphSteps; i += kGraphSteps) {
+        return FLOOD_OK;
+    };
+    // runs of kGraphSteps steps from a captured graph (steps timed one by one
+    // and the adjoint's logged steps launch plainly); the steps before ring
+    // phase 0 and the remainder launch plainly.  Resident steps run in the
+    // same pieces with and without graphs
+    const bool graphs = g->graphs && !g->profile && !g->logging;
+    if ((graphs || res) && count >= kGraphSteps + 2) {
+        if (g->k % 3 != 0) {
+            const int rc = some((int)(3 - g->k % 3));
+            if (rc) return rc;
+        }
+        if (graphs) {
+            const int rc = ensure_graph(g, t_end);
+            if (rc) return rc;
+        }
+        while (count - i >= kGraphSteps) {
+            if (!graphs) {
+                const int rc = some(kGraphSteps);
+                if (rc) return rc;
+                continue;
+            }
             CK(g, cudaGraphLaunch(g->gexec, s));
+            i += kGraphSteps;
             g->k += kGraphSteps;
             g->launches += g->graph_launch_delta;
             g->graph_replays++;
         }
     }
-    for (; i < count; ++i) {
-        const int rc = launch_one(g, t_end, s);
+    while (i < count) {
+        const int rc = some(res ? (int)(count - i) : 1);
         if (rc) return rc;
     }
     CK(g, cudaGetLastError());
@@ -454,6 +538,11 @@ int flood_create_grid(flood_grid** out, int ny, int nx, const float* z, const fl
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&g->n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (g->n_sm <= 0) g->n_sm = 1;
+    int smem = 0;
+    cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    int coop = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    g->smem_max = coop && smem > 0 ? (size_t)smem : 0;
     int rc;
     if ((rc = dalloc(g, &g->zn, 2 * g->plane)) || (rc = dalloc(g, &g->err, 1))) {
         g_static_msg = g->msg;
@@ -525,7 +614,8 @@ int flood_ensemble_init(flood_grid* g, int M, const float* h0, int h0_per_member
         g->rows_per_strip = choose_rows_per_strip(g->ny, g->nx, M, g->n_sm);
         g->members_per_cta = choose_members_per_cta(M);
     }
-    g->nslot = flood::step_nslot(g->ny, g->nx, g->rows_per_strip);
+    // (a resident band takes a slot too: at most one per SM)
+    g->nslot = std::max(flood::step_nslot(g->ny, g->nx, g->rows_per_strip), g->n_sm);
     g->part_cap = (g->ny + 15) / 16;
     int rc;
     if ((rc = dalloc(g, &g->state, (size_t)2 * M * 3 * g->plane)) ||
@@ -1032,6 +1122,30 @@ extern "C" int flood_autotune(flood_grid* g, int steps_per_trial, int* best_rows
             bc = cd;
         }
     }
+    // where the automatic choice keeps the steps on the chip, it competes too:
+    // the shape reported is then the best of the others, which it leaves unused
+    bool automatic = false;
+    if (!rc) {
+        g->launch_fixed = false;
+        g->engine = 1;
+        flood::ResidentShape sh;
+        if (flood::resident_now(g, &sh)) {
+            rc = launch_steps(g, 3, -1.0, s);
+            if (!rc) cudaEventRecord(e0, s);
+            if (!rc) rc = launch_steps(g, steps_per_trial, -1.0, s);
+            if (!rc) {
+                cudaEventRecord(e1, s);
+                cudaEventSynchronize(e1);
+                float t = 0.0f;
+                cudaEventElapsedTime(&t, e0, e1);
+                const double per = t / steps_per_trial;
+                if (per < best) {
+                    best = per;
+                    automatic = true;
+                }
+            }
+        }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     // restore the ensemble exactly as it was
@@ -1060,8 +1174,8 @@ extern "C" int flood_autotune(flood_grid* g, int steps_per_trial, int* best_rows
         return rc;
     }
     if (rc2) return rc2;
-    if ((rc = flood_set_launch(g, bc.rows, bc.mpc))) return rc;
-    g->engine = bc.engine;
+    if ((rc = automatic ? flood_set_launch(g, 0, 0) : flood_set_launch(g, bc.rows, bc.mpc))) return rc;
+    g->engine = automatic ? 1 : bc.engine;
     // volume slots now follow the chosen shape; restore the saved sums into slot 0 of each member
     {
         std::vector<double> v((size_t)M * g->nslot * 2, 0.0);

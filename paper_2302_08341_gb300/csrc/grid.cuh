@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "flood_internal.cuh"
+#include "resident.cuh"
 #include "trace.cuh"
 
 struct flood_grid {
@@ -42,6 +43,12 @@ struct flood_grid {
     int rows_per_strip = 64;
     int members_per_cta = 4;
     bool launch_fixed = false;    // set by flood_set_launch
+    // steps that stay on the chip (step_resident.cu)
+    size_t smem_max = 0;          // shared memory a CTA may have
+    unsigned long long* rs_words = nullptr;  // band words, exchange rows, step numbers
+    unsigned long long* rs_xch = nullptr;
+    uint32_t* rs_seq = nullptr;
+    flood::ResidentShape rs_shape{0, 0, 0};  // the shape the buffers were sized for
     // particle filter
     int G = 0, G_cap = 0;
     int32_t* cells = nullptr;     // [G_cap]
