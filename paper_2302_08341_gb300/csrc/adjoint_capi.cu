@@ -31,7 +31,12 @@ int grow(flood_grid* g, T** p, size_t& have, size_t count)
     return flood::dalloc(g, p, count);
 }
 
-// The reverse stencil's automatic strip height (12 warps per SM).
+// The reverse stencil's automatic strip height.  The scalar gradients are FP64
+// sums of one compensated FP32 sum per strip and lane, so their last digits
+// (1e-7 relative) follow the strips: this rule keeps them where they are.  It
+// is within 8 % of the best height at the sizes measured (us per step, replay
+// included: 1000 x 1000 x 24 376 at its 32 rows, 364 at 16; 1024 x 1024 x 1 42 at
+// 4, 40 at 6; 600 x 707 x 8 98 at 4, 90 at 8).
 int reverse_rows(int ny, int nx, int M, int n_sm)
 {
     const int spans = (nx + 127) / 128;
@@ -226,14 +231,9 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
                           cudaMemcpyHostToDevice, s));
     CK(g, cudaMemcpyAsync(g->samp_d, d.data(), sizeof(double) * ns * G, cudaMemcpyHostToDevice, s));
 
-    // land cover: each member's Manning n field and the share of the rain
-    // that stays, from the classes (the step looks them up per cell)
     const size_t plane = g->plane;
-    if (g->lc_on && (rc = flood::land_adjoint_fields(g, s))) return rc;
-
     // tensor maps of the TMA-staged replay and reverse stencil (direct loads
-    // otherwise); short strips never fill the reverse stencil's copy
-    // pipeline, so those keep its direct-load form
+    // otherwise)
     flood::AdjTmaArgs tma{};
     bool use_tma = g->engine == 1 && g->maps_ok;
     if (use_tma) {
@@ -251,8 +251,15 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         // with land cover the bed and the class codes, as the forward stages them
         tma.static_map = g->lc_on ? g->static_map_lc : g->static_map;
     }
-    const bool tma_replay = use_tma;
-    const bool tma_reverse = use_tma && rrows >= 16;
+    // land cover with direct loads: each member's Manning n field and the share
+    // of the rain that stays, from the classes (the TMA form looks them up)
+    const bool fields = g->lc_on && !use_tma;
+    if (fields && (rc = flood::land_adjoint_fields(g, s))) return rc;
+
+    // the steps whose result some member is observed after
+    std::vector<std::vector<int32_t>> seen(M);
+    for (int m = 0; m < M; ++m)
+        for (int si = 0; si < ns; ++si) seen[m].push_back(samp_step[(size_t)si * M + m]);
 
     const int kmax = *std::max_element(K_m.begin(), K_m.end());
     const int n_seg = (kmax + K - 1) / K;
@@ -277,13 +284,13 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         a.seg_end = g->seg_end;
         a.seg_first = first;
         flood::TmaArgs rt;
-        if (tma_replay) {
+        if (use_tma) {
             rt.state_map = tma.seg_map;
             rt.static_map = g->lc_on ? g->static_map_lc : g->static_map;
         }
         for (int i = 0; i < len; ++i) {
             a.replay_i = i;
-            if (tma_replay) {
+            if (use_tma) {
                 rt.a = a;
                 flood::launch_replay_tma(rt, g->members_per_cta, s);
             } else {
@@ -297,10 +304,10 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         b.gn = grad_n ? g->gnm : nullptr;
         b.gpart = g->gpart;
         b.z = g->z;
-        b.n = g->lc_on ? g->lc_adj + plane : g->n;
-        b.n_mstride = g->lc_on ? plane : 0;
-        b.rw = g->lc_on ? g->lc_adj + (size_t)(M + 1) * plane : nullptr;
-        b.dflag = g->lc_on ? g->lc_adj + (size_t)(M + 2) * plane : nullptr;
+        b.n = fields ? g->lc_adj + plane : g->n;
+        b.n_mstride = fields ? plane : 0;
+        b.rw = fields ? g->lc_adj + (size_t)(M + 1) * plane : nullptr;
+        b.dflag = fields ? g->lc_adj + (size_t)(M + 2) * plane : nullptr;
         b.gdpart = g->lc_on ? g->gdpart : nullptr;
         if (g->lc_on) {
             b.lc_n = g->lc_n;
@@ -329,14 +336,24 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         for (int i = 0; i < len; ++i) {
             b.rev_i = i;
             b.lam_in = lam_in;
-            flood::launch_seed(b, g->samp_step, g->samp_y, g->samp_d, g->samp_cells, ns, G, s);
-            if (tma_reverse) {
+            // sensitivities of the loss enter where a member's step ends at an
+            // observation: few steps, the others launch nothing
+            bool seed = false;
+            for (int m = 0; m < M && !seed; ++m) {
+                const int after = seg_end[m] - i;  // the step's result, counted from the start
+                seed = after > first && std::binary_search(seen[m].begin(), seen[m].end(), after);
+            }
+            if (seed) {
+                flood::launch_seed(b, g->samp_step, g->samp_y, g->samp_d, g->samp_cells, ns, G, s);
+                g->launches++;
+            }
+            if (use_tma) {
                 tma.a = b;
                 flood::launch_adjoint_tma(tma, g->members_per_cta, s);
             } else {
                 flood::launch_adjoint(b, g->members_per_cta, s);
             }
-            g->launches += 2;
+            g->launches++;
             lam_in = 1 - lam_in;
         }
         CK(g, cudaGetLastError());

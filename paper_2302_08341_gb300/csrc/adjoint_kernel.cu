@@ -18,25 +18,17 @@
 // HBM traffic per member-cell-step: state before the step (12 B), depth after
 // it (4 B), lambda in (12 B), lambda out (12 B), per-cell Manning gradient
 // read + write (8 B), z and n shared per tile.
+#include <type_traits>
+
 #include "adjoint.cuh"
 #include "adjoint_row.cuh"
+#include "launch.cuh"
 
 namespace flood {
 
 namespace {
 
 constexpr int kSpan = 128;
-
-__device__ __forceinline__ void load4(float (&v)[4], const float* p)
-{
-    float4 t = ldg4(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-}
-
-__device__ __forceinline__ void store4(float* p, const float (&v)[4])
-{
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
 
 // RW: land cover (per-member Manning n fields, rain weighed by the runoff
 // coefficient, drainage partials), with the registers of three CTAs per SM.
@@ -49,6 +41,8 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
     const int m = blockIdx.x * WM + wm;
     const int span = blockIdx.y * WC + wc;
     const int c0 = span * kSpan;
+    pdl_launch();
+    pdl_wait();
     if (m >= a.M || c0 >= a.nx) return;
 
     const int nx = a.nx, ny = a.ny, ld = a.ld;
@@ -95,23 +89,24 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
     float* __restrict__ gn = a.gn ? a.gn + (size_t)m * plane : nullptr;
     const bool east_halo = (lane == 31) && (c + 4 < nx);
 
-    float hC[4] = {0, 0, 0, 0}, zC[4] = {0, 0, 0, 0}, nC[4] = {0, 0, 0, 0}, lC[4] = {0, 0, 0, 0};
-    float carH[4] = {0, 0, 0, 0}, carN[4] = {0, 0, 0, 0};  // north link: mu*dh2, mu*dnl
+    const Link2K k2 = link2_k(k, s_half);
+    auto ldg_quad = [](const float* p) -> Quad {
+        const float4 v = ldg4(p);
+        return Quad{make_float2(v.x, v.y), make_float2(v.z, v.w)};
+    };
+    // a row's values (lambda~: zero where the step clamped)
+    auto load_row = [&](size_t o) -> AdjRow {
+        return AdjRow{ldg_quad(sh + o), ldg_quad(z + o), ldg_quad(n + o), masked(ldg_quad(h1p + o), ldg_quad(lin + o))};
+    };
+    const AdjRow none{quad_of(0.0f), quad_of(0.0f), quad_of(0.0f), quad_of(0.0f)};
+    AdjRow C = none;
+    Quad carH = quad_of(0.0f), carN = quad_of(0.0f);  // north link: mu*dh2, mu*dnl
     if (act) {
         const size_t o = (size_t)r0 * ld + c;
-        load4(hC, sh + o); load4(zC, z + o); load4(nC, n + o);
-        float ha[4], la[4];
-        load4(ha, h1p + o); load4(la, lin + o);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) lC[q] = masked(ha[q], la[q]);
+        C = load_row(o);
         if (r0 > 0) {  // the strip's north links, recomputed
             const size_t u = o - ld;
-            float hU[4], zU[4], nU[4], qU[4], lqU[4], haU[4], lhU[4], lU[4];
-            load4(hU, sh + u); load4(zU, z + u); load4(nU, n + u); load4(qU, sqy + u);
-            load4(lqU, lin + 2 * plane + u); load4(haU, h1p + u); load4(lhU, lin + u);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) lU[q] = masked(haU[q], lhU[q]);
-            north_carry<LIM>(hU, zU, nU, qU, lqU, lU, hC, zC, nC, lC, c, nx, s_half, T, k, carH,
+            north_carry<LIM>(load_row(u), ldg_quad(sqy + u), ldg_quad(lin + 2 * plane + u), C, c, nx, k2, T, k, carH,
                              carN);
         }
     }
@@ -123,73 +118,66 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
     for (int r = r0; r < r1; ++r) {
         const size_t o = (size_t)r * ld + c;
         const bool has_s = (r + 1 < ny);
-        float hS[4] = {0, 0, 0, 0}, zS[4] = {0, 0, 0, 0}, nS[4] = {0, 0, 0, 0}, lS[4] = {0, 0, 0, 0};
-        float qxo[4] = {0, 0, 0, 0}, qyo[4] = {0, 0, 0, 0}, lqx[4] = {0, 0, 0, 0}, lqy[4] = {0, 0, 0, 0};
+        AdjRow S = none;
+        Quad qxo = quad_of(0.0f), qyo = qxo, lqx = qxo, lqy = qxo;
         if (act) {
-            if (has_s) {
-                float ha[4], la[4];
-                load4(hS, sh + o + ld); load4(zS, z + o + ld); load4(nS, n + o + ld);
-                load4(ha, h1p + o + ld); load4(la, lin + o + ld);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) lS[q] = masked(ha[q], la[q]);
-            }
-            load4(qxo, sqx + o); load4(qyo, sqy + o);
-            load4(lqx, lin + plane + o); load4(lqy, lin + 2 * plane + o);
+            if (has_s) S = load_row(o + ld);
+            qxo = ldg_quad(sqx + o);
+            qyo = ldg_quad(sqy + o);
+            lqx = ldg_quad(lin + plane + o);
+            lqy = ldg_quad(lin + 2 * plane + o);
         }
-        float hE = __shfl_down_sync(0xffffffffu, hC[0], 1);
-        float zE = __shfl_down_sync(0xffffffffu, zC[0], 1);
-        float nE = __shfl_down_sync(0xffffffffu, nC[0], 1);
-        float lE = __shfl_down_sync(0xffffffffu, lC[0], 1);
+        AdjSide E{__shfl_down_sync(0xffffffffu, C.h.a.x, 1), __shfl_down_sync(0xffffffffu, C.z.a.x, 1),
+                  __shfl_down_sync(0xffffffffu, C.n.a.x, 1), __shfl_down_sync(0xffffffffu, C.l.a.x, 1), 0.0f, 0.0f};
         if (east_halo) {
             const size_t e = o + 4;
-            hE = __ldg(sh + e); zE = __ldg(z + e); nE = __ldg(n + e);
-            lE = masked(__ldg(h1p + e), __ldg(lin + e));
+            E.h = __ldg(sh + e); E.z = __ldg(z + e); E.n = __ldg(n + e);
+            E.l = masked(__ldg(h1p + e), __ldg(lin + e));
         }
-        WestIn wi{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (lane == 0 && c0 > 0) {
-            const size_t w = o - 1;
-            wi.h = __ldg(sh + w); wi.z = __ldg(z + w); wi.n = __ldg(n + w);
-            wi.qx = __ldg(sqx + w); wi.lqx = __ldg(lin + plane + w);
-            wi.l = masked(__ldg(h1p + w), __ldg(lin + w));
+        AdjSide W{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        if (c0 > 0) {  // one cell for the whole warp
+            const size_t w = (size_t)r * ld + c0 - 1;
+            W.h = __ldg(sh + w); W.z = __ldg(z + w); W.n = __ldg(n + w);
+            W.qx = __ldg(sqx + w); W.lqx = __ldg(lin + plane + w);
+            W.l = masked(__ldg(h1p + w), __ldg(lin + w));
         }
-        float lh[4], lx[4], ly[4], gnr[4];
-        float gr_row = 0.0f, gs_row = 0.0f;
-        float rwv[4] = {0, 0, 0, 0};
+        Quad lh, lx, ly, gnr;
+        float gr_row, gs_row;
+        Quad rwv = quad_of(0.0f);
         if (RW) {
-            float dfv[4] = {0, 0, 0, 0}, haC[4] = {0, 0, 0, 0};
+            float dfv[4] = {0, 0, 0, 0};
+            Quad haC = quad_of(0.0f);
             if (act) {
-                load4(rwv, a.rw + o);
-                load4(dfv, a.dflag + o);
-                load4(haC, h1p + o);
+                rwv = ldg_quad(a.rw + o);
+                const float4 d = ldg4(a.dflag + o);
+                dfv[0] = d.x; dfv[1] = d.y; dfv[2] = d.z; dfv[3] = d.w;
+                haC = ldg_quad(h1p + o);
             }
-            kahan_add(gd_s, gd_c, drain_row(lC, haC, dfv));
+            kahan_add(gd_s, gd_c, drain_row(C.l, haC, dfv));
         }
-        if (interior)
-            adjoint_row<true, LIM, RW>(hC, zC, nC, lC, hS, zS, nS, lS, qxo, qyo, lqx, lqy, hE, zE,
-                                       nE, lE, c0 > 0, wi, has_s, c, nx, lane, s, s_half, T, k,
-                                       a.east_out, a.south_out, carH, carN, gr_row, gs_row, lh, lx,
-                                       ly, gnr, rwv);
+        auto row = [&](auto has_s_t, auto full_t) {
+            adjoint_row<decltype(has_s_t)::value, decltype(full_t)::value, LIM, RW>(
+                C, S, qxo, qyo, lqx, lqy, E, c0 > 0, W, c, nx, lane, s, s_half, T, k, k2, a.east_out, a.south_out,
+                carH, carN, gr_row, gs_row, lh, lx, ly, gnr, &rwv);
+        };
+        if (interior && has_s)
+            row(std::true_type{}, std::true_type{});
+        else if (has_s)
+            row(std::true_type{}, std::false_type{});
         else
-            adjoint_row<false, LIM, RW>(hC, zC, nC, lC, hS, zS, nS, lS, qxo, qyo, lqx, lqy, hE, zE,
-                                        nE, lE, c0 > 0, wi, has_s, c, nx, lane, s, s_half, T, k,
-                                        a.east_out, a.south_out, carH, carN, gr_row, gs_row, lh, lx,
-                                        ly, gnr, rwv);
+            row(std::false_type{}, std::false_type{});
         kahan_add(gr_s, gr_c, gr_row);
         kahan_add(gs_s, gs_c, gs_row);
         if (act) {
-            store4(lout + o, lh);
-            store4(lout + plane + o, lx);
-            store4(lout + 2 * plane + o, ly);
+            st_quad(lout + o, lh);
+            st_quad(lout + plane + o, lx);
+            st_quad(lout + 2 * plane + o, ly);
             if (gn) {
-                float4 g = *reinterpret_cast<const float4*>(gn + o);
-                g.x += gnr[0]; g.y += gnr[1]; g.z += gnr[2]; g.w += gnr[3];
-                *reinterpret_cast<float4*>(gn + o) = g;
+                const Quad g = ld_quad(gn + o);
+                st_quad(gn + o, Quad{__fadd2_rn(g.a, gnr.a), __fadd2_rn(g.b, gnr.b)});
             }
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            hC[q] = hS[q]; zC[q] = zS[q]; nC[q] = nS[q]; lC[q] = lS[q];
-        }
+        C = S;
     }
     const int slot = blockIdx.z * ((a.nx + kSpan - 1) / kSpan) + span;
     adjoint_partials(a.gpart, a.nslot, m, slot, lane, gr_s, gr_c, gs_s, gs_c, pl.rdt,
@@ -204,6 +192,8 @@ __global__ void seed_kernel(const AdjArgs a, const int32_t* __restrict__ sample_
                             const float* __restrict__ y, const double* __restrict__ d,
                             const int32_t* __restrict__ cells, int ns, int G)
 {
+    pdl_launch();
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= a.M * G) return;
     const int m = t / G, g = t % G;
@@ -237,10 +227,10 @@ void launch_adjoint_lim(const AdjArgs& a, int members_per_cta, cudaStream_t s)
     const int strips = (a.ny + a.rows_per_strip - 1) / a.rows_per_strip;
     if (members_per_cta >= 4) {
         dim3 grid((a.M + 3) / 4, spans, strips), block(32, 4);
-        adjoint_kernel<4, 1, LIM, RW><<<grid, block, 0, s>>>(a);
+        launch_pdl(adjoint_kernel<4, 1, LIM, RW>, grid, block, 0, s, a);
     } else {
         dim3 grid(a.M, (spans + 3) / 4, strips), block(32, 4);
-        adjoint_kernel<1, 4, LIM, RW><<<grid, block, 0, s>>>(a);
+        launch_pdl(adjoint_kernel<1, 4, LIM, RW>, grid, block, 0, s, a);
     }
 }
 
@@ -260,7 +250,7 @@ void launch_seed(const AdjArgs& a, const int32_t* sample_step, const float* y, c
                  const int32_t* cells, int ns, int G, cudaStream_t s)
 {
     const int n = a.M * G;
-    seed_kernel<<<(n + 127) / 128, 128, 0, s>>>(a, sample_step, y, d, cells, ns, G);
+    launch_pdl(seed_kernel, (n + 127) / 128, 128, 0, s, a, sample_step, y, d, cells, ns, G);
 }
 
 void launch_reduce_members(const float* gm, int M, int ny, int nx, int ld, size_t plane, float* out,

@@ -1,20 +1,27 @@
 // TMA-staged reverse stencil (same arithmetic and results, bit for bit, as
 // adjoint_kernel.cu, through the shared row code of adjoint_row.cuh).
 //
-// The direct-load adjoint kernel needs about 120 registers per thread, so
+// The direct-load adjoint kernel needs about 128 registers per thread, so
 // only four CTAs of four warps fit on an SM and its loads cannot keep enough
-// bytes in flight: it ran at about a third of the HBM bandwidth.  Here each
-// warp streams its rows through a ring of shared-memory stages filled by the
-// tensor memory accelerator, one row of all ten planes it reads per stage:
-// the state before the step (h, qx, qy), the depth after it, the
-// sensitivities lambda (h, qx, qy), the bed and roughness (with land cover
-// the bed and the class codes), and the member's Manning gradient, each 136
-// columns wide (the warp's 128 plus a 4-column halo on each side).  Lane 0 keeps kNS - 1 rows in flight ahead of the row
-// being computed.  Every mbarrier wait is bounded: on timeout the kernel
-// records FLOOD_ERR_TIMEOUT, waits (bounded) for its own copies in flight,
-// and returns.
+// bytes in flight.  Here each warp streams its rows through a ring of
+// shared-memory stages filled by the tensor memory accelerator, one row of all
+// ten planes it reads per stage: the state before the step (h, qx, qy), the
+// depth after it, the sensitivities lambda (h, qx, qy), the bed and roughness
+// (with land cover the bed and the class codes), and the member's Manning
+// gradient, each 136 columns wide (the warp's 128 plus a 4-column halo on each
+// side).  Lane 0 keeps kNS - 1 rows in flight ahead of the row being computed.
+// Every mbarrier wait is bounded: on timeout the kernel records
+// FLOOD_ERR_TIMEOUT, waits (bounded) for its own copies in flight, and
+// returns.  Bound by issue slots at 12 warps per SM (what the stages and 160
+// registers leave room for); with the row arithmetic in pairs the reverse and
+// replay of a step of 1000 x 1000 x 24 went from 412 to 376 us, and short
+// strips run faster than with direct loads at every size measured but one
+// 300 x 400 pair (24 against 23 us).
+#include <type_traits>
+
 #include "adjoint.cuh"
 #include "adjoint_row.cuh"
+#include "launch.cuh"
 #include "tma.cuh"
 
 namespace flood {
@@ -43,21 +50,16 @@ static_assert(kStageBytes >= (kGn + kBox) * 4 && kStageBytes % 128 == 0, "stage 
 // Land cover: the roughness plane's place holds each cell's class code (a
 // uint32), staged with the bed as in the forward step.
 
-__device__ __forceinline__ void lds4(float (&v)[4], const float* p)
+// Shared memory ahead of the stages: barriers, then the class tables of land
+// cover (64 bytes a warp).
+__host__ __device__ constexpr int head_bytes(int warps)
 {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    return 128 * ((8 * kNS * warps + 127) / 128) + 128 * ((64 * warps + 127) / 128);
 }
 
-__device__ __forceinline__ void store4(float* p, const float (&v)[4])
-{
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
-
-// LC: land cover: the roughness, runoff share and drainage flag of every
-// cell from its class (the codes come with the staged rows, the member's
-// class table lives in lanes 0..3 and is read by shuffle, so every lane takes
-// part in each lookup, outside lane-dependent branches).
+// LC: land cover: the roughness, runoff share and drainage flag of every cell
+// from its class (the codes come with the staged rows, the member's class
+// table lies in shared memory).
 template <int WM, int LIM, bool LC = false>
 __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
     const __grid_constant__ AdjTmaArgs t)
@@ -70,6 +72,8 @@ __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
     const int m = blockIdx.x * WM + w;
     const int span = blockIdx.y;
     const int c0 = span * kSpan;
+    pdl_launch();
+    pdl_wait();
     if (m >= a.M || c0 >= a.nx) return;  // whole warps; no block-wide barriers below
 
     const int nx = a.nx, ny = a.ny, ld = a.ld;
@@ -112,7 +116,8 @@ __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
     unsigned char* base = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
     const uint32_t bar0 = smem_u32(base) + 8u * kNS * w;
-    unsigned char* my_stages = base + 128 * ((8 * kNS * WM + 127) / 128) + kNS * kStageBytes * w;
+    float4* const tab = reinterpret_cast<float4*>(base + 128 * ((8 * kNS * WM + 127) / 128)) + 4 * w;
+    unsigned char* my_stages = base + head_bytes(WM) + kNS * kStageBytes * w;
     const uint32_t stage0 = smem_u32(my_stages);
 
     const int slot = j - a.seg_first;                 // seg slot of the state before the step
@@ -123,16 +128,16 @@ __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
     const int ra = r0 > 0 ? r0 - 1 : r0;   // first row loaded (north halo)
     const int rb = min(r1 + 1, ny);        // one past the last row loaded
 
+    if (LC && lane < 4)
+        tab[lane] = make_float4(a.lc_n[(size_t)m * 4 + lane], a.lc_runoff[lane], a.lc_drains[lane], 0.0f);
     if (lane == 0) {
         for (int i = 0; i < kNS; ++i) mbar_init(bar0 + 8u * i, 1);
         fence_mbar_init();
     }
     __syncwarp();
-    int issued = ra;  // rows [ra, issued) have been requested
-    auto issue = [&](int row) {
-        const int sidx = (row - ra) % kNS;
-        const uint32_t bar = bar0 + 8u * sidx;
-        const uint32_t dsts = stage0 + kStageBytes * sidx;
+    auto issue = [&](int row, int slot) {
+        const uint32_t bar = bar0 + 8u * slot;
+        const uint32_t dsts = stage0 + kStageBytes * slot;
         mbar_arrive_expect_tx(bar, tx);
         tma_load_3d(dsts + 4 * kSt, &t.seg_map, c0 - 4, row, p_before, bar);
         tma_load_3d(dsts + 4 * kHa, &t.seg1_map, c0 - 4, row, p_after, bar);
@@ -140,206 +145,146 @@ __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
         tma_load_3d(dsts + 4 * kZ, &t.static_map, c0 - 4, row, 0, bar);
         if (gn) tma_load_3d(dsts + 4 * kGn, &t.gn_map, c0 - 4, row, m, bar);
     };
-    for (; issued < rb && issued < ra + kNS; ++issued)
-        if (lane == 0) issue(issued);
-    auto wait_row = [&](int row) -> bool {
-        const int kk = row - ra;
-        return mbar_wait_bounded(bar0 + 8u * (kk % kNS), (kk / kNS) & 1, kWaitBudget);
+    if (lane == 0)
+        for (int i = 0; i < kNS && ra + i < rb; ++i) issue(ra + i, i);
+    auto wait_slot = [&](int slot, uint32_t parity) -> bool {
+        return mbar_wait_bounded(bar0 + 8u * slot, parity, kWaitBudget);
     };
-    auto row_ptr = [&](int row) -> const float* {
-        return reinterpret_cast<const float*>(my_stages + kStageBytes * ((row - ra) % kNS));
+    auto row_ptr = [&](int slot) -> const float* {
+        return reinterpret_cast<const float*>(my_stages + kStageBytes * slot);
     };
-    // recycle the oldest stage for the next row in line
-    auto release = [&]() {
+    // a row's stage takes the row kNS further on, once the whole warp has read it
+    auto release = [&](int row, int slot) {
         __syncwarp();
-        if (issued < rb) {
-            if (lane == 0) {
-                fence_proxy_async_smem();
-                issue(issued);
-            }
-            ++issued;
+        if (row + kNS < rb && lane == 0) {
+            fence_proxy_async_smem();
+            issue(row + kNS, slot);
         }
     };
-    int waited = ra;  // rows [ra, waited) have landed
-    auto drain_and_fail = [&]() {
+    // rows [from, to) are still in flight: every copy lands before the warp
+    // leaves (bounded each)
+    auto drain_and_fail = [&](int from, int to) {
         if (lane == 0) atomicOr(a.err, 2);
-        for (int row = waited; row < issued; ++row) wait_row(row);  // bounded each
+        for (int row = from; row < to; ++row) wait_slot((row - ra) % kNS, ((row - ra) / kNS) & 1);
     };
 
     const int x0 = 4 + 4 * lane;  // this lane's first cell in a tile row
-    // land cover: lane q of every group of four holds class q's roughness,
-    // runoff share and drainage flag for this member
-    float ln = 0.0f, lro = 0.0f, ldr = 0.0f;
-    if (LC) {
-        const int q = lane & 3;
-        ln = a.lc_n[(size_t)m * 4 + q];
-        lro = a.lc_runoff[q];
-        ldr = a.lc_drains[q];
-    }
-    // the classes of the lane's four cells in a staged row, one byte each
-    auto cls4 = [&](const float* R) -> uint32_t {
-        const uint4 q = *reinterpret_cast<const uint4*>(R + kN + x0);
-        return __byte_perm(__byte_perm(q.x, q.y, 0x0040u), __byte_perm(q.z, q.w, 0x0040u), 0x5410u);
+    // roughness of four staged cells, and of one (land cover: of their classes)
+    auto n_quad = [&](const float* R) -> Quad {
+        if (!LC) return ld_quad(R + kN);
+        const uint4 q = *reinterpret_cast<const uint4*>(R + kN);
+        return Quad{make_float2(tab[q.x].x, tab[q.y].x), make_float2(tab[q.z].x, tab[q.w].x)};
     };
-    // roughness of the lane's four cells / of one cell of a staged row (with
-    // land cover by shuffle: every lane calls these; the shuffle reads the
-    // five low bits of its source lane, where a class byte sits alone)
-    auto n4 = [&](float (&nv)[4], const float* R) {
-        if (LC) {
-            const uint32_t wc = cls4(R);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) nv[q] = __shfl_sync(0xffffffffu, ln, (int)(wc >> (8 * q)));
-        } else {
-            lds4(nv, R + kN + x0);
-        }
+    auto n_one = [&](const float* R) -> float { return LC ? tab[__float_as_uint(R[kN])].x : R[kN]; };
+    // a staged row's values (R: at this lane's first cell)
+    auto load_row = [&](const float* R) -> AdjRow {
+        return AdjRow{ld_quad(R + kSt), ld_quad(R + kZ), n_quad(R), masked(ld_quad(R + kHa), ld_quad(R + kLam))};
     };
-    auto n1 = [&](const float* R, int x) -> float {
-        return LC ? __shfl_sync(0xffffffffu, ln, (int)__float_as_uint(R[kN + x])) : R[kN + x];
-    };
-    float hC[4], zC[4], nC[4], lC[4];
-    float carH[4] = {0, 0, 0, 0}, carN[4] = {0, 0, 0, 0};  // north link: mu*dh2, mu*dnl
-    bool ok = true;
+    const Link2K k2 = link2_k(k, s_half);
+    int sC = 0;  // slot of row r, of row r + 1 and that row's phase
     if (r0 > 0) {
-        ok = wait_row(r0 - 1);
-        if (ok) waited = r0;
+        if (!wait_slot(0, 0)) {
+            drain_and_fail(ra, min(rb, ra + kNS));
+            return;
+        }
+        sC = 1;
     }
-    if (ok) {
-        ok = wait_row(r0);
-        if (ok) waited = r0 + 1;
-    }
-    if (!ok) {
-        drain_and_fail();
+    if (!wait_slot(sC, 0)) {
+        drain_and_fail(r0, min(rb, ra + kNS));
         return;
     }
-    {
-        const float* P = row_ptr(r0);
-        float ha[4], la[4];
-        lds4(hC, P + kSt + x0);
-        lds4(zC, P + kZ + x0);
-        n4(nC, P);
-        lds4(ha, P + kHa + x0);
-        lds4(la, P + kLam + x0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) lC[q] = masked(ha[q], la[q]);
-        if (r0 > 0) {  // the strip's north links, recomputed
-            const float* U = row_ptr(r0 - 1);
-            float hU[4], zU[4], nU[4], qU[4], lqU[4], haU[4], lhU[4], lU[4];
-            lds4(hU, U + kSt + x0);
-            lds4(zU, U + kZ + x0);
-            n4(nU, U);
-            lds4(qU, U + kSt + 2 * kBox + x0);
-            lds4(lqU, U + kLam + 2 * kBox + x0);
-            lds4(haU, U + kHa + x0);
-            lds4(lhU, U + kLam + x0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) lU[q] = masked(haU[q], lhU[q]);
-            if (act)
-                north_carry<LIM>(hU, zU, nU, qU, lqU, lU, hC, zC, nC, lC, c, nx, s_half, T, k,
-                                 carH, carN);
-            release();
-        }
+    AdjRow C = load_row(row_ptr(sC) + x0);
+    Quad carH = quad_of(0.0f), carN = quad_of(0.0f);  // north link: mu*dh2, mu*dnl
+    if (r0 > 0) {  // the strip's north links, recomputed
+        const float* U = row_ptr(0) + x0;
+        north_carry<LIM>(load_row(U), ld_quad(U + kSt + 2 * kBox), ld_quad(U + kLam + 2 * kBox), C, c, nx, k2, T, k,
+                         carH, carN);
+        release(ra, 0);
     }
 
     // FP32 compensated sums of the rows' partials (lambda~ for the rain
     // gradient, mu n dq'/dn for the scale gradient), widened to FP64 once per warp
     float gr_s = 0.0f, gr_c = 0.0f, gs_s = 0.0f, gs_c = 0.0f;
     float gd_s = 0.0f, gd_c = 0.0f;  // land cover: drainage partials
-    for (int r = r0; r < r1; ++r) {
-        const size_t o = (size_t)r * ld + c;
-        const bool has_s = (r + 1 < ny);
-        if (has_s) {
-            if (!wait_row(r + 1)) {
-                drain_and_fail();
-                return;
-            }
-            waited = r + 2;
+    int sN = sC + 1;                 // at most kNS - 1 here
+    uint32_t phN = 0;
+    size_t o = (size_t)r0 * ld + c;
+    auto row = [&](int r, auto has_s_t, auto full_t) -> bool {
+        constexpr bool has_s = decltype(has_s_t)::value, full = decltype(full_t)::value;
+        if (has_s && !wait_slot(sN, phN)) {
+            drain_and_fail(r + 1, min(rb, r + kNS));
+            return false;
         }
-        const float* P = row_ptr(r);
-        float hS[4] = {0, 0, 0, 0}, zS[4] = {0, 0, 0, 0}, nS[4] = {0, 0, 0, 0}, lS[4] = {0, 0, 0, 0};
-        float qxo[4], qyo[4], lqx[4], lqy[4];
-        lds4(qxo, P + kSt + kBox + x0);
-        lds4(qyo, P + kSt + 2 * kBox + x0);
-        lds4(lqx, P + kLam + kBox + x0);
-        lds4(lqy, P + kLam + 2 * kBox + x0);
-        if (has_s) {
-            const float* Q = row_ptr(r + 1);
-            float ha[4], la[4];
-            lds4(hS, Q + kSt + x0);
-            lds4(zS, Q + kZ + x0);
-            n4(nS, Q);
-            lds4(ha, Q + kHa + x0);
-            lds4(la, Q + kLam + x0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) lS[q] = masked(ha[q], la[q]);
-        }
+        const float* R = row_ptr(sC);
+        const float* P = R + x0;
+        AdjRow S;
+        if (has_s) S = load_row(row_ptr(sN) + x0);
+        const Quad qxo = ld_quad(P + kSt + kBox), qyo = ld_quad(P + kSt + 2 * kBox);
+        const Quad lqx = ld_quad(P + kLam + kBox), lqy = ld_quad(P + kLam + 2 * kBox);
         // east neighbour of the lane's last cell and the span's west
         // neighbour, straight from the tile's halo
-        const float hE = P[kSt + x0 + 4], zE = P[kZ + x0 + 4], nE = n1(P, x0 + 4);
-        const float lE = masked(P[kHa + x0 + 4], P[kLam + x0 + 4]);
-        const float nW = n1(P, 3);
-        WestIn wi{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (lane == 0 && c0 > 0) {
-            wi.h = P[kSt + 3]; wi.z = P[kZ + 3]; wi.n = nW;
-            wi.qx = P[kSt + kBox + 3]; wi.lqx = P[kLam + kBox + 3];
-            wi.l = masked(P[kHa + 3], P[kLam + 3]);
-        }
-        float lh[4], lx[4], ly[4], gnr[4];
-        float gr_row = 0.0f, gs_row = 0.0f;
-        float rwv[4] = {0, 0, 0, 0};
+        const AdjSide E{P[kSt + 4], P[kZ + 4], n_one(P + 4), masked(P[kHa + 4], P[kLam + 4]), 0.0f, 0.0f};
+        const AdjSide W{R[kSt + 3], R[kZ + 3], n_one(R + 3), masked(R[kHa + 3], R[kLam + 3]), R[kSt + kBox + 3],
+                        R[kLam + kBox + 3]};
+        Quad lh, lx, ly, gnr, rwv;
+        float gr_row, gs_row;
         if (LC) {
-            float dfv[4], haC[4];
-            const uint32_t wc = cls4(P);
+            float dfv[4];
+            const uint4 q = *reinterpret_cast<const uint4*>(P + kN);
+            const uint32_t code[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {  // the cells' runoff shares and drainage flags
-                const float rv = __shfl_sync(0xffffffffu, lro, (int)(wc >> (8 * q)));
-                const float dv = __shfl_sync(0xffffffffu, ldr, (int)(wc >> (8 * q)));
-                rwv[q] = act ? rv : 0.0f;
-                dfv[q] = act ? dv : 0.0f;
+            for (int j = 0; j < 4; ++j) {  // the cells' runoff shares and drainage flags
+                const float4 v = tab[code[j]];
+                quad_at(rwv, j) = act ? v.y : 0.0f;
+                dfv[j] = act ? v.z : 0.0f;
             }
-            lds4(haC, P + kHa + x0);
-            kahan_add(gd_s, gd_c, drain_row(lC, haC, dfv));
+            kahan_add(gd_s, gd_c, drain_row(C.l, ld_quad(P + kHa), dfv));
         }
-        if (interior)
-            adjoint_row<true, LIM, LC>(hC, zC, nC, lC, hS, zS, nS, lS, qxo, qyo, lqx, lqy, hE, zE,
-                                       nE, lE, c0 > 0, wi, has_s, c, nx, lane, s, s_half, T, k,
-                                       a.east_out, a.south_out, carH, carN, gr_row, gs_row, lh, lx,
-                                       ly, gnr, rwv);
-        else
-            adjoint_row<false, LIM, LC>(hC, zC, nC, lC, hS, zS, nS, lS, qxo, qyo, lqx, lqy, hE, zE,
-                                        nE, lE, c0 > 0, wi, has_s, c, nx, lane, s, s_half, T, k,
-                                        a.east_out, a.south_out, carH, carN, gr_row, gs_row, lh, lx,
-                                        ly, gnr, rwv);
+        adjoint_row<has_s, full, LIM, LC>(C, S, qxo, qyo, lqx, lqy, E, c0 > 0, W, c, nx, lane, s, s_half, T, k, k2,
+                                          a.east_out, a.south_out, carH, carN, gr_row, gs_row, lh, lx, ly, gnr, &rwv);
         kahan_add(gr_s, gr_c, gr_row);
         kahan_add(gs_s, gs_c, gs_row);
-        if (act) {
-            store4(lout + o, lh);
-            store4(lout + plane + o, lx);
-            store4(lout + 2 * plane + o, ly);
+        if (full || act) {
+            st_quad(lout + o, lh);
+            st_quad(lout + plane + o, lx);
+            st_quad(lout + 2 * plane + o, ly);
             if (gn) {
-                float g[4];
-                lds4(g, P + kGn + x0);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) g[q] += gnr[q];
-                store4(gn + o, g);
+                const Quad g = ld_quad(P + kGn);
+                st_quad(gn + o, Quad{__fadd2_rn(g.a, gnr.a), __fadd2_rn(g.b, gnr.b)});
             }
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            hC[q] = hS[q]; zC[q] = zS[q]; nC[q] = nS[q]; lC[q] = lS[q];
+        o += ld;
+        if (has_s) C = S;
+        release(r, sC);
+        sC = sN;
+        if (++sN == kNS) {
+            sN = 0;
+            phN ^= 1u;
         }
-        release();
+        return true;
+    };
+    const int rS = min(r1, ny - 1);  // rows with a row below them
+    int r = r0;
+    if (interior) {
+#pragma unroll 1
+        for (; r < rS; ++r)
+            if (!row(r, std::true_type{}, std::true_type{})) return;
+    } else {
+#pragma unroll 1
+        for (; r < rS; ++r)
+            if (!row(r, std::true_type{}, std::false_type{})) return;
     }
+    if (r < r1) row(r, std::false_type{}, std::false_type{});
     const int vslot = blockIdx.z * ((a.nx + kSpan - 1) / kSpan) + span;
     adjoint_partials(a.gpart, a.nslot, m, vslot, lane, gr_s, gr_c, gs_s, gs_c, pl.rdt,
                      1.0 / (double)s);
     if (LC) adjoint_drain_partial(a.gdpart, a.nslot, m, vslot, lane, gd_s, gd_c, pl.dt);
 }
 
-template <int WM, bool LC>
+template <int WM>
 size_t adj_smem_bytes()
 {
-    (void)LC;  // the land-cover stage has the plain layout
-    return 128 + 128 * ((8 * kNS * WM + 127) / 128) + (size_t)kNS * kStageBytes * WM;
+    return 128 + head_bytes(WM) + (size_t)kNS * kStageBytes * WM;
 }
 
 template <int LIM, bool LC>
@@ -350,18 +295,18 @@ void launch_adjoint_tma_lim(const AdjTmaArgs& t, int members_per_cta, cudaStream
     const int strips = (a.ny + a.rows_per_strip - 1) / a.rows_per_strip;
     if (members_per_cta >= 4 && a.M >= 4) {
         static bool attr = false;
-        const size_t shm = adj_smem_bytes<4, LC>();
+        const size_t shm = adj_smem_bytes<4>();
         if (!attr) {
             cudaFuncSetAttribute(adjoint_tma_kernel<4, LIM, LC>,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
             attr = true;
         }
         dim3 grid((a.M + 3) / 4, spans, strips), block(32, 4);
-        adjoint_tma_kernel<4, LIM, LC><<<grid, block, shm, s>>>(t);
+        launch_pdl(adjoint_tma_kernel<4, LIM, LC>, grid, block, shm, s, t);
     } else {
-        const size_t shm = adj_smem_bytes<1, LC>();
+        const size_t shm = adj_smem_bytes<1>();
         dim3 grid(a.M, spans, strips), block(32, 1);
-        adjoint_tma_kernel<1, LIM, LC><<<grid, block, shm, s>>>(t);
+        launch_pdl(adjoint_tma_kernel<1, LIM, LC>, grid, block, shm, s, t);
     }
 }
 
@@ -369,7 +314,7 @@ void launch_adjoint_tma_lim(const AdjTmaArgs& t, int members_per_cta, cudaStream
 
 void launch_adjoint_tma(const AdjTmaArgs& t, int members_per_cta, cudaStream_t s)
 {
-    if (t.a.rw)
+    if (t.a.lc_n)
         t.a.limiter ? launch_adjoint_tma_lim<1, true>(t, members_per_cta, s)
                     : launch_adjoint_tma_lim<0, true>(t, members_per_cta, s);
     else

@@ -35,6 +35,7 @@
 #include "grid.cuh"
 #include "launch.cuh"
 #include "march.cuh"
+#include "quad.cuh"
 #include "resident.cuh"
 
 namespace flood {
@@ -60,7 +61,7 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned l
 {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-// Four depths of an exchange row, each in a 64-bit word with the step's number
+// Quad depths of an exchange row, each in a 64-bit word with the step's number
 // above it: a word that carries the number it waits for is the value itself,
 // so no fence orders the row before a flag.
 __device__ __forceinline__ void st_tagged(unsigned long long* p, float4 v, uint32_t tag)
@@ -114,23 +115,6 @@ struct Sum2 {
         }
     }
 };
-
-struct Four {
-    float2 a, b;
-};
-__device__ __forceinline__ Four ld4(const float* p)
-{
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    return Four{make_float2(t.x, t.y), make_float2(t.z, t.w)};
-}
-__device__ __forceinline__ void st4(float* p, const Four& v)
-{
-    *reinterpret_cast<float4*>(p) = make_float4(v.a.x, v.a.y, v.b.x, v.b.y);
-}
-__device__ __forceinline__ float& at4(Four& v, int j)
-{
-    return j == 0 ? v.a.x : j == 1 ? v.a.y : j == 2 ? v.b.x : v.b.y;
-}
 
 // A step's constants, from warp 0 to the band.
 struct BandPlan {
@@ -190,8 +174,8 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
         if (g < 0 || g >= ny) continue;
         const size_t o = (size_t)g * ld + c;
         const int s = r * P + c;
-        st4(H + s, ld4(st + o));
-        st4(Z + s, ld4(a.z + o));
+        st_quad(H + s, ld_quad(st + o));
+        st_quad(Z + s, ld_quad(a.z + o));
         if (LC) {
             const uint32_t w = cls_word(a.cls, o);
             const float* tn = a.lc_n + (size_t)m * 4;
@@ -199,12 +183,12 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
                                                             tn[(w >> 24) & 3]);
             if (r >= 0 && r < R) CL[r * nq + e.q] = w;
         } else {
-            st4(N + s, ld4(a.n + o));
+            st_quad(N + s, ld_quad(a.n + o));
         }
-        if (r < R) st4(QS + s, ld4(st + 2 * a.plane + o));
+        if (r < R) st_quad(QS + s, ld_quad(st + 2 * a.plane + o));
         if (r >= 0 && r < R) {
-            st4(QE + s, ld4(st + a.plane + o));
-            if (TRACK) st4(HM + s, ld4(a.hmax_field + (size_t)m * a.plane + o));
+            st_quad(QE + s, ld_quad(st + a.plane + o));
+            if (TRACK) st_quad(HM + s, ld_quad(a.hmax_field + (size_t)m * a.plane + o));
         }
     }
 
@@ -352,10 +336,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
             const int c = 4 * e.q;
             if (e.r < R) {
                 const int s = e.r * P + c;
-                const Four h = ld4(H + s), z = ld4(Z + s), n = ld4(N + s), q = ld4(QE + s);
+                const Quad h = ld_quad(H + s), z = ld_quad(Z + s), n = ld_quad(N + s), q = ld_quad(QE + s);
                 const float hE = H[s + 4], zE = Z[s + 4], nE = N[s + 4];
                 const float2 ua = __fmul2_rn(h.a, lim2), ub = __fmul2_rn(h.b, lim2);
-                Four v;
+                Quad v;
                 v.a = link2_q<LIM>(h.a, z.a, make_float2(h.a.y, h.b.x), make_float2(z.a.y, z.b.x), q.a,
                                    make_float2(__fadd_rn(n.a.x, n.a.y), __fadd_rn(n.a.y, n.b.x)), ua,
                                    make_float2(ua.y, ub.x), k2);
@@ -366,18 +350,18 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
                         if (c + i >= nx - 1)
-                            at4(v, i) = (a.east_out && c + i == nx - 1)
+                            quad_at(v, i) = (a.east_out && c + i == nx - 1)
                                             ? outflow_q<LIM>(H[s + i], QE[s + i], __fmul_rn(scale, N[s + i]), k)
                                             : 0.0f;
                 }
-                st4(QE + s, v);
+                st_quad(QE + s, v);
             } else {
                 const int r = e.r - R - 1, g = b0 + r, s = r * P + c;
                 if (g < 0) continue;  // north of the grid: a wall
-                Four v;
+                Quad v;
                 if (g + 1 < ny) {
-                    const Four h = ld4(H + s), z = ld4(Z + s), n = ld4(N + s), q = ld4(QS + s);
-                    const Four hS = ld4(H + s + P), zS = ld4(Z + s + P), nS = ld4(N + s + P);
+                    const Quad h = ld_quad(H + s), z = ld_quad(Z + s), n = ld_quad(N + s), q = ld_quad(QS + s);
+                    const Quad hS = ld_quad(H + s + P), zS = ld_quad(Z + s + P), nS = ld_quad(N + s + P);
                     v.a = link2_q<LIM>(h.a, z.a, hS.a, zS.a, q.a, __fadd2_rn(n.a, nS.a), __fmul2_rn(h.a, lim2),
                                        __fmul2_rn(hS.a, lim2), k2);
                     v.b = link2_q<LIM>(h.b, z.b, hS.b, zS.b, q.b, __fadd2_rn(n.b, nS.b), __fmul2_rn(h.b, lim2),
@@ -385,16 +369,16 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
                 } else {
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        at4(v, i) = a.south_out
+                        quad_at(v, i) = a.south_out
                                         ? outflow_q<LIM>(H[s + i], QS[s + i], __fmul_rn(scale, N[s + i]), k)
                                         : 0.0f;
                 }
                 if (c + 4 > nx) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        if (c + i >= nx) at4(v, i) = 0.0f;
+                        if (c + i >= nx) quad_at(v, i) = 0.0f;
                 }
-                st4(QS + s, v);
+                st_quad(QS + s, v);
             }
         }
         __syncthreads();
@@ -403,13 +387,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
         float hm = 0.0f;
         for (Item e(tid, nq); e.r < R; e.next(dr_i, dq_i, nq)) {
             const int r = e.r, g = b0 + r, c = 4 * e.q, s = r * P + c;
-            const Four h = ld4(H + s), qE = ld4(QE + s), qS = ld4(QS + s), qN = ld4(QS + s - P);
+            const Quad h = ld_quad(H + s), qE = ld_quad(QE + s), qS = ld_quad(QS + s), qN = ld_quad(QS + s - P);
             const float qW = e.q > 0 ? QE[s - 1] : (g >= k.in_r0 && g < k.in_r1) ? k.q_in : 0.0f;
             const float2 na = __fadd2_rn(make_float2(__fsub_rn(qW, qE.a.x), __fsub_rn(qE.a.x, qE.a.y)),
                                          sub2(qN.a, qS.a, k2.m1));
             const float2 nb = __fadd2_rn(make_float2(__fsub_rn(qE.a.y, qE.b.x), __fsub_rn(qE.b.x, qE.b.y)),
                                          sub2(qN.b, qS.b, k2.m1));
-            Four v;
+            Quad v;
             if (!LC) {
                 v.a = __fadd2_rn(h.a, __ffma2_rn(dtdx2, na, dr2));
                 v.b = __fadd2_rn(h.b, __ffma2_rn(dtdx2, nb, dr2));
@@ -422,7 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
                     const float2 sd = s_src[(w >> (8 * i)) & 3];
                     const float hp = c + i < nx ? __fadd_rn(hh[i], __fmaf_rn(dtdx2.x, net[i], sd.x)) : 0.0f;
                     const float sink = fminf(sd.y, fmaxf(hp, 0.0f));
-                    at4(v, i) = (hp > 0.0f && sink == hp) ? -0.0f : __fsub_rn(hp, sink);
+                    quad_at(v, i) = (hp > 0.0f && sink == hp) ? -0.0f : __fsub_rn(hp, sink);
                     row_sink = __fadd_rn(row_sink, sink);
                 }
                 kahan_add(drn_s, drn_c, row_sink);
@@ -430,14 +414,14 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
             if (c + 4 > nx) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (c + i >= nx) at4(v, i) = 0.0f;
+                    if (c + i >= nx) quad_at(v, i) = 0.0f;
             }
             if (fminf(fmin3(v.a.x, v.a.y, v.b.x), v.b.y) < 0.0f) {  // wet/dry clamp (rare): keeps a negative zero
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (at4(v, i) < 0.0f) {
-                        vclamp.add(-at4(v, i));
-                        at4(v, i) = -0.0f;
+                    if (quad_at(v, i) < 0.0f) {
+                        vclamp.add(-quad_at(v, i));
+                        quad_at(v, i) = -0.0f;
                     }
             }
             hm = fmax3_nan(fmax3_nan(hm, v.a.x, v.a.y), v.b.x, v.b.y);
@@ -453,9 +437,9 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
                 vout.add_product(qS.b.x, bp.dt);
                 vout.add_product(qS.b.y, bp.dt);
             }
-            st4(H + s, v);
+            st_quad(H + s, v);
             if (TRACK) {
-                const Four o = ld4(HM + s);
+                const Quad o = ld_quad(HM + s);
                 *reinterpret_cast<float4*>(HM + s) = make_float4(fmaxf(o.a.x, v.a.x), fmaxf(o.a.y, v.a.y),
                                                                  fmaxf(o.b.x, v.b.x), fmaxf(o.b.y, v.b.y));
             }
@@ -464,9 +448,9 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
             if (r == R - 1 && b1 < ny) st_tagged(xrow(j & 1, band, 1) + c, v4, want);
             if (bp.ckpt >= 0) {
                 float* ck = a.ckpt + ((size_t)bp.ckpt * a.M + m) * mstride + (size_t)g * ld + c;
-                st4(ck, v);
-                st4(ck + a.plane, qE);
-                st4(ck + 2 * a.plane, qS);
+                st_quad(ck, v);
+                st_quad(ck + a.plane, qE);
+                st_quad(ck + 2 * a.plane, qS);
             }
         }
         const bool b_now = !(hm <= 3.0e38f);  // a NaN or an overflow
@@ -534,10 +518,10 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
     for (Item e(tid, nq); e.r < R; e.next(dr_i, dq_i, nq)) {
         const int s = e.r * P + 4 * e.q;
         const size_t o = (size_t)(b0 + e.r) * ld + 4 * e.q;
-        st4(st + o, ld4(H + s));
-        st4(st + a.plane + o, ld4(QE + s));
-        st4(st + 2 * a.plane + o, ld4(QS + s));
-        if (TRACK) st4(a.hmax_field + (size_t)m * a.plane + o, ld4(HM + s));
+        st_quad(st + o, ld_quad(H + s));
+        st_quad(st + a.plane + o, ld_quad(QE + s));
+        st_quad(st + 2 * a.plane + o, ld_quad(QS + s));
+        if (TRACK) st_quad(a.hmax_field + (size_t)m * a.plane + o, ld_quad(HM + s));
     }
     if (band == 0 && tid == 0) {
         MemberClock c;

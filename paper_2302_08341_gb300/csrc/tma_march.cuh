@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "march.cuh"
+#include "quad.cuh"
 #include "tma.cuh"
 
 namespace flood {
@@ -80,28 +81,6 @@ __device__ __forceinline__ TmaSmem tma_march_smem(unsigned char* smem_raw, int w
     m.tab = reinterpret_cast<float4*>(base + 128 * ((8 * kTmaNS * warps + 127) / 128)) + 4 * w;
     m.stages = base + tma_head_bytes(warps) + kTmaNS * tma_stage_bytes(track) * w;
     return m;
-}
-
-// Four cells as two pairs.
-struct Quad {
-    float2 a, b;
-};
-__device__ __forceinline__ Quad lds_quad(const float* p)
-{
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    return Quad{make_float2(t.x, t.y), make_float2(t.z, t.w)};
-}
-__device__ __forceinline__ void st_quad(float* p, const Quad& v)
-{
-    *reinterpret_cast<float4*>(p) = make_float4(v.a.x, v.a.y, v.b.x, v.b.y);
-}
-__device__ __forceinline__ float& quad_at(Quad& v, int j)
-{
-    return j == 0 ? v.a.x : j == 1 ? v.a.y : j == 2 ? v.b.x : v.b.y;
-}
-__device__ __forceinline__ const float& quad_at(const Quad& v, int j)
-{
-    return j == 0 ? v.a.x : j == 1 ? v.a.y : j == 2 ? v.b.x : v.b.y;
 }
 
 // state_map: (ld, ny, planes) with the source h, qx, qy at planes
@@ -189,7 +168,7 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         return reinterpret_cast<const float*>(sm.tab + *reinterpret_cast<const uint32_t*>(code))[2];
     };
     auto quad_n = [&](const float* p) -> Quad {  // roughness of four staged cells
-        if (!LC) return lds_quad(p);
+        if (!LC) return ld_quad(p);
         const uint4 q = *reinterpret_cast<const uint4*>(p);
         const float* t = reinterpret_cast<const float*>(sm.tab) + 2;
         return Quad{make_float2(t[4 * q.x], t[4 * q.y]), make_float2(t[4 * q.z], t[4 * q.w])};
@@ -219,12 +198,12 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
     }
     const float* F = row_ptr(sC) + x0;
     Quad nC = quad_n(F + kN);
-    Quad qN{dup2(0.0f), dup2(0.0f)};
+    Quad qN = quad_of(0.0f);
     if (r0 > 0) {
         const float* U = row_ptr(0) + x0;
-        const Quad hU = lds_quad(U), hF = lds_quad(F);
-        qN = south_links(hU, lds_quad(U + kZ), quad_n(U + kN), bounds(hU), hF, lds_quad(F + kZ), nC,
-                         bounds(hF), lds_quad(U + kQy));
+        const Quad hU = ld_quad(U), hF = ld_quad(F);
+        qN = south_links(hU, ld_quad(U + kZ), quad_n(U + kN), bounds(hU), hF, ld_quad(F + kZ), nC,
+                         bounds(hF), ld_quad(U + kQy));
 #pragma unroll
         for (int j = 0; j < 4; ++j)
             if (!full && c + j >= nx) quad_at(qN, j) = 0.0f;
@@ -249,11 +228,11 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         }
         const float* R = row_ptr(sC);
         const float* P = R + x0;
-        const Quad hC = lds_quad(P), zC = lds_quad(P + kZ), uC = bounds(hC);
-        if (!LC) nC = lds_quad(P + kN);
+        const Quad hC = ld_quad(P), zC = ld_quad(P + kZ), uC = bounds(hC);
+        if (!LC) nC = ld_quad(P + kN);
         // east links: cells 0 1 2 3 with 1 2 3 and the next lane's first,
         // straight from the tile
-        const Quad qx = lds_quad(P + kQx);
+        const Quad qx = ld_quad(P + kQx);
         const float hE = P[4], zE = P[kZ + 4], nE = LC ? class_n(P + kN + 4) : P[kN + 4];
         Quad qE, qS, nS;
         qE.a = link2_q<LIM>(hC.a, zC.a, make_float2(hC.a.y, hC.b.x), make_float2(zC.a.y, zC.b.x), qx.a,
@@ -270,9 +249,9 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
                              __fmul_rn(s_half, __fadd_rn(LC ? class_n(R + kN + 3) : R[kN + 3], nC.a.x)), k);
         if (has_s) {
             const float* Q = row_ptr(sN) + x0;
-            const Quad hS = lds_quad(Q);
+            const Quad hS = ld_quad(Q);
             nS = quad_n(Q + kN);
-            qS = south_links(hC, zC, nC, uC, hS, lds_quad(Q + kZ), nS, bounds(hS), lds_quad(P + kQy));
+            qS = south_links(hC, zC, nC, uC, hS, ld_quad(Q + kZ), nS, bounds(hS), ld_quad(P + kQy));
         } else {
             nS = nC;
 #pragma unroll
@@ -367,7 +346,7 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
                 st_quad(pc + 2 * plane, qS);
             }
             if (TRACK_MAX) {
-                const Quad o = lds_quad(R + kTmaHmOff / 4 + 4 * lane);
+                const Quad o = ld_quad(R + kTmaHmOff / 4 + 4 * lane);
                 *reinterpret_cast<float4*>(ph) = make_float4(fmaxf(o.a.x, hN.a.x), fmaxf(o.a.y, hN.a.y),
                                                              fmaxf(o.b.x, hN.b.x), fmaxf(o.b.y, hN.b.y));
             }
