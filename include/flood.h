@@ -204,8 +204,10 @@ typedef struct {
  * is differentiated with the step lengths held at the recorded schedule and
  * the derivative of the branch taken at every kink (Eq. 3's max, limiter,
  * wet/dry test, outflow clip, negative-depth clamp).  Memory: a checkpoint
- * every ckpt_every steps (0: about sqrt(steps)) plus ckpt_every + 1 replayed
- * states, each 12 bytes per cell per member.
+ * every ckpt_every steps plus ckpt_every + 1 replayed states, each 12 bytes per
+ * cell per member; ckpt_every = 0: every state of the window where they take at
+ * most a third of the free device memory (nothing is then replayed), else a
+ * checkpoint about every sqrt(steps).  Results do not depend on it.
  *   grad_n      [ny][nx] FP32  sum_i dL_i/dn_base (or NULL)
  *   grad_rain   [N] FP64       dL_i/d(rain multiplier of i) (or NULL)
  *   grad_scale  [N] FP64       dL_i/d(Manning scale of i) (or NULL)

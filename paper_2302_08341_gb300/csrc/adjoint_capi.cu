@@ -45,6 +45,23 @@ int reverse_rows(int ny, int nx, int M, int n_sm)
     return rh;
 }
 
+// Whether to keep every state of a window (`floats` of them in all) instead of
+// checkpoints to recompute from: the recomputation moves 26 bytes per
+// member-cell-step and takes a quarter of the gradient's time, the slots cost
+// nothing extra to write (24 members of 1000 x 1000, 60 steps, 20 GB: 28.9 ms
+// recomputing, 21.9 ms keeping).  Up to a third of the memory that is free
+// beside the slots already held.
+bool keep_states(const flood_grid* g, size_t floats)
+{
+    if (floats <= g->ckpt_floats) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return floats * sizeof(float) <= (free_b + g->ckpt_floats * sizeof(float)) / 3;
+}
+
 // Put the state saved in ckpt slot 0 back into each member's current buffer
 // and restore the saved clocks and volume counters (a forward that overflowed
 // the step log is redone).
@@ -115,20 +132,38 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     std::vector<int32_t> samp_step((size_t)ns * M);
     size_t have_ckpt = 0, have_log = 0, have_sy = 0;
     int K = 0;
+    bool keep = false;  // every state of the window is kept: nothing is recomputed
+    size_t n_ckpt = 0;
     cudaEvent_t e0, e1, e2;
     CK(g, cudaEventCreate(&e0));
     CK(g, cudaEventCreate(&e1));
     CK(g, cudaEventCreate(&e2));
     for (int attempt = 0;; ++attempt) {
-        K = ckpt_every > 0 ? ckpt_every : std::max(1, (int)std::lround(std::sqrt((double)cap)));
-        const size_t n_ckpt = (size_t)cap / K + 1;
+        keep = ckpt_every == 0 && keep_states(g, (size_t)(cap + 1) * M * ms);
+        for (;;) {
+            K = ckpt_every > 0 ? ckpt_every : keep ? 1 : std::max(1, (int)std::lround(std::sqrt((double)cap)));
+            n_ckpt = (size_t)cap / K + 1;
+            if (n_ckpt * M * ms <= g->ckpt_floats) break;
+            have_ckpt = 0;
+            g->ckpt_floats = 0;
+            rc = grow(g, &g->ckpt, have_ckpt, n_ckpt * M * ms);
+            if (!rc) {
+                g->ckpt_floats = n_ckpt * M * ms;
+                break;
+            }
+            if (!keep || rc != FLOOD_ERR_OOM) return rc;
+            cudaGetLastError();
+            keep = false;  // another allocation took the room meanwhile
+        }
+        // where every state is kept the TMA step goes from slot to slot (the
+        // resident steps write each state to its slot as a checkpoint)
+        g->slots = keep && g->engine == 1 && g->maps_ok && g->wait_budget < 0 && !flood::steps_resident(g);
+        if (g->slots)
+            g->slots = flood::encode_map_3d(&g->ckpt_map, g->ckpt, g->ld, g->ny, (uint64_t)n_ckpt * M * 3,
+                                            sizeof(float) * g->ld, sizeof(float) * g->plane,
+                                            flood::tma_box_cols(), 1, 3) == 0;
         have_log = 0;
         if ((rc = grow(g, &g->log, have_log, (size_t)M * cap))) return rc;
-        if (n_ckpt * M * ms > g->ckpt_floats) {
-            have_ckpt = 0;
-            if ((rc = grow(g, &g->ckpt, have_ckpt, n_ckpt * M * ms))) return rc;
-            g->ckpt_floats = n_ckpt * M * ms;
-        }
         have_sy = 0;
         if ((rc = grow(g, &g->samp_y, have_sy, (size_t)ns * M * G))) return rc;
         g->log_cap = cap;
@@ -149,7 +184,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         for (int sidx = 1; sidx <= ns; ++sidx) {
             rc = flood_step(g, 0, t0 + sidx * L->sample_dt, stream);
             if (rc) {
-                g->logging = false;
+                g->logging = g->slots = false;
                 return rc;
             }
             // the cells live in samp_cells (device) for both gauge sampling and seeding
@@ -159,12 +194,16 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
                 CK(g, cudaMemcpyAsync(g->samp_cells, cells.data(), sizeof(int32_t) * G,
                                       cudaMemcpyHostToDevice, s));
             }
-            flood::launch_gauge(g->state, g->ms + (g->k % 3) * M, g->samp_cells, G, M, g->ld, g->nx,
-                                g->plane, g->samp_y + (size_t)(sidx - 1) * M * G, s);
+            if (g->slots)
+                flood::launch_gauge_slots(g->ckpt, g->ms + (g->k % 3) * M, cap, g->samp_cells, G, M, g->ld, g->nx,
+                                          g->plane, g->samp_y + (size_t)(sidx - 1) * M * G, s);
+            else
+                flood::launch_gauge(g->state, g->ms + (g->k % 3) * M, g->samp_cells, G, M, g->ld, g->nx,
+                                    g->plane, g->samp_y + (size_t)(sidx - 1) * M * G, s);
             g->launches++;
             std::vector<MemberClock> cc;
             if ((rc = flood::read_clocks(g, cc, s))) {
-                g->logging = false;
+                g->logging = g->slots = false;
                 return rc;
             }
             for (int m = 0; m < M; ++m) {
@@ -173,8 +212,16 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
                 kmax = std::max<int64_t>(kmax, cc[m].steps);
             }
         }
+        if (g->slots && kmax <= cap) {  // the window's end is the ensemble's state
+            std::vector<MemberClock> cc;
+            if ((rc = flood::read_clocks(g, cc, s))) return rc;
+            for (int m = 0; m < M; ++m)
+                CK(g, cudaMemcpyAsync(g->state + (size_t)(cc[m].cur * M + m) * ms,
+                                      g->ckpt + ((size_t)K_m[m] * M + m) * ms, sizeof(float) * ms,
+                                      cudaMemcpyDeviceToDevice, s));
+        }
         CK(g, cudaEventRecord(e1, s));
-        g->logging = false;
+        g->logging = g->slots = false;
         if (kmax <= cap) break;
         if (attempt >= 4) return flood::fail(g, FLOOD_ERR_STATE, "step log could not hold the window");
         if ((rc = restore_start(g, c0, rain0, vacc0, s))) return rc;
@@ -197,10 +244,15 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
 
     // reverse sweep buffers
     size_t have = 0;
-    if ((size_t)(K + 1) * M * ms > g->seg_floats) {
+    // the states the reverse pass reads: a segment recomputed from its
+    // checkpoint, or the whole window's slots
+    if (keep) K = cap;
+    const size_t n_slots = keep ? n_ckpt : (size_t)K + 1;
+    if (!keep && (size_t)(K + 1) * M * ms > g->seg_floats) {
         if ((rc = grow(g, &g->seg, have, (size_t)(K + 1) * M * ms))) return rc;
         g->seg_floats = (size_t)(K + 1) * M * ms;
     }
+    float* const seg = keep ? g->ckpt : g->seg;
     have = 0;
     if ((rc = grow(g, &g->lam, have, 2 * (size_t)M * ms))) return rc;
     const int rrows = g->launch_fixed ? g->rows_per_strip : reverse_rows(g->ny, g->nx, M, g->n_sm);
@@ -240,9 +292,9 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         const int bc = flood::adjoint_tma_box_cols();
         const uint64_t s1 = sizeof(float) * g->ld, s2 = sizeof(float) * g->plane;
         use_tma =
-            flood::encode_map_3d(&tma.seg_map, g->seg, g->ld, g->ny, (uint64_t)(K + 1) * M * 3, s1,
+            flood::encode_map_3d(&tma.seg_map, seg, g->ld, g->ny, (uint64_t)n_slots * M * 3, s1,
                                  s2, bc, 1, 3) == 0 &&
-            flood::encode_map_3d(&tma.seg1_map, g->seg, g->ld, g->ny, (uint64_t)(K + 1) * M * 3, s1,
+            flood::encode_map_3d(&tma.seg1_map, seg, g->ld, g->ny, (uint64_t)n_slots * M * 3, s1,
                                  s2, bc, 1, 1) == 0 &&
             flood::encode_map_3d(&tma.lam_map, g->lam, g->ld, g->ny, (uint64_t)2 * M * 3, s1, s2, bc,
                                  1, 3) == 0 &&
@@ -274,13 +326,14 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         }
         if (len <= 0) continue;
         CK(g, cudaMemcpyAsync(g->seg_end, seg_end.data(), sizeof(int) * M, cudaMemcpyHostToDevice, s));
-        CK(g, cudaMemcpyAsync(g->seg, g->ckpt + (size_t)cs * M * ms, sizeof(float) * M * ms,
-                              cudaMemcpyDeviceToDevice, s));
+        if (!keep)
+            CK(g, cudaMemcpyAsync(g->seg, g->ckpt + (size_t)cs * M * ms, sizeof(float) * M * ms,
+                                  cudaMemcpyDeviceToDevice, s));
         flood::StepArgs a = flood::step_args(g, -1.0);
         a.log = g->log;
         a.dt_log_cap = g->log_cap;
         a.ckpt = nullptr;
-        a.seg = g->seg;
+        a.seg = seg;
         a.seg_end = g->seg_end;
         a.seg_first = first;
         flood::TmaArgs rt;
@@ -288,7 +341,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             rt.state_map = tma.seg_map;
             rt.static_map = g->lc_on ? g->static_map_lc : g->static_map;
         }
-        for (int i = 0; i < len; ++i) {
+        for (int i = 0; i < len && !keep; ++i) {
             a.replay_i = i;
             if (use_tma) {
                 rt.a = a;
@@ -299,7 +352,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             g->launches++;
         }
         flood::AdjArgs b{};
-        b.seg = g->seg;
+        b.seg = seg;
         b.lam = g->lam;
         b.gn = grad_n ? g->gnm : nullptr;
         b.gpart = g->gpart;

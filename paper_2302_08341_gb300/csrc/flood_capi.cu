@@ -115,6 +115,7 @@ StepArgs step_args(const flood_grid* g, double t_end)
     a.dt_log_cap = g->log_cap;
     a.ckpt = g->logging ? g->ckpt : nullptr;
     a.ckpt_every = g->ckpt_every > 0 ? g->ckpt_every : 1;
+    a.slots = g->logging && g->slots ? 1 : 0;
     a.err = g->err;
     a.wait_budget = g->wait_budget < 0 ? flood::kTmaWaitBudgetDefault : g->wait_budget;
     a.hmax_field = g->track_max ? g->hmax_field : nullptr;
@@ -201,7 +202,7 @@ static int launch_one(flood_grid* g, double t_end, cudaStream_t s)
     }
     if (g->engine == 1 && g->maps_ok) {
         flood::TmaArgs t;
-        t.state_map = g->state_map;
+        t.state_map = a.slots ? g->ckpt_map : g->state_map;
         t.static_map = a.lc_on ? g->static_map_lc : g->static_map;
         if (a.hmax_field) t.hm_map = g->hm_map;
         if (skips_tiles(g, a)) {
@@ -238,6 +239,12 @@ static bool resident_now(const flood_grid* g, ResidentShape* sh)
     if (g->engine != 1 || !g->maps_ok || g->profile || g->launch_fixed || g->wait_budget >= 0) return false;
     *sh = resident_shape(g->ny, g->nx, g->M, g->n_sm, g->smem_max, g->track_max, g->lc_on);
     return sh->bands > 0;
+}
+
+bool steps_resident(const flood_grid* g)
+{
+    ResidentShape sh;
+    return resident_now(g, &sh);
 }
 
 // The buffers of steps in that shape (allocates: not while capturing).

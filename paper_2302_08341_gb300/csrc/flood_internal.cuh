@@ -42,6 +42,7 @@ struct StepArgs {
     struct MemberPlan* log;     // [M][dt_log_cap] plans of the steps taken (or null)
     float* ckpt;                // [n_ckpt][M][3][plane] checkpoint states (or null)
     int ckpt_every;             // a checkpoint after every ckpt_every steps of a member
+    int slots;                  // every state is kept: a step reads checkpoint slot i, writes slot i + 1
     // replay of a checkpointed segment (adjoint recomputation): slot i of
     // seg holds the state after step seg_first + i; this launch recomputes
     // step seg_first + replay_i of every member with seg_first + replay_i <
@@ -106,7 +107,8 @@ struct MemberPlan {
     float gdt_dx, gdt, dx_4dt, dt_dx;
     int active;               // 0: the member does not step
     int cur;                  // buffer holding the member's state before the step
-    int ckpt;                 // checkpoint slot that also receives the result, or -1
+    int ckpt;                 // checkpoint slot that also receives the result, or -1 (slots: the
+                              // slot the step reads)
     float q_in;               // inflow flux per unit width of this step (m^2/s), 0 without
 };
 

@@ -90,6 +90,8 @@ struct flood_grid {
     float* ckpt = nullptr;        // [n_ckpt][M][3][plane]
     size_t ckpt_floats = 0;
     int ckpt_every = 0;
+    bool slots = false;           // the logged forward steps from checkpoint slot to slot
+    CUtensorMap ckpt_map;         // the checkpoint slots, for such steps
     float* seg = nullptr;         // [slots][M][3][plane]
     size_t seg_floats = 0;
     float* lam = nullptr;         // [2][M][3][plane]
@@ -161,6 +163,8 @@ int dalloc(flood_grid* g, T** p, size_t count)
 StepArgs step_args(const flood_grid* g, double t_end);
 int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s);
 int read_clocks(flood_grid* g, std::vector<MemberClock>& out, cudaStream_t s);
+// Whether the next steps run on the chip (step_resident.cu).
+bool steps_resident(const flood_grid* g);
 int check_err(flood_grid* g);
 void collect_profile(flood_grid* g);
 void launch_copy_planes(float* field, const int32_t* n_copy, const int32_t* dsts, const int32_t* srcs,

@@ -25,6 +25,19 @@ __global__ void gauge_kernel(const float* __restrict__ state, const MemberClock*
     y[t] = h[(size_t)r * ld + c];
 }
 
+// The same from checkpoint slots: each member's state after its steps so far.
+__global__ void gauge_slots_kernel(const float* __restrict__ slots, const MemberClock* __restrict__ ms, int last,
+                                   const int32_t* __restrict__ cells, int G, int M, int ld, int nx, size_t plane,
+                                   float* __restrict__ y)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= M * G) return;
+    const int m = t / G, k = t % G;
+    const int cell = cells[k];
+    const int64_t i = ms[m].steps < last ? ms[m].steps : last;
+    y[t] = slots[((size_t)i * M + m) * 3 * plane + (size_t)(cell / nx) * ld + cell % nx];
+}
+
 // DA steps (II)-(IV) and the bookkeeping of step (V), one block.
 //
 // Bound by latency: a few hundred FP64 operations per member on a GPU whose
@@ -294,6 +307,12 @@ void launch_gauge(const float* state, const MemberClock* ms, const int32_t* cell
 {
     const int n = M * G;
     gauge_kernel<<<(n + 127) / 128, 128, 0, s>>>(state, ms, cells, G, M, ld, nx, plane, y);
+}
+
+void launch_gauge_slots(const float* slots, const MemberClock* ms, int last, const int32_t* cells, int G, int M,
+                        int ld, int nx, size_t plane, float* y, cudaStream_t s)
+{
+    gauge_slots_kernel<<<(M * G + 127) / 128, 128, 0, s>>>(slots, ms, last, cells, G, M, ld, nx, plane, y);
 }
 
 cudaError_t launch_pf(const PfArgs& a, cudaStream_t s)

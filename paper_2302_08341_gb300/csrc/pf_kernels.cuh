@@ -32,6 +32,8 @@ struct PfArgs {
 
 void launch_gauge(const float* state, const MemberClock* ms, const int32_t* cells, int G, int M,
                   int ld, int nx, size_t plane, float* y, cudaStream_t s);
+void launch_gauge_slots(const float* slots, const MemberClock* ms, int last, const int32_t* cells, int G, int M,
+                        int ld, int nx, size_t plane, float* y, cudaStream_t s);
 cudaError_t launch_pf(const PfArgs& a, cudaStream_t s);
 void launch_copy(float* state, const MemberClock* ms, const int32_t* n_copy, const int32_t* dsts,
                  const int32_t* srcs, int M, size_t plane, int n_sm, cudaStream_t s);

@@ -64,7 +64,9 @@ __global__ void plan_kernel(const StepArgs a)
     a.ms_out[m].steps = in.steps + 1;
     a.ms_out[m].cur = 1 - in.cur;  // hmax_bits: atomicMax by the step kernel (slot was cleared)
     a.rain_acc[m] += (double)sp.dr * a.cell_area * a.ncell;
-    if (a.ckpt && (in.steps + 1) % a.ckpt_every == 0 && in.steps + 1 <= a.dt_log_cap)
+    if (a.slots)  // (steps past the log's end stay in its last slots: the window is run again)
+        p.ckpt = (int)(in.steps < a.dt_log_cap ? in.steps : a.dt_log_cap - 1);
+    else if (a.ckpt && (in.steps + 1) % a.ckpt_every == 0 && in.steps + 1 <= a.dt_log_cap)
         p.ckpt = (int)((in.steps + 1) / a.ckpt_every);
     if (a.log && in.steps < a.dt_log_cap) a.log[(size_t)m * a.dt_log_cap + in.steps] = p;
     a.plan[m] = p;

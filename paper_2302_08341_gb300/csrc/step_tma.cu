@@ -46,8 +46,12 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
     // each warp is its own member here: the warp at the first span and strip owns its clock
     const MemberPlan pl = a.plan[m];
     if (!pl.active) return;
-    float* __restrict__ dst = a.state + (size_t)((1 - pl.cur) * a.M + m) * mstride;
-    float* ck = (CK && pl.ckpt >= 0) ? a.ckpt + ((size_t)pl.ckpt * a.M + m) * mstride : nullptr;
+    // the other state buffer, and a checkpoint slot every so many steps; or,
+    // where every state is kept, from one slot to the next
+    const bool slots = CK && a.slots;
+    float* __restrict__ dst = slots ? a.ckpt + ((size_t)(pl.ckpt + 1) * a.M + m) * mstride
+                                    : a.state + (size_t)((1 - pl.cur) * a.M + m) * mstride;
+    float* ck = (CK && !slots && pl.ckpt >= 0) ? a.ckpt + ((size_t)pl.ckpt * a.M + m) * mstride : nullptr;
 
     FaceK k;
     k.gdt_dx = pl.gdt_dx;
@@ -66,7 +70,7 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
     float* hm = TRACK_MAX ? a.hmax_field + (size_t)m * a.plane : nullptr;
     LandK lk;
     if (LC) lk = land_k(a, m, pl.dr, pl.dt, lane);
-    if (!tma_march<TRACK_MAX, LC, LIM, HOOK>(&t.state_map, &t.static_map, (pl.cur * a.M + m) * 3, sm,
+    if (!tma_march<TRACK_MAX, LC, LIM, HOOK>(&t.state_map, &t.static_map, ((slots ? pl.ckpt : pl.cur) * a.M + m) * 3, sm,
                                   dst, ck, hm, a.err, a.plane, a.ny, a.nx, a.ld, c0, r0,
                                   r1, lane, k, pl.dt_dx, a.scale[m], pl.dr, a.east_out, a.south_out,
                                   mo, &lk, a.wait_budget, &t.hm_map, m))

@@ -249,3 +249,40 @@ def test_adjoint_at_the_calibration_window_size_follows_the_fp64_adjoint(capi):
           f"FD rain {abs(fd_rain - out['grad_rain'][0]) / abs(fd_rain):.2e}, "
           f"FD cells median {np.median(errs):.2e} worst {errs.max():.2e}")
     assert np.median(errs) <= 1e-3 and errs.max() <= 1e-2, (np.median(errs), errs.max())
+
+
+@pytest.mark.parametrize("ny,nx,M,shape,land,h0", [(40, 56, 1, None, False, 0.2), (37, 300, 5, None, True, 0.2),
+                                                   (33, 131, 4, (8, 4), False, 0.2), (50, 140, 3, (16, 1), True, 0.2),
+                                                   (40, 60, 2, (8, 1), False, 3.0), (40, 60, 2, None, False, 3.0)])
+def test_kept_states_give_the_recomputed_gradients(capi, ny, nx, M, shape, land, h0):
+    """ckpt_every = 0 keeps every state of a small window (steps from slot to
+    slot with a fixed launch shape, steps on the chip without one; deep water
+    outgrows the first step log, so the window is run twice); explicit
+    checkpoints recompute them.  The same gradients, losses and ensemble, bit
+    for bit."""
+    rng = np.random.default_rng(ny * nx)
+    terr = synth.make_terrain(ny, nx, seed=ny, building_frac=0.0)
+    hy = synth.hyetograph_triangular(60.0, 1200.0, 3600.0)
+    rm, sc = synth.ensemble_prior(5, M)
+    start = (h0 * rng.uniform(0.5, 1.0, (M, ny, nx))).astype(np.float32)
+    cells = rng.choice(ny * nx, 4, replace=False).astype(np.int32)
+    d = rng.uniform(0.5 * h0, h0, (3, 4))
+    res = []
+    for every in (0, 5):
+        with capi.Grid(terr.z, terr.n) as g:
+            if land:
+                g.set_land_cover(synth.land_cover(terr, seed=3, pond_side=(4, 9)), synth.LAND_CLASSES)
+            g.ensemble_init(M, rm, np.ones(M, np.float32) if land else sc, hy, h0=start)
+            if land:
+                g.set_land_params(*synth.land_prior(3, M))
+            if shape:
+                g.set_launch(*shape)
+            out = g.adjoint(cells, d, 10.0, ckpt_every=every)
+            got = [out[k] for k in ("loss", "grad_n", "grad_rain", "grad_scale", "grad_h0")]
+            got += list(g.adjoint_land_grad()) if land else []
+            g.step(3)                       # the ensemble goes on from the window's end
+            mem = g.members()
+            got += [mem["t"], mem["steps"], mem["hmax"]] + [x for m in range(M) for x in g.get_state(m)]
+        res.append(got)
+    for a, b in zip(*res):
+        np.testing.assert_array_equal(a, b)
