@@ -23,12 +23,16 @@ namespace {
 
 cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
+// Room for `count` values, kept from one adjoint to the next (its buffers were
+// freed and allocated again by every call).
 template <class T>
 int grow(flood_grid* g, T** p, size_t& have, size_t count)
 {
     if (*p && have >= count) return FLOOD_OK;
-    have = count;
-    return flood::dalloc(g, p, count);
+    have = 0;
+    const int rc = flood::dalloc(g, p, count);
+    if (!rc) have = count;
+    return rc;
 }
 
 // The reverse stencil's automatic strip height.  The scalar gradients are FP64
@@ -130,7 +134,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     for (int m = 0; m < M; ++m) steps0[m] = c0[m].steps;
     std::vector<int> K_m(M);
     std::vector<int32_t> samp_step((size_t)ns * M);
-    size_t have_ckpt = 0, have_log = 0, have_sy = 0;
+    flood_grid::AdjointRoom& room = g->adj_room;
     int K = 0;
     bool keep = false;  // every state of the window is kept: nothing is recomputed
     size_t n_ckpt = 0;
@@ -144,13 +148,9 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             K = ckpt_every > 0 ? ckpt_every : keep ? 1 : std::max(1, (int)std::lround(std::sqrt((double)cap)));
             n_ckpt = (size_t)cap / K + 1;
             if (n_ckpt * M * ms <= g->ckpt_floats) break;
-            have_ckpt = 0;
+            rc = grow(g, &g->ckpt, g->ckpt_floats, n_ckpt * M * ms);
+            if (!rc) break;
             g->ckpt_floats = 0;
-            rc = grow(g, &g->ckpt, have_ckpt, n_ckpt * M * ms);
-            if (!rc) {
-                g->ckpt_floats = n_ckpt * M * ms;
-                break;
-            }
             if (!keep || rc != FLOOD_ERR_OOM) return rc;
             cudaGetLastError();
             keep = false;  // another allocation took the room meanwhile
@@ -162,10 +162,8 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             g->slots = flood::encode_map_3d(&g->ckpt_map, g->ckpt, g->ld, g->ny, (uint64_t)n_ckpt * M * 3,
                                             sizeof(float) * g->ld, sizeof(float) * g->plane,
                                             flood::tma_box_cols(), 1, 3) == 0;
-        have_log = 0;
-        if ((rc = grow(g, &g->log, have_log, (size_t)M * cap))) return rc;
-        have_sy = 0;
-        if ((rc = grow(g, &g->samp_y, have_sy, (size_t)ns * M * G))) return rc;
+        if ((rc = grow(g, &g->log, room.log, (size_t)M * cap))) return rc;
+        if ((rc = grow(g, &g->samp_y, room.samp_y, (size_t)ns * M * G))) return rc;
         g->log_cap = cap;
         g->ckpt_every = K;
         // checkpoint 0: the starting state; clocks count steps from 0
@@ -189,8 +187,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             }
             // the cells live in samp_cells (device) for both gauge sampling and seeding
             if (sidx == 1) {
-                size_t hc = 0;
-                if ((rc = grow(g, &g->samp_cells, hc, G))) return rc;
+                if ((rc = grow(g, &g->samp_cells, room.samp_cells, G))) return rc;
                 CK(g, cudaMemcpyAsync(g->samp_cells, cells.data(), sizeof(int32_t) * G,
                                       cudaMemcpyHostToDevice, s));
             }
@@ -243,40 +240,30 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         }
 
     // reverse sweep buffers
-    size_t have = 0;
     // the states the reverse pass reads: a segment recomputed from its
     // checkpoint, or the whole window's slots
     if (keep) K = cap;
     const size_t n_slots = keep ? n_ckpt : (size_t)K + 1;
     if (!keep && (size_t)(K + 1) * M * ms > g->seg_floats) {
-        if ((rc = grow(g, &g->seg, have, (size_t)(K + 1) * M * ms))) return rc;
-        g->seg_floats = (size_t)(K + 1) * M * ms;
+        if ((rc = grow(g, &g->seg, g->seg_floats, (size_t)(K + 1) * M * ms))) return rc;
     }
     float* const seg = keep ? g->ckpt : g->seg;
-    have = 0;
-    if ((rc = grow(g, &g->lam, have, 2 * (size_t)M * ms))) return rc;
+    if ((rc = grow(g, &g->lam, room.lam, 2 * (size_t)M * ms))) return rc;
     const int rrows = g->launch_fixed ? g->rows_per_strip : reverse_rows(g->ny, g->nx, M, g->n_sm);
     const int nslot = flood::step_nslot(g->ny, g->nx, rrows);
-    have = 0;
-    if ((rc = grow(g, &g->gpart, have, (size_t)M * nslot * 2))) return rc;
-    have = 0;
-    if ((rc = grow(g, &g->seg_end, have, M))) return rc;
-    have = 0;
-    if ((rc = grow(g, &g->samp_step, have, (size_t)ns * M))) return rc;
-    have = 0;
-    if ((rc = grow(g, &g->samp_d, have, (size_t)ns * G))) return rc;
+    if ((rc = grow(g, &g->gpart, room.gpart, (size_t)M * nslot * 2))) return rc;
+    if ((rc = grow(g, &g->seg_end, room.seg_end, M))) return rc;
+    if ((rc = grow(g, &g->samp_step, room.samp_step, (size_t)ns * M))) return rc;
+    if ((rc = grow(g, &g->samp_d, room.samp_d, (size_t)ns * G))) return rc;
     if (grad_n) {
-        have = 0;
-        if ((rc = grow(g, &g->gnm, have, (size_t)M * g->plane))) return rc;
-        have = 0;
-        if ((rc = grow(g, &g->gn_out, have, (size_t)g->ny * g->nx))) return rc;
+        if ((rc = grow(g, &g->gnm, room.gnm, (size_t)M * g->plane))) return rc;
+        if ((rc = grow(g, &g->gn_out, room.gn_out, (size_t)g->ny * g->nx))) return rc;
         CK(g, cudaMemsetAsync(g->gnm, 0, sizeof(float) * M * g->plane, s));
     }
     CK(g, cudaMemsetAsync(g->lam, 0, sizeof(float) * 2 * M * ms, s));
     CK(g, cudaMemsetAsync(g->gpart, 0, sizeof(double) * M * nslot * 2, s));
     if (g->lc_on) {
-        have = 0;
-        if ((rc = grow(g, &g->gdpart, have, (size_t)M * nslot))) return rc;
+        if ((rc = grow(g, &g->gdpart, room.gdpart, (size_t)M * nslot))) return rc;
         CK(g, cudaMemsetAsync(g->gdpart, 0, sizeof(double) * M * nslot, s));
     }
     CK(g, cudaMemcpyAsync(g->samp_step, samp_step.data(), sizeof(int32_t) * ns * M,

@@ -80,6 +80,7 @@ void free_ensemble(flood_grid* g)
     g->lam = nullptr; g->gnm = nullptr; g->gn_out = nullptr; g->gpart = nullptr;
     g->seg_end = nullptr; g->samp_step = nullptr; g->samp_y = nullptr; g->samp_d = nullptr;
     g->samp_cells = nullptr; g->log_cap = 0; g->ckpt_floats = 0; g->seg_floats = 0;
+    g->adj_room = flood_grid::AdjointRoom{};
     g->logging = false;
     g->state = nullptr; g->rain_mult = nullptr; g->scale = nullptr; g->hyeto = nullptr;
     g->w = nullptr; g->w_post = nullptr; g->ms = nullptr; g->vacc = nullptr;

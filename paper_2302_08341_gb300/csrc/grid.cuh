@@ -103,6 +103,10 @@ struct flood_grid {
     float* samp_y = nullptr;      // [ns][M][G]
     double* samp_d = nullptr;     // [ns][G]
     int32_t* samp_cells = nullptr;
+    struct AdjointRoom {          // values each of the adjoint's buffers holds
+        size_t log = 0, samp_y = 0, samp_cells = 0, lam = 0, gpart = 0, seg_end = 0, samp_step = 0,
+               samp_d = 0, gnm = 0, gn_out = 0, gdpart = 0;
+    } adj_room;
     double adj_fwd_ms = 0.0, adj_rev_ms = 0.0;
     // land cover (land_cover.cu; Section 4.1)
     bool lc_on = false;
