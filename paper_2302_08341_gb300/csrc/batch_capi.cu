@@ -11,7 +11,7 @@
 #include "../../include/flood.h"
 #include "batch.cuh"
 #include "trace.cuh"
-#include "pf_kernels.cuh"
+#include "readout.cuh"
 #include "tma.cuh"
 
 using flood::MemberClock;
@@ -53,8 +53,8 @@ struct flood_batch {
     double* vacc = nullptr;           // [nslot][2]
     double* rain_acc = nullptr;       // [S]
     double* storage = nullptr;        // [S]
-    double* part = nullptr;           // storage partials
-    int part_cap = 0;
+    double* part = nullptr;           // storage partials, [S][ceil(ny_max / 16)]
+    int ny_max = 0;
     int* err = nullptr;
     double* t_stop = nullptr;         // device scalar
     flood::MemberPlan* plan = nullptr; // [S]
@@ -255,11 +255,11 @@ int set_entries(flood_batch* b, const std::vector<int>& counts)
     for (float* p : b->state)
         if (p) cudaFree(p);
     b->state.clear();
-    void* old[] = {b->d_desc, b->ms, b->rain_acc, b->storage, b->plan, b->d_maps};
+    void* old[] = {b->d_desc, b->ms, b->rain_acc, b->storage, b->part, b->plan, b->d_maps};
     for (void* p : old)
         if (p) cudaFree(p);
     b->d_desc = nullptr; b->ms = nullptr; b->rain_acc = nullptr; b->storage = nullptr;
-    b->plan = nullptr; b->d_maps = nullptr;
+    b->part = nullptr; b->plan = nullptr; b->d_maps = nullptr;
     drop_graph(b);
     int S = 0;
     b->first.assign(b->n_scen + 1, 0);
@@ -308,6 +308,8 @@ int set_entries(flood_batch* b, const std::vector<int>& counts)
     BCK(b, cudaMalloc(&b->rain_acc, sizeof(double) * S));
     BCK(b, cudaMemset(b->rain_acc, 0, sizeof(double) * S));
     BCK(b, cudaMalloc(&b->storage, sizeof(double) * S));
+    b->ny_max = *std::max_element(b->sny.begin(), b->sny.end());
+    BCK(b, cudaMalloc(&b->part, sizeof(double) * S * (size_t)((b->ny_max + 15) / 16)));
     BCK(b, cudaMalloc(&b->plan, sizeof(flood::MemberPlan) * S));
     BCK(b, cudaMalloc(&b->d_desc, sizeof(flood::ScenDesc) * S));
     BCK(b, cudaMemcpy(b->d_desc, b->desc.data(), sizeof(flood::ScenDesc) * S, cudaMemcpyHostToDevice));
@@ -416,9 +418,6 @@ int flood_batch_create(flood_batch** out, int n, const int32_t* ny, const int32_
     }
     cudaError_t e = cudaMalloc(&b->err, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->t_stop, sizeof(double));
-    int maxny = *std::max_element(b->sny.begin(), b->sny.end());
-    b->part_cap = (maxny + 15) / 16;
-    if (e == cudaSuccess) e = cudaMalloc(&b->part, sizeof(double) * b->part_cap);
     if (e != cudaSuccess) {
         int rc = bad(e);
         flood_batch_destroy(b);
@@ -673,12 +672,19 @@ int flood_batch_get_member_state(flood_batch* b, int scen, int member, float* h,
         return bfail(b, FLOOD_ERR_ARG, "member out of range");
     const int i = b->first[scen] + member;
     cudaStream_t s = S_(stream);
-    MemberClock c;
-    BCK(b, cudaMemcpyAsync(&c, b->ms + (b->k % 3) * b->S + i, sizeof(c), cudaMemcpyDeviceToHost, s));
-    BCK(b, cudaStreamSynchronize(s));
+    MemberClock* clk = b->ms + (b->k % 3) * b->S + i;
     const flood::ScenDesc& d = b->desc[i];
-    const float* base = d.state + (size_t)c.cur * 3 * d.plane;
     float* outs[3] = {h, qx, qy};
+    if (flood::read_by_kernel(h, qx, qy, (size_t)d.ny * d.nx, s)) {
+        flood::launch_read_state(d.state, 3 * d.plane, clk, d.ny, d.nx, d.ld, d.plane, h, qx, qy, b->n_sm, s);
+        BCK(b, cudaGetLastError());
+        BCK(b, cudaStreamSynchronize(s));
+        return FLOOD_OK;
+    }
+    MemberClock c;
+    BCK(b, cudaMemcpyAsync(&c, clk, sizeof(c), cudaMemcpyDeviceToHost, s));
+    BCK(b, cudaStreamSynchronize(s));
+    const float* base = d.state + (size_t)c.cur * 3 * d.plane;
     for (int k = 0; k < 3; ++k)
         if (outs[k])
             BCK(b, cudaMemcpy2DAsync(outs[k], sizeof(float) * d.nx, base + k * d.plane,
@@ -720,13 +726,8 @@ int flood_batch_members(flood_batch* b, double* t, int64_t* steps, double* stora
         }
     }
     if (storage) {
-        for (int i = 0; i < b->S; ++i) {
-            const flood::ScenDesc& d = b->desc[i];
-            if (flood::launch_storage(d.state, b->ms + (b->k % 3) * b->S + i, 1, d.ny, d.nx, d.ld,
-                                      d.plane, b->p.dx * b->p.dx, b->part, b->part_cap,
-                                      b->storage + i, 0))
-                return bfail(b, FLOOD_ERR_STATE, "storage partial buffer too small");
-        }
+        flood::launch_batch_storage(b->d_desc, b->ms + (b->k % 3) * b->S, b->S, b->ny_max, b->part,
+                                    b->p.dx * b->p.dx, b->storage, 0);
         BCK(b, cudaGetLastError());
         BCK(b, cudaMemcpy(storage, b->storage, sizeof(double) * b->S, cudaMemcpyDeviceToHost));
     }

@@ -11,6 +11,7 @@
 
 #include "grid.cuh"
 #include "pf_kernels.cuh"
+#include "readout.cuh"
 #include "tma.cuh"
 
 using flood::MemberClock;
@@ -62,7 +63,7 @@ void free_ensemble(flood_grid* g)
 {
     dfree(g->state); dfree(g->rain_mult); dfree(g->scale); dfree(g->hyeto); dfree(g->w);
     dfree(g->w_post); dfree(g->ms); dfree(g->vacc); dfree(g->rain_acc); dfree(g->y);
-    dfree(g->y_in); dfree(g->beta); dfree(g->pfi); dfree(g->pf_small); dfree(g->neff);
+    dfree(g->y_in); dfree(g->beta); dfree(g->rows);
     dfree(g->part); dfree(g->storage); dfree(g->cells); dfree(g->d); dfree(g->sigma);
     dfree(g->plan); dfree(g->log); dfree(g->ckpt); dfree(g->seg); dfree(g->lam);
     dfree(g->gnm); dfree(g->gn_out); dfree(g->gpart); dfree(g->seg_end); dfree(g->samp_step);
@@ -87,6 +88,7 @@ void free_ensemble(flood_grid* g)
     g->rain_acc = nullptr; g->y = nullptr; g->y_in = nullptr; g->beta = nullptr;
     g->pfi = nullptr; g->pf_small = nullptr; g->neff = nullptr; g->part = nullptr;
     g->storage = nullptr; g->cells = nullptr; g->d = nullptr; g->sigma = nullptr;
+    g->rows = nullptr;
     g->M = 0; g->G = 0; g->G_cap = 0;
 }
 
@@ -625,20 +627,23 @@ int flood_ensemble_init(flood_grid* g, int M, const float* h0, int h0_per_member
     // (a resident band takes a slot too: at most one per SM)
     g->nslot = std::max(flood::step_nslot(g->ny, g->nx, g->rows_per_strip), g->n_sm);
     g->part_cap = (g->ny + 15) / 16;
+    const size_t pf_doubles = (size_t)M + 1 + 2 + 2 * (size_t)M;  // w_post, neff, the flags, idx to copy_src
     int rc;
     if ((rc = dalloc(g, &g->state, (size_t)2 * M * 3 * g->plane)) ||
         (rc = dalloc(g, &g->rain_mult, M)) || (rc = dalloc(g, &g->scale, M)) ||
         (rc = dalloc(g, &g->hyeto, n_blocks)) || (rc = dalloc(g, &g->w, M)) ||
-        (rc = dalloc(g, &g->w_post, M)) || (rc = dalloc(g, &g->ms, (size_t)3 * M)) ||
+        (rc = dalloc(g, &g->w_post, pf_doubles)) || (rc = dalloc(g, &g->rows, M)) || (rc = dalloc(g, &g->ms, (size_t)3 * M)) ||
         (rc = dalloc(g, &g->vacc, (size_t)M * g->nslot * 2)) || (rc = dalloc(g, &g->rain_acc, M)) ||
         (rc = dalloc(g, &g->inflow_acc, M)) ||
-        (rc = dalloc(g, &g->beta, M)) || (rc = dalloc(g, &g->pfi, (size_t)4 * M)) ||
-        (rc = dalloc(g, &g->pf_small, 4)) || (rc = dalloc(g, &g->neff, 1)) ||
+        (rc = dalloc(g, &g->beta, M)) ||
         (rc = dalloc(g, &g->part, (size_t)M * g->part_cap)) || (rc = dalloc(g, &g->storage, M)) ||
         (rc = dalloc(g, &g->plan, M))) {
         free_ensemble(g);
         return rc;
     }
+    g->neff = g->w_post + M;
+    g->pf_small = reinterpret_cast<int32_t*>(g->neff + 1);
+    g->pfi = g->pf_small + 4;
     CK(g, cudaMemsetAsync(g->state, 0, sizeof(float) * 2 * (size_t)M * 3 * g->plane, s));
     g->maps_ok = flood::encode_map_3d(&g->state_map, g->state, g->ld, g->ny, (uint64_t)2 * M * 3,
                                       sizeof(float) * g->ld, sizeof(float) * g->plane,
@@ -729,7 +734,10 @@ int flood_gauge_sample(flood_grid* g, int G, const int32_t* cell_idx, float* y_o
     if (G < 1 || !cell_idx) return fail(g, FLOOD_ERR_ARG, "need n_gauges >= 1 and cell_idx");
     cudaStream_t s = S(stream);
     std::vector<int32_t> cells(G);
-    CK(g, cudaMemcpy(cells.data(), cell_idx, sizeof(int32_t) * G, cudaMemcpyDefault));
+    if (!flood::capturing(s) && flood::pageable(cell_idx))
+        std::memcpy(cells.data(), cell_idx, sizeof(int32_t) * G);
+    else
+        CK(g, cudaMemcpy(cells.data(), cell_idx, sizeof(int32_t) * G, cudaMemcpyDefault));
     for (int k = 0; k < G; ++k)
         if (cells[k] < 0 || (int64_t)cells[k] >= (int64_t)g->ny * g->nx)
             return fail(g, FLOOD_ERR_ARG, "gauge cell index out of range");
@@ -742,9 +750,14 @@ int flood_gauge_sample(flood_grid* g, int G, const int32_t* cell_idx, float* y_o
         g->G_cap = G;
     }
     g->G = G;
-    CK(g, cudaMemcpyAsync(g->cells, cells.data(), sizeof(int32_t) * G, cudaMemcpyHostToDevice, s));
-    flood::launch_gauge(g->state, g->ms + (g->k % 3) * g->M, g->cells, G, g->M, g->ld, g->nx,
-                        g->plane, g->y, s);
+    if (G <= flood::kGaugeArgs) {
+        flood::GaugeCells list{};
+        std::copy(cells.begin(), cells.end(), list.cell);
+        flood::launch_gauge_args(g->state, g->ms + (g->k % 3) * g->M, list, G, g->M, g->ld, g->nx, g->plane, g->y, s);
+    } else {
+        CK(g, cudaMemcpyAsync(g->cells, cells.data(), sizeof(int32_t) * G, cudaMemcpyHostToDevice, s));
+        flood::launch_gauge(g->state, g->ms + (g->k % 3) * g->M, g->cells, G, g->M, g->ld, g->nx, g->plane, g->y, s);
+    }
     g->launches++;
     CK(g, cudaGetLastError());
     if (y_out)
@@ -821,6 +834,21 @@ int pf_assimilate(flood_grid* g, int G, const float* y, const double* d, const d
         g->launches++;
     }
     CK(g, cudaGetLastError());
+    // the outputs lie in one block (w_post, neff, the flags, idx): one copy
+    // where all go to ordinary host memory
+    auto host = [](const void* p) { return !p || flood::pageable(p); };
+    if (host(weights_out) && host(idx_out) && host(neff_out) && host(resampled_out) && !flood::capturing(s)) {
+        if (!weights_out && !idx_out && !neff_out && !resampled_out) return FLOOD_OK;
+        const size_t small = sizeof(double) * ((size_t)M + 1), idx = small + sizeof(int32_t) * 4;
+        std::vector<char> out(idx + sizeof(int32_t) * M);
+        CK(g, cudaMemcpyAsync(out.data(), g->w_post, out.size(), cudaMemcpyDeviceToHost, s));
+        CK(g, cudaStreamSynchronize(s));
+        if (weights_out) std::memcpy(weights_out, out.data(), sizeof(double) * M);
+        if (neff_out) std::memcpy(neff_out, out.data() + sizeof(double) * M, sizeof(double));
+        if (resampled_out) std::memcpy(resampled_out, out.data() + small + sizeof(int32_t), sizeof(int32_t));
+        if (idx_out) std::memcpy(idx_out, out.data() + idx, sizeof(int32_t) * M);
+        return FLOOD_OK;
+    }
     if (weights_out) CK(g, cudaMemcpyAsync(weights_out, g->w_post, sizeof(double) * M, cudaMemcpyDefault, s));
     if (idx_out) CK(g, cudaMemcpyAsync(idx_out, a.idx, sizeof(int32_t) * M, cudaMemcpyDefault, s));
     if (neff_out) CK(g, cudaMemcpyAsync(neff_out, g->neff, sizeof(double), cudaMemcpyDefault, s));
@@ -857,8 +885,16 @@ int flood_get_state(flood_grid* g, int member, float* h, float* qx, float* qy, v
     if (g->M == 0) return fail(g, FLOOD_ERR_STATE, "flood_ensemble_init has not been called");
     if (member < 0 || member >= g->M) return fail(g, FLOOD_ERR_ARG, "member out of range");
     cudaStream_t s = S(stream);
+    const MemberClock* clk = g->ms + (g->k % 3) * g->M + member;
+    if (flood::read_by_kernel(h, qx, qy, (size_t)g->ny * g->nx, s)) {
+        flood::launch_read_state(g->state + (size_t)member * 3 * g->plane, (size_t)g->M * 3 * g->plane, clk, g->ny,
+                                 g->nx, g->ld, g->plane, h, qx, qy, g->n_sm, s);
+        g->launches++;
+        CK(g, cudaGetLastError());
+        return FLOOD_OK;
+    }
     MemberClock c;
-    CK(g, cudaMemcpyAsync(&c, g->ms + (g->k % 3) * g->M + member, sizeof(c), cudaMemcpyDeviceToHost, s));
+    CK(g, cudaMemcpyAsync(&c, clk, sizeof(c), cudaMemcpyDeviceToHost, s));
     CK(g, cudaStreamSynchronize(s));
     const float* base = g->state + (size_t)(c.cur * g->M + member) * 3 * g->plane;
     float* outs[3] = {h, qx, qy};
@@ -909,12 +945,27 @@ int flood_get_members(flood_grid* g, double* t, int64_t* steps, float* rain_mult
     if (g->M == 0) return fail(g, FLOOD_ERR_STATE, "flood_ensemble_init has not been called");
     const int M = g->M;
     CK(g, cudaDeviceSynchronize());
-    std::vector<MemberClock> c(M);
-    CK(g, cudaMemcpy(c.data(), g->ms + (g->k % 3) * M, sizeof(MemberClock) * M, cudaMemcpyDeviceToHost));
+    flood::launch_pack_members(g->ms + (g->k % 3) * M, g->rain_mult, g->scale, g->w, M, g->rows, 0);
+    g->launches++;
+    CK(g, cudaGetLastError());
+    std::vector<flood::MemberRow> r(M);
+    CK(g, cudaMemcpy(r.data(), g->rows, sizeof(flood::MemberRow) * M, cudaMemcpyDeviceToHost));
+    if (rain_mult && flood::pageable(rain_mult)) {
+        for (int m = 0; m < M; ++m) rain_mult[m] = r[m].rain;
+        rain_mult = nullptr;
+    }
+    if (manning_scale && flood::pageable(manning_scale)) {
+        for (int m = 0; m < M; ++m) manning_scale[m] = r[m].scale;
+        manning_scale = nullptr;
+    }
+    if (weights && flood::pageable(weights)) {
+        for (int m = 0; m < M; ++m) weights[m] = r[m].w;
+        weights = nullptr;
+    }
     for (int m = 0; m < M; ++m) {
-        if (t) t[m] = c[m].t;
-        if (steps) steps[m] = c[m].steps;
-        if (hmax) std::memcpy(&hmax[m], &c[m].hmax_bits, sizeof(float));
+        if (t) t[m] = r[m].t;
+        if (steps) steps[m] = r[m].steps;
+        if (hmax) hmax[m] = r[m].hmax;
     }
     if (rain_mult) CK(g, cudaMemcpy(rain_mult, g->rain_mult, sizeof(float) * M, cudaMemcpyDefault));
     if (manning_scale) CK(g, cudaMemcpy(manning_scale, g->scale, sizeof(float) * M, cudaMemcpyDefault));

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "flood_internal.cuh"
+#include "readout.cuh"
 #include "resident.cuh"
 #include "trace.cuh"
 
@@ -57,9 +58,13 @@ struct flood_grid {
     double* d = nullptr;          // [G_cap]
     double* sigma = nullptr;      // [G_cap]
     float* beta = nullptr;        // [M]
-    int32_t* pfi = nullptr;       // idx, src, copy_dst, copy_src: 4 x [M]
-    int32_t* pf_small = nullptr;  // n_copy, resampled, status
-    double* neff = nullptr;       // [1]
+    // the filter's outputs, one allocation (w_post's): neff [1] follows w_post
+    // [M], then n_copy, resampled, status and a spare, then idx, src,
+    // copy_dst, copy_src: 4 x [M]
+    double* neff = nullptr;
+    int32_t* pf_small = nullptr;
+    int32_t* pfi = nullptr;
+    flood::MemberRow* rows = nullptr;  // [M] flood_get_members' scalars
     double* part = nullptr;       // storage partials
     int part_cap = 0;
     double* storage = nullptr;    // [M]

@@ -12,9 +12,8 @@ namespace flood {
 namespace {
 
 // DA step (I): y[i][k] = depth of member i at gauge cell k.
-__global__ void gauge_kernel(const float* __restrict__ state, const MemberClock* __restrict__ ms,
-                             const int32_t* __restrict__ cells, int G, int M, int ld, int nx,
-                             size_t plane, float* __restrict__ y)
+__device__ __forceinline__ void gauge_one(const float* state, const MemberClock* ms, const int32_t* cells, int G,
+                                          int M, int ld, int nx, size_t plane, float* y)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= M * G) return;
@@ -23,6 +22,20 @@ __global__ void gauge_kernel(const float* __restrict__ state, const MemberClock*
     const int r = cell / nx, c = cell % nx;
     const float* h = state + (size_t)(ms[m].cur * M + m) * 3 * plane;
     y[t] = h[(size_t)r * ld + c];
+}
+
+__global__ void gauge_kernel(const float* __restrict__ state, const MemberClock* __restrict__ ms,
+                             const int32_t* __restrict__ cells, int G, int M, int ld, int nx,
+                             size_t plane, float* __restrict__ y)
+{
+    gauge_one(state, ms, cells, G, M, ld, nx, plane, y);
+}
+
+__global__ void gauge_args_kernel(const float* __restrict__ state, const MemberClock* __restrict__ ms,
+                                  const __grid_constant__ GaugeCells cells, int G, int M, int ld, int nx, size_t plane,
+                                  float* __restrict__ y)
+{
+    gauge_one(state, ms, cells.cell, G, M, ld, nx, plane, y);
 }
 
 // The same from checkpoint slots: each member's state after its steps so far.
@@ -307,6 +320,12 @@ void launch_gauge(const float* state, const MemberClock* ms, const int32_t* cell
 {
     const int n = M * G;
     gauge_kernel<<<(n + 127) / 128, 128, 0, s>>>(state, ms, cells, G, M, ld, nx, plane, y);
+}
+
+void launch_gauge_args(const float* state, const MemberClock* ms, const GaugeCells& cells, int G, int M, int ld,
+                       int nx, size_t plane, float* y, cudaStream_t s)
+{
+    gauge_args_kernel<<<(M * G + 127) / 128, 128, 0, s>>>(state, ms, cells, G, M, ld, nx, plane, y);
 }
 
 void launch_gauge_slots(const float* slots, const MemberClock* ms, int last, const int32_t* cells, int G, int M,

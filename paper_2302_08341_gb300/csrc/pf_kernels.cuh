@@ -32,6 +32,14 @@ struct PfArgs {
 
 void launch_gauge(const float* state, const MemberClock* ms, const int32_t* cells, int G, int M,
                   int ld, int nx, size_t plane, float* y, cudaStream_t s);
+// The same with the gauges' cells as a launch argument (a copy to the device
+// costs more than the samples).
+constexpr int kGaugeArgs = 64;
+struct GaugeCells {
+    int32_t cell[kGaugeArgs];
+};
+void launch_gauge_args(const float* state, const MemberClock* ms, const GaugeCells& cells, int G, int M, int ld,
+                       int nx, size_t plane, float* y, cudaStream_t s);
 void launch_gauge_slots(const float* slots, const MemberClock* ms, int last, const int32_t* cells, int G, int M,
                         int ld, int nx, size_t plane, float* y, cudaStream_t s);
 cudaError_t launch_pf(const PfArgs& a, cudaStream_t s);
