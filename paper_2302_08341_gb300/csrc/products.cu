@@ -156,6 +156,16 @@ struct ProdTma {
 
 constexpr int kProdWarps = 4;  // warps per CTA of the staged kernel
 
+// CTAs an SM holds of the kernel of MT slots: its registers (the slots and
+// about 30 more a thread) and its stages allow as many.
+constexpr int prod_ctas(int mt) { return mt <= 32 ? 8 : mt <= 48 ? 6 : mt <= 64 ? 5 : mt <= 96 ? 4 : 3; }
+
+// Unequal weights: the weights in units of 2^-60 as a table of kCopies copies
+// side by side, [member][lane % kCopies]: the lanes of a warp look up
+// different members, which in one copy met in the same banks.
+constexpr int kCopies = 8;
+constexpr int kBlock = 8;      // sorted keys whose weights are summed together
+
 template <int MT>
 __host__ __device__ constexpr int prod_stage_bytes() { return (MT * 32 * 4 + 127) / 128 * 128; }
 
@@ -180,9 +190,10 @@ __host__ __device__ constexpr int prod_stage_bytes() { return (MT * 32 * 4 + 127
 // FP32 numbers (about four binades); beyond that it is shifted right by the
 // fewest bits that fit, so values closer than 2^shift representable numbers
 // may share a place and come out in index order.  One pass over the sorted
-// keys sums the weights (exact integers) and keeps, per level, the key at
-// the first position whose cumulative weight reaches it, and the weight of
-// the members at or above the threshold.  A lane with shifted places then
+// keys sums the weights (exact integers) by blocks of eight, noting per level
+// the block that reaches it; the key is then looked for in that block, and the
+// weight at or above the threshold is the total less that of the keys below
+// it, found by binary search.  A lane with shifted places then
 // checks its sorted keys: a level whose key is alone in its place takes that
 // member's value from its maxima in global memory; where members share it,
 // the answer lies among them (every place below holds smaller values, every
@@ -190,23 +201,36 @@ __host__ __device__ constexpr int prod_stage_bytes() { return (MT * 32 * 4 + 127
 // against the exact weighted distribution function.  The members in the
 // threshold's place, counted as reaching it, are checked against it.
 //
+// What bounds it: the ALU pipe (a comparator is two instructions at half
+// rate; 16-bit pairs run at the same rate a register, but nine bits of place
+// tie too often), and with unequal weights the fetching of instructions.  The
+// pass over every key for every level took 1920 instructions a cell of 4900;
+// by blocks it takes 900.  2000 x 2000 x 96, unequal weights: 1.55 -> 1.21 ms.
+// Slots come in steps of 8 to 16 members (LO: the step below, whose slots need
+// no test for padding) where 32, 64, 96 and 128 were: 1000 x 1000 cells
+// with 8 members 130 -> 73 us, 40 members 251 -> 159 us, 128 721 -> 601 us;
+// equal weights 73 -> 49, 126 -> 104, 337 -> 309 us.
+//
 // Every wait is bounded: one that gives up records FLOOD_ERR_TIMEOUT in the
 // error word, waits for the warp's copy in flight and returns.
-template <int MT, bool EQUAL>
-__global__ void __launch_bounds__(32 * kProdWarps, MT <= 96 ? 4 : 2)
+template <int MT, int LO, bool EQUAL>
+__global__ void __launch_bounds__(32 * kProdWarps, prod_ctas(MT))
     tma_products_kernel(const __grid_constant__ ProdTma t)
 {
     extern __shared__ unsigned char smem_raw[];
     const ProdArgs& a = t.a;
     constexpr int kStage = prod_stage_bytes<MT>();
     constexpr long long kBudget = flood::kTmaWaitBudgetDefault;
-    constexpr uint32_t kPad = 0xFFFFFFFFu;   // key of a padding slot: index 127, no weight
-    __shared__ long long us[EQUAL ? 1 : 128];
+    constexpr uint32_t kPad = 0xFFFFFF80u | (MT - 1);   // key of a padding slot: a member past M, no weight
+    __shared__ long long us_all[EQUAL ? 1 : MT * kCopies];
     if (!EQUAL) {
-        for (int j = threadIdx.x; j < 128; j += blockDim.x) us[j] = j < a.M ? a.u[j] : 0;
+        for (int j = threadIdx.x; j < MT * kCopies; j += blockDim.x)
+            us_all[j] = j / kCopies < a.M ? a.u[j / kCopies] : 0;
         __syncthreads();
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long* const us = us_all + (EQUAL ? 0 : lane % kCopies);
+    auto weight = [&](uint32_t key) { return us[(key & 0x7Fu) * kCopies]; };
     unsigned char* base = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
     const uint32_t bar = flood::smem_u32(base) + 8u * w;
@@ -250,7 +274,7 @@ __global__ void __launch_bounds__(32 * kProdWarps, MT <= 96 ? 4 : 2)
             float v[MT];
 #pragma unroll
             for (int j = 0; j < MT; ++j)
-                v[j] = j < a.M ? stage[j * 32 + lane] : __int_as_float(0x7f800000);
+                v[j] = j < LO || j < a.M ? stage[j * 32 + lane] : __int_as_float(0x7f800000);
             odd_even_merge_sort<float, N, MT>(v);
             // the sorted slots go back into this lane's column of the stage
             // (the lane alone reads and writes it): a level then reads one
@@ -279,55 +303,97 @@ __global__ void __launch_bounds__(32 * kProdWarps, MT <= 96 ? 4 : 2)
                 a.pct[(size_t)q * a.ny * a.nx + out] = pv[q];
             }
         } else {
-            uint32_t key[MT];
-            uint32_t omin = kPad, omax = 0u;
-#pragma unroll
-            for (int j = 0; j < MT; ++j) {
-                if (j < a.M) {
-                    const uint32_t o = ord_of(stage[j * 32 + lane]);
-                    key[j] = o;
+            // The loops over the members are short and rolled wherever the
+            // slots need not be registers: the sort alone is 34 KB of code at
+            // 96 slots, and with as much again unrolled around it the warps
+            // waited for instructions (10 of 13.7 cycles an instruction).
+            uint32_t* const kcol = reinterpret_cast<uint32_t*>(stage) + lane;
+            uint32_t omin = 0xFFFFFFFFu, omax = 0u;
+#pragma unroll 8
+            for (int j = 0; j < a.M; ++j) {
+                omin = min(omin, kcol[j * 32]);
+                omax = max(omax, kcol[j * 32]);
+            }
+            // bits of non-negative values lie as their ord does
+            uint32_t base0 = 0x80000000u;
+            if (__any_sync(0xffffffffu, omax >= 0x80000000u)) {
+                base0 = 0u;
+                omin = 0xFFFFFFFFu;
+                omax = 0u;
+#pragma unroll 2
+                for (int j = 0; j < a.M; ++j) {
+                    const uint32_t o = ord_of(__uint_as_float(kcol[j * 32]));
+                    kcol[j * 32] = o;
                     omin = min(omin, o);
                     omax = max(omax, o);
-                } else {
-                    key[j] = kPad;
                 }
             }
             const uint32_t d = omax - omin;
             int sh = max(0, 7 - __clz(d));              // bits of d above 25
             if ((d >> sh) == 0x1FFFFFFu) ++sh;          // keeps real keys below kPad
             const bool exact = sh == 0;
+            uint32_t key[MT];
 #pragma unroll
             for (int j = 0; j < MT; ++j)
-                if (j < a.M) key[j] = (((key[j] - omin) >> sh) << 7) | (uint32_t)j;
+                key[j] = j < LO || j < a.M ? (((kcol[j * 32] - omin) >> sh) << 7) | (uint32_t)j : kPad;
+            omin += base0;
+            omax += base0;
             odd_even_merge_sort<uint32_t, N, MT>(key);
             // the sorted keys go into this lane's column of the stage (its
-            // values are in registers now), and the pass over them is a short
-            // loop: unrolled over the registers it doubled the code and the
-            // warps waited on instruction fetch
-            uint32_t* const kcol = reinterpret_cast<uint32_t*>(stage) + lane;
+            // values are in registers now)
 #pragma unroll
             for (int k = 0; k < MT; ++k) kcol[k * 32] = key[k];
+            // sorted keys below kq
+            auto below_key = [&](uint32_t kq) -> int {
+                int n = 0;
+#pragma unroll
+                for (int st = kStep; st > 0; st >>= 1)
+                    if (n + st <= MT && kcol[(n + st - 1) * 32] < kq) n += st;
+                return n;
+            };
             // the threshold as a key: the first key of its place (shifted
             // lanes settle the members of that place below)
             const uint32_t kth =
                 a.th_ord <= omin ? 0u : a.th_ord > omax ? kPad : ((a.th_ord - omin) >> sh) << 7;
-            long long P = 0, ex = 0;
-            uint32_t kc[kLevelsPerPass];
+            // The weights are summed by blocks of keys, P those of the blocks
+            // so far; per level W is the sum before the block that reaches it
+            // and nb that block, and below the sum before the threshold's.
+            const int nth = a.exceed ? below_key(kth) : 0;  // the keys below the threshold
+            long long P = 0, below = 0, W[kLevelsPerPass];
+            int nb[kLevelsPerPass];
 #pragma unroll
-            for (int q = 0; q < kLevelsPerPass; ++q) kc[q] = kPad;
-#pragma unroll 4
-            for (int k = 0; k < MT; ++k) {
-                const uint32_t kk = kcol[k * 32];
-                const long long uk = us[kk & 0x7Fu];
+            for (int q = 0; q < kLevelsPerPass; ++q) W[q] = nb[q] = 0;
+#pragma unroll 1
+            for (int k = 0; k < MT; k += kBlock) {
 #pragma unroll
-                for (int q = 0; q < kLevelsPerPass; ++q) kc[q] = P < a.A[q] ? kk : kc[q];
-                P += uk;
-                ex += kk >= kth ? uk : 0;
+                for (int q = 0; q < kLevelsPerPass; ++q)
+                    if (P < a.A[q]) {
+                        W[q] = P;
+                        nb[q] = k;
+                    }
+                if (k <= nth) below = P;
+#pragma unroll
+                for (int i = 0; i < kBlock; ++i) P += weight(kcol[(k + i) * 32]);
             }
-            // per level the ord of the answer (none reached: the largest value)
-            uint32_t oq[kLevelsPerPass];
+            long long ex = P - below;
+            for (int k = min(nth / kBlock * kBlock, MT - kBlock); k < nth; ++k) ex -= weight(kcol[k * 32]);
+            // per level the first key whose cumulative weight reaches it and
+            // its ord (none reached: the largest value)
+            uint32_t kc[kLevelsPerPass], oq[kLevelsPerPass];
 #pragma unroll
-            for (int q = 0; q < kLevelsPerPass; ++q) oq[q] = P < a.A[q] ? omax : (kc[q] >> 7) + omin;
+            for (int q = 0; q < kLevelsPerPass; ++q) {
+                kc[q] = 0u;
+                oq[q] = omax;
+                if (q >= a.n_levels) continue;
+                const uint32_t* kb = kcol + nb[q] * 32;
+#pragma unroll
+                for (int k = 0; k < kBlock; ++k) {
+                    const uint32_t kk = kb[k * 32];
+                    if (W[q] < a.A[q]) kc[q] = kk;
+                    W[q] += weight(kk);
+                }
+                if (P >= a.A[q]) oq[q] = (kc[q] >> 7) + omin;
+            }
             if (!exact) {
                 // a lane with shifted places: its keys order the members up
                 // to values that share a place.  The exceedance counted every
@@ -337,19 +403,12 @@ __global__ void __launch_bounds__(32 * kProdWarps, MT <= 96 ? 4 : 2)
                 // (the stage holds the keys now; the group's lines are still
                 // in L2)
                 const float* fc = a.field + (size_t)r * a.ld + c;
-                auto below_key = [&](uint32_t kq) -> int {  // sorted keys below kq
-                    int n = 0;
-#pragma unroll
-                    for (int st = kStep; st > 0; st >>= 1)
-                        if (n + st <= MT && kcol[(n + st - 1) * 32] < kq) n += st;
-                    return n;
-                };
                 if (a.th_ord > omin && a.th_ord <= omax) {
                     const uint32_t pth = (a.th_ord - omin) >> sh;
                     const int end = below_key((pth + 1) << 7);
                     for (int p = below_key(pth << 7); p < end; ++p) {
                         const uint32_t id = kcol[p * 32] & 0x7Fu;  // a real member: < M
-                        if (id < (uint32_t)a.M && ord_of(fc[(size_t)id * a.plane]) < a.th_ord) ex -= us[id];
+                        if (id < (uint32_t)a.M && ord_of(fc[(size_t)id * a.plane]) < a.th_ord) ex -= weight(id);
                     }
                 }
 #pragma unroll
@@ -378,7 +437,7 @@ __global__ void __launch_bounds__(32 * kProdWarps, MT <= 96 ? 4 : 2)
                         uint32_t nxt = hi;
                         for (int j = 0; j < a.M; ++j) {
                             const uint32_t o = ord_of(fc[(size_t)j * a.plane]);
-                            if (o <= v) W += us[j];
+                            if (o <= v) W += weight((uint32_t)j);
                             else nxt = min(nxt, o);
                         }
                         if (W >= a.A[q]) break;
@@ -445,21 +504,29 @@ __global__ void __launch_bounds__(kCells) staged_products_kernel(const ProdArgs 
 
 size_t products_smem(int M) { return sizeof(long long) * M + sizeof(float) * (size_t)M * kCells; }
 
-template <int MT, bool EQUAL>
+template <int MT, int LO, bool EQUAL>
 void launch_tma_products(ProdTma& t, int n_sm, cudaStream_t s)
 {
     constexpr size_t shm = 128 + (size_t)prod_stage_bytes<MT>() * kProdWarps + 128;
     static int per_sm = 0;
     if (!per_sm) {
-        cudaFuncSetAttribute(tma_products_kernel<MT, EQUAL>,
+        cudaFuncSetAttribute(tma_products_kernel<MT, LO, EQUAL>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tma_products_kernel<MT, EQUAL>,
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tma_products_kernel<MT, LO, EQUAL>,
                                                       32 * kProdWarps, shm);
         per_sm = std::max(per_sm, 1);
     }
     const int need = (t.n_groups + kProdWarps - 1) / kProdWarps;
     const int blocks = std::max(1, std::min(need, n_sm * per_sm));
-    tma_products_kernel<MT, EQUAL><<<blocks, 32 * kProdWarps, shm, s>>>(t);
+    tma_products_kernel<MT, LO, EQUAL><<<blocks, 32 * kProdWarps, shm, s>>>(t);
+}
+
+// The kernel with the fewest slots that hold every member.
+template <bool EQUAL, int LO, int MT, int... MORE>
+void launch_slots(ProdTma& t, int n_sm, cudaStream_t s)
+{
+    if (t.a.M <= MT) return launch_tma_products<MT, LO, EQUAL>(t, n_sm, s);
+    if constexpr (sizeof...(MORE) > 0) launch_slots<EQUAL, MT, MORE...>(t, n_sm, s);
 }
 
 // The staged kernel up to 128 members (its copy box holds every member of
@@ -471,15 +538,9 @@ void launch_products(ProdTma& t, bool have_map, bool equal, int n_sm, cudaStream
         dim3 grid((t.a.nx + kCells - 1) / kCells, t.a.ny);
         staged_products_kernel<<<grid, kCells, products_smem(M), s>>>(t.a);
     } else if (equal) {
-        if (M <= 32) launch_tma_products<32, true>(t, n_sm, s);
-        else if (M <= 64) launch_tma_products<64, true>(t, n_sm, s);
-        else if (M <= 96) launch_tma_products<96, true>(t, n_sm, s);
-        else launch_tma_products<128, true>(t, n_sm, s);
+        launch_slots<true, 0, 8, 16, 24, 32, 48, 64, 80, 96, 112, 128>(t, n_sm, s);
     } else {
-        if (M <= 32) launch_tma_products<32, false>(t, n_sm, s);
-        else if (M <= 64) launch_tma_products<64, false>(t, n_sm, s);
-        else if (M <= 96) launch_tma_products<96, false>(t, n_sm, s);
-        else launch_tma_products<128, false>(t, n_sm, s);
+        launch_slots<false, 0, 8, 16, 24, 32, 48, 64, 80, 96, 112, 128>(t, n_sm, s);
     }
 }
 
@@ -596,7 +657,6 @@ extern "C" int flood_ensemble_products(flood_grid* g, double threshold, int n_le
         if (rc) return rc;
     }
     long long* du = g->prod_u;
-    CK(g, cudaMemcpyAsync(du, u.data(), sizeof(long long) * M, cudaMemcpyHostToDevice, s));
     static bool attr = false;
     if (!attr) {
         CK(g, cudaFuncSetAttribute(staged_products_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -609,6 +669,8 @@ extern "C" int flood_ensemble_products(flood_grid* g, double threshold, int n_le
         M <= 128 && flood::encode_map_3d(&tm.map, g->hmax_field, g->nx, g->ny, (uint64_t)M,
                                          sizeof(float) * g->ld, sizeof(float) * g->plane, 32, 1,
                                          (uint32_t)M) == 0;
+    if (!have_map || !equal)  // (equal weights: the ranks say all)
+        CK(g, cudaMemcpyAsync(du, u.data(), sizeof(long long) * M, cudaMemcpyHostToDevice, s));
     tm.groups_per_row = (g->nx + 31) / 32;
     tm.n_groups = tm.groups_per_row * g->ny;
     ProdArgs& a = tm.a;
@@ -648,9 +710,9 @@ extern "C" int flood_ensemble_products(flood_grid* g, double threshold, int n_le
     if (n_levels && !pct_dev_ok)
         CK(g, cudaMemcpyAsync(pct, dpct, sizeof(float) * cells * n_levels, cudaMemcpyDefault, s));
     if (buf) CK(g, cudaFreeAsync(buf, s));
-    CK(g, cudaStreamSynchronize(s));
     int err = 0;
-    CK(g, cudaMemcpy(&err, g->err, sizeof(int), cudaMemcpyDeviceToHost));
+    CK(g, cudaMemcpyAsync(&err, g->err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(g, cudaStreamSynchronize(s));
     if (err & 2) return flood::fail(g, FLOOD_ERR_TIMEOUT, "a bounded wait for staged maxima gave up");
     return FLOOD_OK;
 }

@@ -286,3 +286,29 @@ def test_weighted_keys_with_several_groups_per_warp(capi):
     sub = hm[:, rows]
     assert np.array_equal(exceed[rows], prod.exceedance(sub, w_dev, 0.2))
     assert np.array_equal(pct[:, rows], prod.percentiles(sub, w_dev, levels))
+
+
+@pytest.mark.parametrize("M", [1, 8, 9, 16, 17, 24, 25, 32, 48, 49, 80, 81, 112, 113, 128])
+@pytest.mark.parametrize("equal", [True, False])
+def test_products_at_the_edges_of_the_slot_counts(capi, M, equal):
+    """Member counts that fill a kernel's slots or leave most of the last ones
+    padding, with thresholds below, among and above all maxima: the maps equal
+    the oracle's, bit for bit."""
+    ny, nx = 9, 70
+    terr = synth.make_terrain(ny, nx, seed=56)
+    rm, sc = synth.ensemble_prior(56, M)
+    rng = np.random.default_rng(1000 + M)
+    w = np.full(M, 1.0 / M) if equal else rng.random(M) ** 2
+    w = w / w.sum()
+    h0 = (rng.uniform(0.02, 0.4, (ny, nx)) * rm[:, None, None] * rng.uniform(0.9, 1.1, (M, ny, nx))).astype(np.float32)
+    h0[:, :3, :40] = np.exp(rng.uniform(-14.0, -4.0, (M, 3, 40)))   # films over many binades
+    levels = (0.1, 0.5, 0.9)
+    with capi.Grid(terr.z, terr.n) as g:
+        g.ensemble_init(M, rm, sc, synth.hyetograph_constant(10.0, 60.0), h0=h0)
+        g.track_max_depth(True)
+        g.set_members(weights=w)
+        w = g.members()["weights"]
+        for threshold in (0.0, 1e-4, 0.1, 10.0):
+            exceed, pct = g.ensemble_products(threshold, levels)
+            assert np.array_equal(exceed, prod.exceedance(h0, w, threshold))
+            assert np.array_equal(pct, prod.percentiles(h0, w, levels))
