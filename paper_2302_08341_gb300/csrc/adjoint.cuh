@@ -24,6 +24,7 @@ struct AdjArgs {
     float lc_drains[4];
     double* gdpart;          // [M][nslot] per-warp partials of dL/d(drainage rate) (land cover)
     const float* scale;      // [M]
+    const double* rscale;    // [M] 1 / scale
     const MemberPlan* log;   // [M][dt_log_cap] plans of the recorded steps
     const int* seg_end;      // [M] first step index past this segment, per member
     int dt_log_cap;
@@ -54,6 +55,7 @@ void launch_adjoint_tma(const AdjTmaArgs& t, int members_per_cta, cudaStream_t s
 int adjoint_tma_box_cols();
 void launch_seed(const AdjArgs& a, const int32_t* sample_step, const float* y, const double* d,
                  const int32_t* cells, int ns, int G, cudaStream_t s);
+void launch_reciprocals(const float* x, int n, double* out, cudaStream_t s);
 void launch_reduce_members(const float* gm, int M, int ny, int nx, int ld, size_t plane, float* out,
                            cudaStream_t s);
 

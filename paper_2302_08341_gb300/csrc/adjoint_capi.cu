@@ -251,7 +251,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     if ((rc = grow(g, &g->lam, room.lam, 2 * (size_t)M * ms))) return rc;
     const int rrows = g->launch_fixed ? g->rows_per_strip : reverse_rows(g->ny, g->nx, M, g->n_sm);
     const int nslot = flood::step_nslot(g->ny, g->nx, rrows);
-    if ((rc = grow(g, &g->gpart, room.gpart, (size_t)M * nslot * 2))) return rc;
+    if ((rc = grow(g, &g->gpart, room.gpart, (size_t)M * nslot * 2 + M))) return rc;
     if ((rc = grow(g, &g->seg_end, room.seg_end, M))) return rc;
     if ((rc = grow(g, &g->samp_step, room.samp_step, (size_t)ns * M))) return rc;
     if ((rc = grow(g, &g->samp_d, room.samp_d, (size_t)ns * G))) return rc;
@@ -262,6 +262,9 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     }
     CK(g, cudaMemsetAsync(g->lam, 0, sizeof(float) * 2 * M * ms, s));
     CK(g, cudaMemsetAsync(g->gpart, 0, sizeof(double) * M * nslot * 2, s));
+    double* const rscale = g->gpart + (size_t)M * nslot * 2;  // 1 / scale of every member, behind the partials
+    flood::launch_reciprocals(g->scale, M, rscale, s);
+    g->launches++;
     if (g->lc_on) {
         if ((rc = grow(g, &g->gdpart, room.gdpart, (size_t)M * nslot))) return rc;
         CK(g, cudaMemsetAsync(g->gdpart, 0, sizeof(double) * M * nslot, s));
@@ -357,6 +360,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             }
         }
         b.scale = g->scale;
+        b.rscale = rscale;
         b.log = g->log;
         b.seg_end = g->seg_end;
         b.dt_log_cap = g->log_cap;

@@ -180,9 +180,14 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
         C = S;
     }
     const int slot = blockIdx.z * ((a.nx + kSpan - 1) / kSpan) + span;
-    adjoint_partials(a.gpart, a.nslot, m, slot, lane, gr_s, gr_c, gs_s, gs_c, pl.rdt,
-                     1.0 / (double)s);
-    if (RW) adjoint_drain_partial(a.gdpart, a.nslot, m, slot, lane, gd_s, gd_c, pl.dt);
+    adjoint_partials(a.gpart, RW ? a.gdpart : nullptr, a.nslot, m, slot, lane, Sum2{gr_s, -gr_c}, Sum2{gs_s, -gs_c},
+                     Sum2{gd_s, -gd_c}, pl.rdt, a.rscale[m], pl.dt);
+}
+
+__global__ void reciprocals_kernel(const float* __restrict__ x, int n, double* __restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = 1.0 / (double)x[i];
 }
 
 // Loss sensitivity at observation times: the state after step j is observed
@@ -251,6 +256,11 @@ void launch_seed(const AdjArgs& a, const int32_t* sample_step, const float* y, c
 {
     const int n = a.M * G;
     launch_pdl(seed_kernel, (n + 127) / 128, 128, 0, s, a, sample_step, y, d, cells, ns, G);
+}
+
+void launch_reciprocals(const float* x, int n, double* out, cudaStream_t s)
+{
+    reciprocals_kernel<<<(n + 127) / 128, 128, 0, s>>>(x, n, out);
 }
 
 void launch_reduce_members(const float* gm, int M, int ny, int nx, int ld, size_t plane, float* out,

@@ -276,9 +276,8 @@ __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
     }
     if (r < r1) row(r, std::false_type{}, std::false_type{});
     const int vslot = blockIdx.z * ((a.nx + kSpan - 1) / kSpan) + span;
-    adjoint_partials(a.gpart, a.nslot, m, vslot, lane, gr_s, gr_c, gs_s, gs_c, pl.rdt,
-                     1.0 / (double)s);
-    if (LC) adjoint_drain_partial(a.gdpart, a.nslot, m, vslot, lane, gd_s, gd_c, pl.dt);
+    adjoint_partials(a.gpart, LC ? a.gdpart : nullptr, a.nslot, m, vslot, lane, Sum2{gr_s, -gr_c}, Sum2{gs_s, -gs_c},
+                     Sum2{gd_s, -gd_c}, pl.rdt, a.rscale[m], pl.dt);
 }
 
 template <int WM>

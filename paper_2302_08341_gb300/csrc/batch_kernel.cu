@@ -54,34 +54,25 @@ __device__ __forceinline__ void finish_task(const BatchArgs& a, MemberClock* ms_
 {
     if (mo.bad) atomicOr(a.err, 1);
     const unsigned hb = __reduce_max_sync(0xffffffffu, mo.bad ? 0u : __float_as_uint(mo.hmax) & 0x7fffffffu);
-    double out_acc = mo.out, clamp_acc = mo.clamp;
-    double drn_acc = LC ? mo.drn : 0.0;
-    // most strips neither let water out nor clamped any: no FP64 sums there
-    if (__any_sync(0xffffffffu, out_acc != 0.0 || clamp_acc != 0.0 || drn_acc != 0.0)) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            out_acc += __shfl_xor_sync(0xffffffffu, out_acc, off);
-            clamp_acc += __shfl_xor_sync(0xffffffffu, clamp_acc, off);
-            if (LC) drn_acc += __shfl_xor_sync(0xffffffffu, drn_acc, off);
-        }
-    }
+    Sum2 out, clamp, drn;
+    mo.warp_sums<LC>(out, clamp, drn);
     if (lane == 0) {
         atomicMax(&ms_out[tk.scen].hmax_bits, hb);
-        if (out_acc != 0.0 || clamp_acc != 0.0) {
+        if (!out.zero() || !clamp.zero()) {
             double* v = a.vacc + (size_t)tk.slot * 2;
             if (ATOMIC) {
-                atomicAdd(v, out_acc * p.dt * a.dxd);
-                atomicAdd(v + 1, clamp_acc * a.cell_area);
+                atomicAdd(v, out.value() * p.dt * a.dxd);
+                atomicAdd(v + 1, clamp.value() * a.cell_area);
             } else {
-                v[0] += out_acc * p.dt * a.dxd;
-                v[1] += clamp_acc * a.cell_area;
+                v[0] += out.value() * p.dt * a.dxd;
+                v[1] += clamp.value() * a.cell_area;
             }
         }
-        if (LC && drn_acc != 0.0) {
+        if (LC && !drn.zero()) {
             if (ATOMIC)
-                atomicAdd(a.dacc + tk.slot, drn_acc * a.cell_area);
+                atomicAdd(a.dacc + tk.slot, drn.value() * a.cell_area);
             else
-                a.dacc[tk.slot] += drn_acc * a.cell_area;
+                a.dacc[tk.slot] += drn.value() * a.cell_area;
         }
     }
 }

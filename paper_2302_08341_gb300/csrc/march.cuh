@@ -7,15 +7,31 @@
 #pragma once
 
 #include "flood_internal.cuh"
+#include "sum2.cuh"
 
 namespace flood {
 
 struct MarchOut {
     float hmax;
     bool bad;
-    double out;     // this lane's outflow sum of q over the warp's edge links
-    double clamp;   // sum of the negative depths reset to zero
-    double drn;     // drained depth (land cover)
+    Sum2 out;       // this lane's outflow sum of q over the warp's edge links
+    float clamp;    // sum of the negative depths reset to zero
+    Sum2 drn;       // drained depth (land cover)
+
+    // The lanes' sums over the warp, where any is not zero: most strips neither
+    // let water out nor clamped any.
+    template <bool LC>
+    __device__ __forceinline__ void warp_sums(Sum2& o, Sum2& c, Sum2& d) const
+    {
+        o = out;
+        c.add(clamp);
+        if (LC) d = drn;
+        if (__any_sync(0xffffffffu, !out.zero() || clamp != 0.0f)) {
+            o.warp_sum();
+            c.warp_sum();
+        }
+        if (LC) d.warp_sum();
+    }
 };
 
 __device__ __forceinline__ void m_load4(float (&v)[4], const float* p)
@@ -298,9 +314,9 @@ __device__ __forceinline__ MarchOut march_rows(const float* __restrict__ src, fl
     MarchOut out;
     out.hmax = hmax;
     out.bad = !(hmax <= 3.0e38f);  // a NaN or an overflow anywhere
-    out.out = (double)out_s - (double)out_c;
-    out.clamp = (double)clamp;
-    out.drn = (double)drn_s - (double)drn_c;
+    out.out = Sum2{out_s, -out_c};
+    out.clamp = clamp;
+    out.drn = Sum2{drn_s, -drn_c};
     return out;
 }
 

@@ -128,26 +128,20 @@ __global__ void __launch_bounds__(32 * WM * WC, (LC ? 4 : FLOOD_STEP_MIN_BLOCKS)
                                        &lk);
     if (mo.bad) atomicOr(a.err, 1);
     if (REPLAY) return;
-    // warp reductions: max depth (order-free); volume partials widened to
-    // FP64 once per warp and reduced in a fixed order
+    // warp reductions: max depth (order-free); volume partials in a fixed
+    // order, widened to FP64 once per warp
     const unsigned hb = __reduce_max_sync(0xffffffffu, mo.bad ? 0u : __float_as_uint(mo.hmax) & 0x7fffffffu);
-    double out_acc = mo.out, clamp_acc = mo.clamp;
-    double drn_acc = LC ? mo.drn : 0.0;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        out_acc += __shfl_xor_sync(0xffffffffu, out_acc, off);
-        clamp_acc += __shfl_xor_sync(0xffffffffu, clamp_acc, off);
-        if (LC) drn_acc += __shfl_xor_sync(0xffffffffu, drn_acc, off);
-    }
+    Sum2 out, clamp, drn;
+    mo.warp_sums<LC>(out, clamp, drn);
     if (lane == 0) {
         atomicMax(&a.ms_out[m].hmax_bits, hb);
         const int slot = blockIdx.z * ((a.nx + kSpan - 1) / kSpan) + span;
-        if (out_acc != 0.0 || clamp_acc != 0.0) {
+        if (!out.zero() || !clamp.zero()) {
             double* v = a.vacc + ((size_t)m * a.nslot + slot) * 2;
-            v[0] += out_acc * p.dt * a.dxd;
-            v[1] += clamp_acc * a.cell_area;
+            v[0] += out.value() * p.dt * a.dxd;
+            v[1] += clamp.value() * a.cell_area;
         }
-        if (LC && drn_acc != 0.0) a.dacc[(size_t)m * a.nslot + slot] += drn_acc * a.cell_area;
+        if (LC && !drn.zero()) a.dacc[(size_t)m * a.nslot + slot] += drn.value() * a.cell_area;
     }
 }
 

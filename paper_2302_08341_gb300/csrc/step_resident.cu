@@ -37,6 +37,7 @@
 #include "march.cuh"
 #include "quad.cuh"
 #include "resident.cuh"
+#include "sum2.cuh"
 
 namespace flood {
 
@@ -82,39 +83,6 @@ __device__ __forceinline__ bool ld_tagged(const unsigned long long* p, float4& v
     return (uint32_t)(w[0] >> 32) == tag && (uint32_t)(w[1] >> 32) == tag && (uint32_t)(w[2] >> 32) == tag &&
            (uint32_t)(w[3] >> 32) == tag;
 }
-
-// A sum kept in two FP32 words (hi + lo, about 2^-46 relative): the FP64 pipe
-// takes 64 cycles a warp instruction, so the rows' sums stay off it and are
-// widened once at the end.
-struct Sum2 {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add(float x)
-    {
-        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        hi = s;
-    }
-    // x times the sum of two words
-    __device__ __forceinline__ void add_product(float x, float2 y)
-    {
-        const float p = __fmul_rn(x, y.x);
-        add(p);
-        lo = __fadd_rn(lo, __fmaf_rn(x, y.y, __fmaf_rn(x, y.x, -p)));
-    }
-    __device__ __forceinline__ void merge(float h, float l)
-    {
-        add(h);
-        lo = __fadd_rn(lo, l);
-    }
-    __device__ __forceinline__ void warp_sum()
-    {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float h = __shfl_xor_sync(0xffffffffu, hi, off), l = __shfl_xor_sync(0xffffffffu, lo, off);
-            merge(h, l);
-        }
-    }
-};
 
 // A step's constants, from warp 0 to the band.
 struct BandPlan {
@@ -552,7 +520,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
     if (tid < 3) {
         Sum2 sum;
         for (int w = 0; w < kWarps; ++w) sum.merge(s_red[tid][w].x, s_red[tid][w].y);
-        const double v = (double)sum.hi + (double)sum.lo;
+        const double v = sum.value();
         const size_t slot = (size_t)m * a.nslot + band;
         if (tid == 0 && v != 0.0) a.vacc[slot * 2] += v * a.dxd;
         if (tid == 1 && v != 0.0) a.vacc[slot * 2 + 1] += v * a.cell_area;

@@ -378,9 +378,9 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
 
     out.hmax = hmax;
     out.bad = !(hmax <= 3.0e38f);  // a NaN or an overflow anywhere
-    out.out = (double)out_s - (double)out_c;
-    out.clamp = (double)clamp;
-    out.drn = (double)drn_s - (double)drn_c;
+    out.out = Sum2{out_s, -out_c};
+    out.clamp = clamp;
+    out.drn = Sum2{drn_s, -drn_c};
     return true;
 }
 
