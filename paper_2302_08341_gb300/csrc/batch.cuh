@@ -65,6 +65,7 @@ struct BatchArgs {
     double* rain_acc;          // [S]
     int* err;
     double alpha_dx, g, dt_cap, dt_fixed, h_floor, rain_block, dxd, cell_area;
+    float cap_h;               // capped_below: no step from Eq. 4 below this depth
     float h_eps, edge_drop;
     int limiter, east_out, south_out;
     const CUtensorMap* maps;   // [S][2] per entry: state (ld, ny, 6 planes); z and n, or with

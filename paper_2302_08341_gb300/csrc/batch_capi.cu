@@ -195,6 +195,7 @@ flood::BatchArgs batch_args(const flood_batch* b, int64_t k)
     a.rain_acc = b->rain_acc;
     a.err = b->err;
     a.alpha_dx = b->p.alpha * b->p.dx;
+    a.cap_h = flood::capped_below(a.alpha_dx, b->p.g, b->p.dt_cap);
     a.g = b->p.g;
     a.dt_cap = b->p.dt_cap;
     a.dt_fixed = b->p.dt_fixed;

@@ -14,34 +14,52 @@ namespace flood {
 namespace {
 
 
-// Per-scenario plan (one thread per scenario, FP64): its own Eq. 4 step
+// Per-scenario plan (four lanes per scenario, FP64): its own Eq. 4 step
 // toward min(window end, own end time), clock, rain volume.
 __global__ void batch_plan_kernel(const BatchArgs a, int n_scen)
 {
     pdl_launch();
+    const int ii = blockIdx.x * kPlanMembers + threadIdx.x / 4, i = min(ii, n_scen - 1), lane = threadIdx.x & 3;
+    const ScenDesc& sd = a.scen[i];
+    auto end = [&]() {
+        const double t_stop = __ldcg(a.t_stop);
+        return sd.t_end < t_stop ? sd.t_end : t_stop;
+    };
+    // ahead of the wait, as plan_kernel does
+    PlanQuad<BatchArgs> w{a, lane, end(), sd.hyeto, nullptr, sd.nb, 0, 0, sd.rain_mult};
+    const uint32_t early = __ldcg(&a.ms_in[i].hmax_bits);
+    w.at(__ldcg(&a.ms_in[i].t));
+    w.step(__uint_as_float(early));
+    double v = (double)w.p.dr * a.cell_area;
     pdl_wait();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_scen) return;
-    const ScenDesc sd = a.scen[i];
-    const MemberClock in = a.ms_in[i];
-    const double t_stop = *a.t_stop;
-    const double t_end = sd.t_end < t_stop ? sd.t_end : t_stop;
-    const StepPlan sp = plan_step_p(a.alpha_dx, a.g, a.dt_cap, a.dt_fixed, a.h_floor, a.rain_block,
-                                    t_end, sd.hyeto, sd.nb, sd.rain_mult, in);
-    MemberPlan p;
-    fill_plan(p, sp, a.g, a.dxd);
+    const MemberClock in = ld_clock(a.ms_in + i);
+    if (ii >= n_scen) return;
+    const double t_end = end(), rain0 = a.rain_acc[i];
+    const float hmax = __uint_as_float(in.hmax_bits);
+    const bool moved = __double_as_longlong(in.t) != __double_as_longlong(w.t) ||
+                       __double_as_longlong(t_end) != __double_as_longlong(w.t_end);
+    if (moved ||
+        (in.hmax_bits != early && (w.needs_eq4(hmax) || w.needs_eq4(__uint_as_float(early))))) {
+        w.t_end = t_end;
+        if (moved) w.at(in.t);
+        w.step(hmax);
+        v = (double)w.p.dr * a.cell_area;
+    }
+    MemberPlan& p = w.p;
     p.cur = in.cur;
     p.ckpt = -1;
-    a.ms_clr[i].hmax_bits = 0u;
-    if (!sp.active) {
-        a.ms_out[i] = in;
-    } else {
-        a.ms_out[i].t = sp.t_next;
-        a.ms_out[i].steps = in.steps + 1;
-        a.ms_out[i].cur = 1 - in.cur;
-        a.rain_acc[i] += (double)sp.dr * a.cell_area * sd.ncell;
+    if (lane == 0) {
+        a.plan[i] = p;
+        a.ms_clr[i].hmax_bits = 0u;
+        if (!w.active) {
+            a.ms_out[i] = in;
+        } else {
+            a.ms_out[i].t = p.t_next;
+            a.ms_out[i].steps = in.steps + 1;
+            a.ms_out[i].cur = 1 - in.cur;
+            a.rain_acc[i] = __fma_rn(v, sd.ncell, rain0);
+        }
     }
-    a.plan[i] = p;
 }
 
 // A task's reductions: the scenario's maximum depth (atomicMax into its next
@@ -117,8 +135,8 @@ __global__ void __launch_bounds__(32 * W, 20 / W) batch_tma_kernel(const BatchAr
     const int lane = threadIdx.x;
     const int w = threadIdx.y;
     const int tid = blockIdx.x * W + w;
-    pdl_launch();
     pdl_wait();
+    pdl_launch();  // after the wait: the next plan may then read the clocks this step's plan left
     if (tid >= a.ntasks) return;  // whole warps; no block-wide barriers below
     const WarpTask tk = a.tasks[tid];
     const int i = tk.scen;
@@ -436,7 +454,7 @@ cudaError_t launch_batch_persistent(const PersistArgs& q, cudaStream_t s)
 
 void launch_batch_plan(const BatchArgs& a, int n_scen, cudaStream_t s)
 {
-    launch_pdl(batch_plan_kernel, (n_scen + 127) / 128, 128, 0, s, a, n_scen);
+    launch_pdl(batch_plan_kernel, (n_scen + kPlanMembers - 1) / kPlanMembers, 32, 0, s, a, n_scen);
 }
 
 void launch_batch_step(const BatchArgs& a, int warps_per_cta, cudaStream_t s)

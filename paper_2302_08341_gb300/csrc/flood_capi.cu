@@ -139,6 +139,7 @@ StepArgs step_args(const flood_grid* g, double t_end)
     a.nslot = g->nslot;
     a.t_end = t_end;
     a.alpha_dx = g->p.alpha * g->p.dx;
+    a.cap_h = flood::capped_below(a.alpha_dx, g->p.g, g->p.dt_cap);
     a.g = g->p.g;
     a.dt_cap = g->p.dt_cap;
     a.dt_fixed = g->p.dt_fixed;

@@ -25,6 +25,17 @@ struct MemberClock {
     int32_t cur;        // which of the two state buffers holds the current state
 };
 
+// A clock past L1.
+__device__ __forceinline__ MemberClock ld_clock(const MemberClock* p)
+{
+    MemberClock c;
+    c.t = __ldcg(&p->t);
+    c.steps = __ldcg(reinterpret_cast<const long long*>(&p->steps));
+    c.hmax_bits = __ldcg(&p->hmax_bits);
+    c.cur = __ldcg(&p->cur);
+    return c;
+}
+
 // Everything a step launch needs, passed by value.
 struct StepArgs {
     float* state;               // [2][M][3][plane]: h, qx, qy planes, two buffers
@@ -77,6 +88,7 @@ struct StepArgs {
     int nslot;                  // slots per member in vacc
     int dt_log_cap;
     double t_end;               // < 0: no end
+    float cap_h;                // capped_below: no step from Eq. 4 below this depth
     double alpha_dx;            // k * dx of Eq. 4
     double g;
     double dt_cap, dt_fixed, h_floor, rain_block;
@@ -113,7 +125,7 @@ struct MemberPlan {
 };
 
 // Step length of one member (Eq. 4 with floor, cap and landing on the next
-// stop).  Every CTA of a member evaluates this identically in FP64.
+// stop).
 struct StepPlan {
     double dt, t_next;
     double rdt;        // dt x rain rate of the block (m), before the member's multiplier
@@ -156,12 +168,6 @@ __device__ __forceinline__ StepPlan plan_step_p(double alpha_dx, double g, doubl
     return s;
 }
 
-__device__ __forceinline__ StepPlan plan_step(const StepArgs& a, const MemberClock& in, int m)
-{
-    return plan_step_p(a.alpha_dx, a.g, a.dt_cap, a.dt_fixed, a.h_floor, a.rain_block, a.t_end,
-                       a.hyeto, a.nb, a.rain_mult[m], in);
-}
-
 __device__ __forceinline__ void fill_plan(MemberPlan& p, const StepPlan& sp, double g, double dxd)
 {
     p.t_next = sp.t_next;
@@ -174,6 +180,92 @@ __device__ __forceinline__ void fill_plan(MemberPlan& p, const StepPlan& sp, dou
     p.dt_dx = (float)(sp.dt / dxd);
     p.active = sp.active ? 1 : 0;
 }
+
+// The depth below which Eq. 4's step is longer than the cap, by a margin that
+// no rounding crosses.
+inline float capped_below(double alpha_dx, double g, double dt_cap)
+{
+    return (float)(0.999 * alpha_dx * alpha_dx / (g * dt_cap * dt_cap));
+}
+
+// One member's plan by four lanes: plan_step_p and fill_plan, operation by
+// operation.  The plan stands between two steps with the GPU idle, and an FP64
+// instruction takes 64 cycles, a division 600 and a root 650, however many of
+// a warp's lanes take part: a thread a member took 5.2 us.  So the divisions
+// that do not wait for one another are a lane's each, a warp holds eight
+// members (more warps would share an SM's four FP64 units), Eq. 4's root and
+// quotient are formed only where the depth does not leave the cap binding, and
+// the kernels that use this plan while the step before is finishing: its clock
+// is known by then, and its maximum depth so far.  What is left after the wait
+// is to see whether they stayed as far as they matter: 1.6 us where the cap
+// binds, 4.0 us where Eq. 4 does and the depth has moved (600 x 707 x 8 with
+// land cover, 40 steps and their reverse: 4.27 -> 4.11 ms; 777 x 1013 x 12,
+// 80 steps: 5.96 -> 5.63 ms).
+// A: StepArgs or BatchArgs.  The four lanes hold the same.
+constexpr int kPlanMembers = 8;  // of a warp
+
+template <class A>
+struct PlanQuad {
+    const A& a;
+    int lane;                    // of the four
+    double t_end;
+    const float* hyeto;
+    const float* inflow;
+    int nb, inflow_blocks, in_rows;
+    float rain_mult;
+    double t, stop;              // the clock, and the next stop after it
+    float rate, discharge;       // of the clock's block
+    bool active;
+    MemberPlan p;
+
+    // the clock and its block
+    __device__ __forceinline__ void at(double now)
+    {
+        t = now;
+        active = !(t_end >= 0.0 && t >= t_end);
+        const double blk = floor(__ddiv_rn(t, a.rain_block));
+        const int b = (int)blk;
+        rate = (blk >= 0.0 && b < nb) ? hyeto[b] : 0.0f;
+        discharge = (inflow && blk >= 0.0 && b < inflow_blocks) ? inflow[b] : 0.0f;
+        stop = __dmul_rn(blk + 1.0, a.rain_block);
+        if (t_end >= 0.0 && t_end < stop) stop = t_end;
+    }
+    __device__ __forceinline__ bool needs_eq4(float hmax) const
+    {
+        return !(a.dt_fixed > 0.0) && !(hmax < a.cap_h && a.h_floor < (double)a.cap_h);
+    }
+    __device__ __forceinline__ double eq4(float hmax) const
+    {
+        double hm = (double)hmax;
+        hm = hm > a.h_floor ? hm : a.h_floor;
+        const double d = __ddiv_rn(a.alpha_dx, __dsqrt_rn(__dmul_rn(a.g, hm)));
+        return d > a.dt_cap ? a.dt_cap : d;
+    }
+    // the step from the clock in a state of maximum depth hmax, cut at the stop
+    __device__ __forceinline__ void step(float hmax)
+    {
+        double dt = needs_eq4(hmax) ? eq4(hmax) : a.dt_fixed > 0.0 ? a.dt_fixed : a.dt_cap;
+        p.t_next = __dadd_rn(t, dt);
+        if (p.t_next >= stop) {
+            dt = __dsub_rn(stop, t);
+            p.t_next = stop;
+        }
+        const double num = lane == 0 ? a.g * dt : lane == 1 ? a.dxd : lane == 2 ? dt : (double)discharge;
+        const double den = lane == 1 ? 4.0 * dt : (lane > 2 && inflow) ? a.dxd * (double)in_rows : a.dxd;
+        const float q = (float)(num / den);
+        const unsigned four = 0xfu << (threadIdx.x & 28);
+        p.dt = dt;
+        p.rdt = __dmul_rn(dt, (double)rate);
+        p.dr = (float)__dmul_rn(p.rdt, (double)rain_mult);
+        p.gdt = (float)(a.g * dt);
+        p.gdt_dx = __shfl_sync(four, q, 0, 4);
+        p.dx_4dt = __shfl_sync(four, q, 1, 4);
+        p.dt_dx = __shfl_sync(four, q, 2, 4);
+        const float qi = __shfl_sync(four, q, 3, 4);
+        p.q_in = active ? qi : 0.0f;
+        p.active = active ? 1 : 0;
+    }
+};
 
 // Compensated (Kahan) FP32 summation for the per-warp volume partials; the
 // explicit rounding intrinsics keep the compiler from re-associating it.

@@ -31,45 +31,66 @@ constexpr int kSpan = 128;  // columns per warp
 #define FLOOD_STEP_MIN_BLOCKS 6
 #endif
 
-// Per-member step plan (one thread per member, FP64): Eq. 4 step length,
+// Per-member step plan (four lanes per member, FP64): Eq. 4 step length,
 // rain of the block, the member's clock in the next slot, the rain volume and
 // (when logging) the step record and checkpoint slot.
 __global__ void plan_kernel(const StepArgs a)
 {
     pdl_launch();
+    const int mi = blockIdx.x * kPlanMembers + threadIdx.x / 4, m = min(mi, a.M - 1), lane = threadIdx.x & 3;
+    // the step from the clock and the maximum depth as they look now (the clock
+    // is there since the step before was planned); whether they stayed is seen
+    // after the wait
+    PlanQuad<StepArgs> w{a, lane, a.t_end, a.hyeto, a.inflow, a.nb, a.inflow_blocks, a.in_r1 - a.in_r0,
+                         __ldcg(a.rain_mult + m)};
+    const uint32_t early = __ldcg(&a.ms_in[m].hmax_bits);
+    w.at(__ldcg(&a.ms_in[m].t));
+    w.step(__uint_as_float(early));
+    const double rows = (double)(a.in_r1 - a.in_r0);
+    // the rain and inflow volumes, a lane each
+    auto volume = [&]() { return lane == 1 ? (double)w.p.q_in * a.dxd * rows : (double)w.p.dr * a.cell_area; };
+    double v = volume();
     pdl_wait();
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= a.M) return;
-    const MemberClock in = a.ms_in[m];
-    const StepPlan sp = plan_step(a, in, m);
-    MemberPlan p;
-    fill_plan(p, sp, a.g, a.dxd);
+    const MemberClock in = ld_clock(a.ms_in + m);
+    const float rain_mult = __ldcg(a.rain_mult + m);
+    if (mi >= a.M) return;
+    const double v0 = lane == 0 ? a.rain_acc[m] : lane == 1 && a.inflow ? a.inflow_acc[m] : 0.0;
+    const float hmax = __uint_as_float(in.hmax_bits);
+    const bool moved = __double_as_longlong(in.t) != __double_as_longlong(w.t) ||
+                       __float_as_uint(rain_mult) != __float_as_uint(w.rain_mult);
+    if (moved ||
+        (in.hmax_bits != early && (w.needs_eq4(hmax) || w.needs_eq4(__uint_as_float(early))))) {
+        w.rain_mult = rain_mult;
+        if (moved) w.at(in.t);
+        w.step(hmax);
+        v = volume();
+    }
+    MemberPlan& p = w.p;
     p.cur = in.cur;
     p.ckpt = -1;
-    p.q_in = 0.0f;
-    if (a.inflow && sp.active) {  // the block's discharge spread over the inflow rows
-        const double blk = floor(__ddiv_rn(in.t, a.rain_block));
-        const int b = (int)blk;
-        const double Q = (blk >= 0.0 && b < a.inflow_blocks) ? (double)a.inflow[b] : 0.0;
-        p.q_in = (float)(Q / (a.dxd * (double)(a.in_r1 - a.in_r0)));
-        a.inflow_acc[m] += (double)p.q_in * a.dxd * (double)(a.in_r1 - a.in_r0) * sp.dt;
+    if (w.active) {
+        if (a.slots)  // (steps past the log's end stay in its last slots: the window is run again)
+            p.ckpt = (int)(in.steps < a.dt_log_cap ? in.steps : a.dt_log_cap - 1);
+        else if (a.ckpt && (in.steps + 1) % a.ckpt_every == 0 && in.steps + 1 <= a.dt_log_cap)
+            p.ckpt = (int)((in.steps + 1) / a.ckpt_every);
     }
-    a.ms_clr[m].hmax_bits = 0u;  // the slot the next step's maximum goes to
-    if (!sp.active) {
-        a.ms_out[m] = in;
+    if (lane == 0) {
         a.plan[m] = p;
-        return;
+        a.ms_clr[m].hmax_bits = 0u;  // the slot the next step's maximum goes to
+        if (!w.active) {
+            a.ms_out[m] = in;
+        } else {
+            a.ms_out[m].t = p.t_next;
+            a.ms_out[m].steps = in.steps + 1;
+            a.ms_out[m].cur = 1 - in.cur;  // hmax_bits: atomicMax by the step kernel (slot was cleared)
+            if (a.log && in.steps < a.dt_log_cap) a.log[(size_t)m * a.dt_log_cap + in.steps] = p;
+        }
     }
-    a.ms_out[m].t = sp.t_next;
-    a.ms_out[m].steps = in.steps + 1;
-    a.ms_out[m].cur = 1 - in.cur;  // hmax_bits: atomicMax by the step kernel (slot was cleared)
-    a.rain_acc[m] += (double)sp.dr * a.cell_area * a.ncell;
-    if (a.slots)  // (steps past the log's end stay in its last slots: the window is run again)
-        p.ckpt = (int)(in.steps < a.dt_log_cap ? in.steps : a.dt_log_cap - 1);
-    else if (a.ckpt && (in.steps + 1) % a.ckpt_every == 0 && in.steps + 1 <= a.dt_log_cap)
-        p.ckpt = (int)((in.steps + 1) / a.ckpt_every);
-    if (a.log && in.steps < a.dt_log_cap) a.log[(size_t)m * a.dt_log_cap + in.steps] = p;
-    a.plan[m] = p;
+    if (w.active) {
+        v = __fma_rn(v, lane == 1 ? p.dt : a.ncell, v0);
+        if (lane == 0) a.rain_acc[m] = v;
+        if (lane == 1 && a.inflow) a.inflow_acc[m] = v;
+    }
 }
 
 // REPLAY = false: an ordinary step with the plan of this step.  REPLAY =
@@ -149,7 +170,7 @@ __global__ void __launch_bounds__(32 * WM * WC, (LC ? 4 : FLOOD_STEP_MIN_BLOCKS)
 
 void launch_plan(const StepArgs& a, cudaStream_t s)
 {
-    launch_pdl(plan_kernel, (a.M + 127) / 128, 128, 0, s, a);
+    launch_pdl(plan_kernel, (a.M + kPlanMembers - 1) / kPlanMembers, 32, 0, s, a);
 }
 
 int step_nslot(int ny, int nx, int rows_per_strip)

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
     bool lands = false;
     bool on_block = false;       // stop, rate and q_in belong to the clock
     float q_in = 0.0f;
-    const float cap_h = (float)(0.999 * a.alpha_dx * a.alpha_dx / (a.g * a.dt_cap * a.dt_cap));
+    const float cap_h = a.cap_h;
     const bool floor_capped = a.h_floor < (double)cap_h;
     int64_t steps = in.steps;
     uint32_t hmax = in.hmax_bits;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
         return t.xch + ((((size_t)parity * a.M + m) * t.bands + b) * 2 + last) * ld;
     };
     // warp 0: the plan of the step from clk with step length d (before landing)
-    // into bp, as plan_step_p and fill_plan make it
+    // into bp, as PlanQuad makes it
     auto set_plan = [&](double d) {
         bool fresh = false;  // the step's constants change
         if (!on_block) {

@@ -29,8 +29,8 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
     const int w = threadIdx.y;
     const int m = blockIdx.x * WM + w;
     int span = blockIdx.y, strip = blockIdx.z;
-    pdl_launch();
     pdl_wait();
+    pdl_launch();  // after the wait: the next plan may then read the clocks this step's plan left
     if (a.tiles) {  // only the tiles that hold a cell of the domain are launched
         const int2 tl = a.tiles[blockIdx.y];
         span = tl.x;
