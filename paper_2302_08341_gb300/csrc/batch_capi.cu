@@ -122,7 +122,7 @@ int build_tasks(flood_batch* b)
     if (!b->launch_fixed) {  // as the ensemble's automatic strip height
         int64_t rows = 0;
         for (int e = 0; e < b->S; ++e) rows += (int64_t)b->ny[e] * ((b->nx[e] + kSpan - 1) / kSpan);
-        b->rows_per_strip = flood::strip_rows(rows, b->n_sm * 20);
+        b->rows_per_strip = flood::strip_rows(rows, b->n_sm, false);
     }
     b->tasks.clear();
     b->slot0.assign(b->S, 0);

@@ -513,6 +513,6 @@ int encode_map_3d_u8(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d
 int step_nslot(int ny, int nx, int rows_per_strip);
 // Rows per strip for a step over `warp_rows` rows of 128-column spans (of all
 // members) on a GPU that holds `warps` of the kernel's warps at a time.
-int strip_rows(int64_t warp_rows, int warps);
+int strip_rows(int64_t warp_rows, int n_sm, bool track);
 
 }  // namespace flood

@@ -170,6 +170,7 @@ int dalloc(flood_grid* g, T** p, size_t count)
     return dalloc_bytes(g, reinterpret_cast<void**>(p), sizeof(T) * (count ? count : 1));
 }
 StepArgs step_args(const flood_grid* g, double t_end);
+int auto_rows(flood_grid* g);   // the automatic strip height, with or without tracked maxima
 int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s);
 int read_clocks(flood_grid* g, std::vector<MemberClock>& out, cudaStream_t s);
 // Whether the next steps run on the chip (step_resident.cu).

@@ -564,7 +564,7 @@ extern "C" int flood_track_max_depth(flood_grid* g, int on, void* stream)
     if (!on) {
         CK(g, cudaStreamSynchronize(s));
         g->track_max = false;
-        return FLOOD_OK;
+        return flood::auto_rows(g);
     }
     if (!g->hmax_field) {
         int rc = flood::dalloc(g, &g->hmax_field, (size_t)g->M * g->plane);
@@ -578,7 +578,7 @@ extern "C" int flood_track_max_depth(flood_grid* g, int on, void* stream)
     g->launches++;
     CK(g, cudaGetLastError());
     g->track_max = true;
-    return FLOOD_OK;
+    return flood::auto_rows(g);
 }
 
 extern "C" int flood_get_max_depth(flood_grid* g, int member, float* out, void* stream)

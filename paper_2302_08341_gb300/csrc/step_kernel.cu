@@ -187,15 +187,19 @@ int step_nslot(int ny, int nx, int rows_per_strip)
 //    strips (1024 x 1024 x 1: 3 rows 14, 8 rows 16.5; 2000 x 2000 x 1: 12 rows
 //    32, 4 rows 34; 600 x 707 x 8: 12 rows 28, 8 rows (1.2 rounds) 33);
 //  - a few rounds of strips: 12 rows (1000 x 1000 x 16: 12 rows 83, 32 rows 96,
-//    4 rows 100; 2000 x 2000 x 8: 145, 148, 179);
-//  - from about eight rounds of 24 rows on, 24 (2000 x 2000 x 96: 24 rows 1420,
-//    64 rows 1533, 12 rows 1486; neighbouring strips' halo rows then still
-//    meet in L2).
-int strip_rows(int64_t warp_rows, int warps)
+//    4 rows 100; 2000 x 2000 x 8: 145, 148, 179); where the maxima are tracked
+//    and an SM holds 16 warps, 9 (777 x 1013 x 12: 59.8, 12 rows 62.2; 1000 x
+//    1000 x 24: 129.5, 132.5);
+//  - from about five rounds of 24 rows on, 24 (2000 x 2000 x 96: 24 rows 1420,
+//    64 rows 1533, 12 rows 1486; 1200 x 1310 x 32 with land cover: 201, 217 (48
+//    rows), 206; neighbouring strips' halo rows then still meet in L2).
+int strip_rows(int64_t warp_rows, int n_sm, bool track)
 {
+    const int64_t warps = (int64_t)n_sm * (track ? 16 : 20);
     const int64_t one = (warp_rows + warps - 1) / warps;  // rows a warp when all are resident
-    if (one <= 12) return (int)(one < 1 ? 1 : one);
-    return warp_rows >= (int64_t)warps * 24 * 8 ? 24 : 12;
+    const int few = track ? 9 : 12;
+    if (one <= few) return (int)(one < 1 ? 1 : one);
+    return warp_rows >= warps * 24 * 5 ? 24 : few;
 }
 
 // members_per_cta: warps of one CTA hold this many members of the same span
