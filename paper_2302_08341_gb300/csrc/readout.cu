@@ -18,7 +18,8 @@ namespace flood {
 namespace {
 
 // Rows of the current h, qx, qy planes (blockIdx.y) without their padding.
-// VEC: rows of whole float4s in 16-byte aligned arrays.
+// VEC: rows of whole float4s in 16-byte aligned arrays; otherwise the rows of
+// the output start anywhere, and a thread has eight words in flight instead.
 template <bool VEC>
 __global__ void read_state_kernel(const float* __restrict__ state, size_t buffer, const MemberClock* clk, int ny,
                                   int nx, int ld, size_t plane, float* h, float* qx, float* qy)
@@ -29,11 +30,21 @@ __global__ void read_state_kernel(const float* __restrict__ state, size_t buffer
     for (int r = blockIdx.x * blockDim.y + threadIdx.y; r < ny; r += gridDim.x * blockDim.y) {
         const float* p = src + (size_t)r * ld;
         float* o = out + (size_t)r * nx;
-        if (VEC)
+        if (VEC) {
             for (int c = 4 * threadIdx.x; c < nx; c += 4 * blockDim.x)
                 *reinterpret_cast<float4*>(o + c) = *reinterpret_cast<const float4*>(p + c);
-        else
-            for (int c = threadIdx.x; c < nx; c += blockDim.x) o[c] = p[c];
+            continue;
+        }
+        constexpr int kWords = 8;
+        for (int c = threadIdx.x; c < nx; c += kWords * blockDim.x) {
+            float v[kWords];
+#pragma unroll
+            for (int i = 0; i < kWords; ++i)
+                if (c + i * (int)blockDim.x < nx) v[i] = __ldg(p + c + i * blockDim.x);
+#pragma unroll
+            for (int i = 0; i < kWords; ++i)
+                if (c + i * (int)blockDim.x < nx) o[c + i * blockDim.x] = v[i];
+        }
     }
 }
 
@@ -102,18 +113,27 @@ bool pageable(const void* p)
     return at.type == cudaMemoryTypeUnregistered;
 }
 
-// bytes at p, inside one allocation of the current device and aligned for floats.
-static bool kernel_may_write(const void* p, size_t bytes)
+// An allocation of the current device (size 0: none).
+struct Allocation {
+    uintptr_t base = 0;
+    size_t size = 0;
+    bool holds(const void* p, size_t bytes) const
+    {
+        const uintptr_t q = reinterpret_cast<uintptr_t>(p);
+        return q >= base && q - base <= size && bytes <= size - (q - base);
+    }
+};
+
+static Allocation allocation_of(const void* p)
 {
+    Allocation r;
     cudaPointerAttributes at{};
     int dev = 0;
-    if ((reinterpret_cast<uintptr_t>(p) & 3) != 0 || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return r;
     }
-    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
-    // (a copy refuses an array that is too short, a kernel would write past it)
+    if (at.type != cudaMemoryTypeDevice || at.device != dev) return r;
     static const PFN_cuMemGetAddressRange_v3020 range = [] {
         void* fn = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -124,8 +144,11 @@ static bool kernel_may_write(const void* p, size_t bytes)
     }();
     CUdeviceptr base = 0;
     size_t size = 0;
-    const CUdeviceptr q = reinterpret_cast<CUdeviceptr>(p);
-    return range && range(&base, &size, q) == CUDA_SUCCESS && q - base <= size && bytes <= size - (q - base);
+    if (range && range(&base, &size, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS) {
+        r.base = (uintptr_t)base;
+        r.size = size;
+    }
+    return r;
 }
 
 bool capturing(cudaStream_t s)
@@ -142,10 +165,15 @@ bool read_by_kernel(const float* h, const float* qx, const float* qy, size_t n, 
 {
     const float* out[3] = {h, qx, qy};
     bool any = false;
+    Allocation in;
     for (int i = 0; i < 3; ++i) {
         if (!out[i]) continue;
         any = true;
-        if (!kernel_may_write(out[i], sizeof(float) * n)) return false;
+        if ((reinterpret_cast<uintptr_t>(out[i]) & 3) != 0) return false;
+        // the whole array inside one allocation (a copy refuses an array that
+        // is too short, a kernel would write past it)
+        if (!in.holds(out[i], sizeof(float) * n)) in = allocation_of(out[i]);
+        if (!in.holds(out[i], sizeof(float) * n)) return false;
         for (int j = 0; j < i; ++j)
             if (out[j] && out[i] < out[j] + n && out[j] < out[i] + n) return false;
     }
