@@ -380,19 +380,26 @@ __global__ void __launch_bounds__(32 * kProdWarps, prod_ctas(MT))
             // per level the first key whose cumulative weight reaches it and
             // its ord (none reached: the largest value)
             uint32_t kc[kLevelsPerPass], oq[kLevelsPerPass];
+            int pos[kLevelsPerPass];  // the key's place in the column; W: the weight before it
 #pragma unroll
             for (int q = 0; q < kLevelsPerPass; ++q) {
                 kc[q] = 0u;
                 oq[q] = omax;
-                if (q >= a.n_levels) continue;
+                pos[q] = -1;          // none reached
+                if (q >= a.n_levels || P < a.A[q]) continue;
                 const uint32_t* kb = kcol + nb[q] * 32;
+                long long sum = W[q];
 #pragma unroll
                 for (int k = 0; k < kBlock; ++k) {
                     const uint32_t kk = kb[k * 32];
-                    if (W[q] < a.A[q]) kc[q] = kk;
-                    W[q] += weight(kk);
+                    if (sum < a.A[q]) {
+                        kc[q] = kk;
+                        pos[q] = nb[q] + k;
+                        W[q] = sum;
+                    }
+                    sum += weight(kk);
                 }
-                if (P >= a.A[q]) oq[q] = (kc[q] >> 7) + omin;
+                oq[q] = (kc[q] >> 7) + omin;
             }
             if (!exact) {
                 // a lane with shifted places: its keys order the members up
@@ -403,47 +410,65 @@ __global__ void __launch_bounds__(32 * kProdWarps, prod_ctas(MT))
                 // (the stage holds the keys now; the group's lines are still
                 // in L2)
                 const float* fc = a.field + (size_t)r * a.ld + c;
-                if (a.th_ord > omin && a.th_ord <= omax) {
+                auto value = [&](uint32_t kk) {  // ord of a member's value
+                    return ord_of(fc[(size_t)min(kk & 0x7Fu, (uint32_t)a.M - 1u) * a.plane]);
+                };
+                if (a.exceed && a.th_ord > omin && a.th_ord <= omax) {
                     const uint32_t pth = (a.th_ord - omin) >> sh;
-                    const int end = below_key((pth + 1) << 7);
-                    for (int p = below_key(pth << 7); p < end; ++p) {
-                        const uint32_t id = kcol[p * 32] & 0x7Fu;  // a real member: < M
-                        if (id < (uint32_t)a.M && ord_of(fc[(size_t)id * a.plane]) < a.th_ord) ex -= weight(id);
-                    }
+                    for (int p = nth; p < a.M && kcol[p * 32] >> 7 == pth; ++p)
+                        if (value(kcol[p * 32]) < a.th_ord) ex -= weight(kcol[p * 32]);
                 }
+                unsigned shared = 0u;  // levels whose key shares its place
 #pragma unroll
                 for (int q = 0; q < kLevelsPerPass; ++q) {
-                    if (q >= a.n_levels || P < a.A[q]) continue;
+                    if (pos[q] < 0) continue;
                     const uint32_t pl = kc[q] >> 7;
-                    const int plo = below_key(pl << 7), phi = below_key((pl + 1) << 7);
-                    if (phi - plo == 1) {  // the key's member is alone in its place
-                        oq[q] = ord_of(fc[(size_t)min(kc[q] & 0x7Fu, (uint32_t)a.M - 1u) * a.plane]);
-                        continue;
+                    oq[q] = value(kc[q]);
+                    if ((pos[q] > 0 && kcol[(pos[q] - 1) * 32] >> 7 == pl) ||
+                        (pos[q] + 1 < MT && kcol[(pos[q] + 1) * 32] >> 7 == pl))
+                        shared |= 1u << q;
+                }
+#pragma unroll 1
+                for (; shared; shared &= shared - 1u) {
+                    const int q = __ffs(shared) - 1;
+                    uint32_t pl = kc[0] >> 7;
+                    int plo = pos[0];
+                    long long before = W[0];
+#pragma unroll
+                    for (int i = 1; i < kLevelsPerPass; ++i)
+                        if (i == q) {
+                            pl = kc[i] >> 7;
+                            plo = pos[i];
+                            before = W[i];
+                        }
+                    // the members that share the place, the weight before
+                    // them, their range
+                    int phi = plo + 1;
+                    for (; plo > 0 && kcol[(plo - 1) * 32] >> 7 == pl; --plo) before -= weight(kcol[(plo - 1) * 32]);
+                    while (phi < MT && kcol[phi * 32] >> 7 == pl) ++phi;
+                    uint32_t v = kPad, hi = 0u;
+                    for (int p = plo; p < phi; ++p) {
+                        const uint32_t o = value(kcol[p * 32]);
+                        v = min(v, o);
+                        hi = max(hi, o);
                     }
-                    // members that share the place: their range, then
                     // candidates in increasing order against the exact
                     // weighted distribution function (lower places hold
                     // smaller values, higher places larger ones)
-                    uint32_t lo = kPad, hi = 0u;
-                    for (int p = plo; p < phi; ++p) {
-                        const uint32_t id = min(kcol[p * 32] & 0x7Fu, (uint32_t)a.M - 1u);
-                        const uint32_t o = ord_of(fc[(size_t)id * a.plane]);
-                        lo = min(lo, o);
-                        hi = max(hi, o);
-                    }
-                    uint32_t v = lo;
-                    for (int it = 0; it < a.M && v != hi; ++it) {
-                        long long W = 0;
-                        uint32_t nxt = hi;
-                        for (int j = 0; j < a.M; ++j) {
-                            const uint32_t o = ord_of(fc[(size_t)j * a.plane]);
-                            if (o <= v) W += weight((uint32_t)j);
-                            else nxt = min(nxt, o);
+                    while (v != hi) {
+                        long long sum = before;
+                        uint32_t next = hi;
+                        for (int p = plo; p < phi; ++p) {
+                            const uint32_t o = value(kcol[p * 32]);
+                            if (o <= v) sum += weight(kcol[p * 32]);
+                            else next = min(next, o);
                         }
-                        if (W >= a.A[q]) break;
-                        v = nxt;
+                        if (sum >= a.A[q]) break;
+                        v = next;
                     }
-                    oq[q] = v;
+#pragma unroll
+                    for (int i = 0; i < kLevelsPerPass; ++i)
+                        if (i == q) oq[i] = v;
                 }
             }
             // the shifted lanes have read the keys: the next copy may overwrite them
