@@ -205,10 +205,10 @@ __host__ __device__ constexpr int prod_stage_bytes() { return (MT * 32 * 4 + 127
 // rate; 16-bit pairs run at the same rate a register, but nine bits of place
 // tie too often), and with unequal weights the fetching of instructions.  The
 // pass over every key for every level took 1920 instructions a cell of 4900;
-// by blocks it takes 900.  2000 x 2000 x 96, unequal weights: 1.55 -> 1.21 ms.
+// by blocks it takes 900.  2000 x 2000 x 96, unequal weights: 1.55 -> 1.09 ms.
 // Slots come in steps of 8 to 16 members (LO: the step below, whose slots need
 // no test for padding) where 32, 64, 96 and 128 were: 1000 x 1000 cells
-// with 8 members 130 -> 73 us, 40 members 251 -> 159 us, 128 721 -> 601 us;
+// with 8 members 130 -> 73 us, 40 members 251 -> 159 us, 128 721 -> 452 us;
 // equal weights 73 -> 49, 126 -> 104, 337 -> 309 us.
 //
 // Every wait is bounded: one that gives up records FLOOD_ERR_TIMEOUT in the
