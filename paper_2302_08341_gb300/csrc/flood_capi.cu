@@ -404,6 +404,13 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
             const int rc = ensure_graph(g, t_end);
             if (rc) return rc;
         }
+        // a resident launch costs about 5 us beside its steps (256 x 256 x 1,
+        // 300 steps: runs of 24 833 us, of up to 240 753 us); longer ones
+        // would hold the SMs for milliseconds
+        while (res && count - i >= 11 * kGraphSteps) {
+            const int rc = some(10 * kGraphSteps);
+            if (rc) return rc;
+        }
         while (count - i >= kGraphSteps) {
             if (!graphs) {
                 const int rc = some(kGraphSteps);

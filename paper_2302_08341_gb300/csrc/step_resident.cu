@@ -3,7 +3,7 @@
 // Where a member's state fits in shared memory, reading and writing it through
 // L2 every step and launching two kernels per step costs more than the step:
 // a 256 x 256 model took 10.6 us per step, of which its arithmetic is well
-// under one.  Here one cooperative launch runs up to 24 steps.  Every member
+// under one.  Here one cooperative launch runs up to 240 steps.  Every member
 // is cut into bands of whole rows, one CTA each, which keep h, qx, qy, the bed
 // and the roughness in shared memory from the first step to the last; a step
 // exchanges a row of depths with the bands above and below and the bands'

@@ -17,7 +17,7 @@ def capi():
     return require_gpu()
 
 
-def _run(capi, ny, nx, M, march, land=False, track=False, inflow=False, deep=False, steps=(1, 24, 31)):
+def _run(capi, ny, nx, M, march, land=False, track=False, inflow=False, deep=False, steps=(1, 24, 31, 290)):
     terr = synth.make_terrain(ny, nx, seed=91)
     rm, sc = synth.ensemble_prior(91, M)
     rng = np.random.default_rng(91)
@@ -36,7 +36,7 @@ def _run(capi, ny, nx, M, march, land=False, track=False, inflow=False, deep=Fal
             g.set_launch(8, 1)
         for n in steps:
             g.step(n)
-        g.advance_to(200.0)
+        g.advance_to(450.0)
         out = [np.array(g.get_state(m)) for m in range(M)]
         if track:
             out += [g.max_depth(m) for m in range(M)]
