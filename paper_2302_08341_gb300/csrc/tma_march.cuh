@@ -228,12 +228,31 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         }
         const float* R = row_ptr(sC);
         const float* P = R + x0;
-        const Quad hC = ld_quad(P), zC = ld_quad(P + kZ), uC = bounds(hC);
+        const Quad hC = ld_quad(P), zC = ld_quad(P + kZ);
         if (!LC) nC = ld_quad(P + kN);
         // east links: cells 0 1 2 3 with 1 2 3 and the next lane's first,
         // straight from the tile
-        const Quad qx = ld_quad(P + kQx);
+        const Quad qx = ld_quad(P + kQx), qy = ld_quad(P + kQy);
         const float hE = P[4], zE = P[kZ + 4], nE = LC ? class_n(P + kN + 4) : P[kN + 4];
+        // the link west of the span, from the tile's halo: every lane computes
+        // it from lane 0's addresses, lane 0 keeps it
+        float hW = 0.0f, zW = 0.0f, nW = 0.0f, qWo = 0.0f;
+        if (c0 > 0) {
+            hW = R[3];
+            zW = R[kZ + 3];
+            nW = LC ? class_n(R + kN + 3) : R[kN + 3];
+            qWo = R[kQx + 3];
+        }
+        uint4 codes;
+        if (LC) codes = *reinterpret_cast<const uint4*>(P + kN);
+        Quad hmo;
+        if (TRACK_MAX) hmo = ld_quad(R + kTmaHmOff / 4 + 4 * lane);
+        // with tracked maxima (16 warps an SM and registers to spare) the row
+        // goes into registers whole and its stage takes a later row before the
+        // arithmetic (777 x 1013 x 12, 80 steps: 5.55 -> 5.39 ms); with 20 warps
+        // that costs more than it hides (1000 x 1000 x 16: 5.76 -> 6.22 ms)
+        if (TRACK_MAX) release(r, sC);
+        const Quad uC = bounds(hC);
         Quad qE, qS, nS;
         qE.a = link2_q<LIM>(hC.a, zC.a, make_float2(hC.a.y, hC.b.x), make_float2(zC.a.y, zC.b.x), qx.a,
                             make_float2(__fadd_rn(nC.a.x, nC.a.y), __fadd_rn(nC.a.y, nC.b.x)), uC.a,
@@ -241,23 +260,20 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         qE.b = link2_q<LIM>(hC.b, zC.b, make_float2(hC.b.y, hE), make_float2(zC.b.y, zE), qx.b,
                             make_float2(__fadd_rn(nC.b.x, nC.b.y), __fadd_rn(nC.b.y, nE)), uC.b,
                             make_float2(uC.b.y, __fmul_rn(hE, k.dx_4dt)), lk2);
-        // the link west of the span, from the tile's halo: every lane computes
-        // it from lane 0's addresses, lane 0 keeps it
         float qH = (r >= k.in_r0 && r < k.in_r1) ? k.q_in : 0.0f;  // west edge: wall or inflow
         if (c0 > 0)
-            qH = link_q<LIM>(R[3], R[kZ + 3], hC.a.x, zC.a.x, R[kQx + 3],
-                             __fmul_rn(s_half, __fadd_rn(LC ? class_n(R + kN + 3) : R[kN + 3], nC.a.x)), k);
+            qH = link_q<LIM>(hW, zW, hC.a.x, zC.a.x, qWo, __fmul_rn(s_half, __fadd_rn(nW, nC.a.x)), k);
         if (has_s) {
             const float* Q = row_ptr(sN) + x0;
             const Quad hS = ld_quad(Q);
             nS = quad_n(Q + kN);
-            qS = south_links(hC, zC, nC, uC, hS, ld_quad(Q + kZ), nS, bounds(hS), ld_quad(P + kQy));
+            qS = south_links(hC, zC, nC, uC, hS, ld_quad(Q + kZ), nS, bounds(hS), qy);
         } else {
             nS = nC;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 quad_at(qS, j) =
-                    south_out ? outflow_q<LIM>(quad_at(hC, j), P[kQy + j], __fmul_rn(s, quad_at(nC, j)), k)
+                    south_out ? outflow_q<LIM>(quad_at(hC, j), quad_at(qy, j), __fmul_rn(s, quad_at(nC, j)), k)
                               : 0.0f;
         }
         if (!full) {  // the span holds the grid's last column: its east link, and nothing past it
@@ -267,7 +283,7 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
                 if (cj >= nx - 1) {
                     quad_at(qE, j) =
                         (east_out && cj == nx - 1)
-                            ? outflow_q<LIM>(quad_at(hC, j), P[kQx + j], __fmul_rn(s, quad_at(nC, j)), k)
+                            ? outflow_q<LIM>(quad_at(hC, j), quad_at(qx, j), __fmul_rn(s, quad_at(nC, j)), k)
                             : 0.0f;
                     if (cj >= nx) quad_at(qS, j) = 0.0f;
                 }
@@ -294,8 +310,7 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
                     if (c + j >= nx) quad_at(hN, j) = 0.0f;
             }
         } else {
-            const uint4 q = *reinterpret_cast<const uint4*>(P + kN);
-            const uint32_t code[4] = {q.x, q.y, q.z, q.w};
+            const uint32_t code[4] = {codes.x, codes.y, codes.z, codes.w};
             const float net[4] = {na.x, na.y, nb.x, nb.y};
             float row_sink = 0.0f;  // the row's drained depth, compensated once per row
 #pragma unroll
@@ -346,9 +361,8 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
                 st_quad(pc + 2 * plane, qS);
             }
             if (TRACK_MAX) {
-                const Quad o = ld_quad(R + kTmaHmOff / 4 + 4 * lane);
-                *reinterpret_cast<float4*>(ph) = make_float4(fmaxf(o.a.x, hN.a.x), fmaxf(o.a.y, hN.a.y),
-                                                             fmaxf(o.b.x, hN.b.x), fmaxf(o.b.y, hN.b.y));
+                *reinterpret_cast<float4*>(ph) = make_float4(fmaxf(hmo.a.x, hN.a.x), fmaxf(hmo.a.y, hN.a.y),
+                                                             fmaxf(hmo.b.x, hN.b.x), fmaxf(hmo.b.y, hN.b.y));
             }
         }
         pd += ld;
@@ -357,7 +371,7 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         // march: this row's south links are the next row's north links
         qN = qS;
         if (LC) nC = nS;
-        release(r, sC);
+        if (!TRACK_MAX) release(r, sC);
         sC = sN;
         sN = (sN + 1) & (kNS - 1);
         if (sN == 0) phN ^= 1u;
