@@ -69,7 +69,7 @@ void free_ensemble(flood_grid* g)
     dfree(g->gnm); dfree(g->gn_out); dfree(g->gpart); dfree(g->seg_end); dfree(g->samp_step);
     dfree(g->samp_y); dfree(g->samp_d); dfree(g->samp_cells); dfree(g->closs);
     dfree(g->hmax_field); dfree(g->lc_n); dfree(g->lc_drain); dfree(g->dacc);
-    dfree(g->rs_words); dfree(g->rs_xch); dfree(g->rs_seq);
+    dfree(g->rs_words);
     g->rs_words = nullptr; g->rs_xch = nullptr; g->rs_seq = nullptr; g->rs_shape = {0, 0, 0};
     dfree(g->inflow_acc); dfree(g->lc_adj); dfree(g->lc_cgrad); dfree(g->gdpart); dfree(g->lc_dgrad);
     g->inflow_acc = nullptr; g->lc_adj = nullptr; g->lc_cgrad = nullptr; g->gdpart = nullptr;
@@ -251,18 +251,24 @@ bool steps_resident(const flood_grid* g)
     return resident_now(g, &sh);
 }
 
-// The buffers of steps in that shape (allocates: not while capturing).
-static int resident_buffers(flood_grid* g, const ResidentShape& sh)
+// The buffers of steps in that shape (allocates: not while capturing), one
+// block: band words, exchange rows, step numbers.  Cleared on the steps' own
+// stream: a clear on the default stream is not ordered before a kernel on a
+// non-blocking one, which would read words not yet cleared or lose words that
+// its bands have published.
+static int resident_buffers(flood_grid* g, const ResidentShape& sh, cudaStream_t s)
 {
     if (g->rs_words && g->rs_shape.bands >= sh.bands) return FLOOD_OK;
-    const size_t n = (size_t)2 * g->M * sh.bands;
-    int rc;
-    if ((rc = dalloc(g, &g->rs_words, n)) || (rc = dalloc(g, &g->rs_xch, n * 2 * g->ld)) ||
-        (rc = dalloc(g, &g->rs_seq, g->M)))
-        return rc;
-    CK(g, cudaMemset(g->rs_words, 0, sizeof(unsigned long long) * n));
-    CK(g, cudaMemset(g->rs_xch, 0, sizeof(unsigned long long) * n * 2 * g->ld));
-    CK(g, cudaMemset(g->rs_seq, 0, sizeof(uint32_t) * g->M));
+    const size_t n = (size_t)2 * g->M * sh.bands, rows = n * 2 * g->ld;
+    const size_t words = n + rows + ((size_t)g->M + 1) / 2;
+    g->rs_shape = {0, 0, 0};
+    g->rs_xch = nullptr;
+    g->rs_seq = nullptr;
+    const int rc = dalloc(g, &g->rs_words, words);
+    if (rc) return rc;
+    g->rs_xch = g->rs_words + n;
+    g->rs_seq = reinterpret_cast<uint32_t*>(g->rs_xch + rows);
+    CK(g, cudaMemsetAsync(g->rs_words, 0, sizeof(unsigned long long) * words, s));
     g->rs_shape = sh;
     return FLOOD_OK;
 }
@@ -377,7 +383,7 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
     ResidentShape sh;
     const bool res = resident_now(g, &sh);
     if (res) {
-        const int rc = resident_buffers(g, sh);
+        const int rc = resident_buffers(g, sh, s);
         if (rc) return rc;
     }
     // up to `n` steps, however they run

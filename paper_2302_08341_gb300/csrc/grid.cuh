@@ -46,7 +46,7 @@ struct flood_grid {
     bool launch_fixed = false;    // set by flood_set_launch
     // steps that stay on the chip (step_resident.cu)
     size_t smem_max = 0;          // shared memory a CTA may have
-    unsigned long long* rs_words = nullptr;  // band words, exchange rows, step numbers
+    unsigned long long* rs_words = nullptr;  // one block: band words, exchange rows, step numbers
     unsigned long long* rs_xch = nullptr;
     uint32_t* rs_seq = nullptr;
     flood::ResidentShape rs_shape{0, 0, 0};  // the shape the buffers were sized for
