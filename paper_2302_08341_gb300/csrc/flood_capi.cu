@@ -70,7 +70,7 @@ void free_ensemble(flood_grid* g)
     dfree(g->samp_y); dfree(g->samp_d); dfree(g->samp_cells); dfree(g->closs);
     dfree(g->hmax_field); dfree(g->lc_n); dfree(g->lc_drain); dfree(g->dacc);
     dfree(g->rs_words);
-    g->rs_words = nullptr; g->rs_xch = nullptr; g->rs_seq = nullptr; g->rs_shape = {0, 0, 0};
+    g->rs_words = nullptr; g->rs_xch = nullptr; g->rs_seq = nullptr;
     dfree(g->inflow_acc); dfree(g->lc_adj); dfree(g->lc_cgrad); dfree(g->gdpart); dfree(g->lc_dgrad);
     g->inflow_acc = nullptr; g->lc_adj = nullptr; g->lc_cgrad = nullptr; g->gdpart = nullptr;
     g->lc_dgrad = nullptr;
@@ -240,7 +240,8 @@ static int launch_one(flood_grid* g, double t_end, cudaStream_t s)
 // for that times or limits single step kernels.
 static bool resident_now(const flood_grid* g, ResidentShape* sh)
 {
-    if (g->engine != 1 || !g->maps_ok || g->profile || g->launch_fixed || g->wait_budget >= 0) return false;
+    if (!g->rs_words || g->engine != 1 || !g->maps_ok || g->profile || g->launch_fixed || g->wait_budget >= 0)
+        return false;
     *sh = resident_shape(g->ny, g->nx, g->M, g->n_sm, g->smem_max, g->track_max, g->lc_on);
     return sh->bands > 0;
 }
@@ -251,25 +252,25 @@ bool steps_resident(const flood_grid* g)
     return resident_now(g, &sh);
 }
 
-// The buffers of steps in that shape (allocates: not while capturing), one
-// block: band words, exchange rows, step numbers.  Cleared on the steps' own
-// stream: a clear on the default stream is not ordered before a kernel on a
-// non-blocking one, which would read words not yet cleared or lose words that
-// its bands have published.
-static int resident_buffers(flood_grid* g, const ResidentShape& sh, cudaStream_t s)
+// The buffers of steps that stay on the chip, one block: band words, exchange
+// rows, step numbers.  Made with the ensemble, so that a step never allocates
+// (a stream that records a graph refuses that), and cleared on the stream that
+// flood_ensemble_init waits for, before any step on any stream.  Tracked
+// maxima and land cover take the same bands where they fit at all.  Without
+// room for them the steps march.
+static int resident_buffers(flood_grid* g, cudaStream_t s)
 {
-    if (g->rs_words && g->rs_shape.bands >= sh.bands) return FLOOD_OK;
+    const ResidentShape sh = resident_shape(g->ny, g->nx, g->M, g->n_sm, g->smem_max, false, false);
+    if (sh.bands == 0) return FLOOD_OK;
     const size_t n = (size_t)2 * g->M * sh.bands, rows = n * 2 * g->ld;
     const size_t words = n + rows + ((size_t)g->M + 1) / 2;
-    g->rs_shape = {0, 0, 0};
-    g->rs_xch = nullptr;
-    g->rs_seq = nullptr;
-    const int rc = dalloc(g, &g->rs_words, words);
-    if (rc) return rc;
+    if (dalloc(g, &g->rs_words, words)) {
+        cudaGetLastError();
+        return FLOOD_OK;
+    }
     g->rs_xch = g->rs_words + n;
     g->rs_seq = reinterpret_cast<uint32_t*>(g->rs_xch + rows);
     CK(g, cudaMemsetAsync(g->rs_words, 0, sizeof(unsigned long long) * words, s));
-    g->rs_shape = sh;
     return FLOOD_OK;
 }
 
@@ -382,10 +383,6 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
     int64_t i = 0;
     ResidentShape sh;
     const bool res = resident_now(g, &sh);
-    if (res) {
-        const int rc = resident_buffers(g, sh, s);
-        if (rc) return rc;
-    }
     // up to `n` steps, however they run
     auto some = [&](int n) -> int {
         i += n;
@@ -701,6 +698,7 @@ int flood_ensemble_init(flood_grid* g, int M, const float* h0, int h0_per_member
     CK(g, cudaMemsetAsync(g->inflow_acc, 0, sizeof(double) * M, s));
     CK(g, cudaMemsetAsync(g->pf_small, 0, sizeof(int32_t) * 4, s));
     CK(g, cudaMemsetAsync(g->err, 0, sizeof(int), s));
+    if ((rc = flood::resident_buffers(g, s))) return rc;
     g->k = 0;
     flood::launch_hmax(g->state, g->ms, M, g->ny, g->nx, g->ld, g->plane, g->n_sm, s);
     g->launches++;

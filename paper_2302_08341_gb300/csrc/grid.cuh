@@ -49,7 +49,6 @@ struct flood_grid {
     unsigned long long* rs_words = nullptr;  // one block: band words, exchange rows, step numbers
     unsigned long long* rs_xch = nullptr;
     uint32_t* rs_seq = nullptr;
-    flood::ResidentShape rs_shape{0, 0, 0};  // the shape the buffers were sized for
     // particle filter
     int G = 0, G_cap = 0;
     int32_t* cells = nullptr;     // [G_cap]

@@ -49,3 +49,25 @@ def test_the_first_step_on_a_side_stream_while_the_default_stream_is_busy(capi, 
             for m in range(shape[2]):
                 assert np.array_equal(np.stack(g.get_state(m)), ref[m])
         assert np.array_equal(g.members()["t"], t)
+
+
+@pytest.mark.parametrize("shape", [(64, 131, 7), (40, 129, 200)])
+def test_the_first_steps_may_be_recorded_into_a_graph(capi, shape):
+    """flood_step(n) only launches: it may be an ensemble's first call inside
+    the capture of the caller's stream, on the chip (7 members) as on the march
+    (200), and the graph's replays step the ensemble."""
+    import torch
+    n, replays = 6, 3
+    ref, t = _march(capi, *shape, (n,) * replays)
+    stream = torch.cuda.Stream()
+    with _grid(capi, *shape) as g:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            g.step(n)
+        with torch.cuda.stream(stream):
+            for _ in range(replays):
+                graph.replay()
+            g.sync()
+            for m in range(shape[2]):
+                assert np.array_equal(np.stack(g.get_state(m)), ref[m])
+        assert np.array_equal(g.members()["t"], t)
