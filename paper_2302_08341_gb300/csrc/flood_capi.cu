@@ -491,14 +491,15 @@ using flood::ensure_vacc;
 
 namespace {
 
-// The automatic strip height of the TMA step (strip_rows).
+// The automatic strip height of the TMA step (strip_rows).  The strips of a
+// span lie along grid.z, which holds 65535.
 int choose_rows_per_strip(int ny, int nx, int M, int n_sm, bool track)
 {
     const int64_t spans = (int64_t)M * ((nx + 127) / 128);
     // strips do not cross members or spans: round the strips per span down
     int rh = flood::strip_rows(spans * ny, n_sm, track);
     while (rh < (track ? 9 : 12) && spans * ((ny + rh - 1) / rh) > (int64_t)n_sm * (track ? 16 : 20)) ++rh;
-    return std::min(rh, 4096);
+    return std::min(std::max(rh, (ny + 65534) / 65535), 4096);
 }
 
 // Four members of a tile per CTA where M divides well; CTAs of one or two
