@@ -4,6 +4,8 @@
 // streams its rows through shared memory (tma_march.cuh).
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+
 #include "launch.cuh"
 #include "tma_march.cuh"
 
@@ -32,7 +34,9 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
     pdl_wait();
     pdl_launch();  // after the wait: the next plan may then read the clocks this step's plan left
     if (a.tiles) {  // only the tiles that hold a cell of the domain are launched
-        const int2 tl = a.tiles[blockIdx.y];
+        const int64_t i = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
+        if (i >= a.n_tiles) return;
+        const int2 tl = a.tiles[i];
         span = tl.x;
         strip = tl.y;
     }
@@ -206,7 +210,10 @@ void launch_tma_wm(const TmaArgs& t, cudaStream_t s)
         attr = true;
     }
     const StepArgs& a = t.a;
-    const dim3 grid((a.M + WM - 1) / WM, a.tiles ? a.n_tiles : spans_of(a), a.tiles ? 1 : strips_of(a));
+    // listed tiles lie along y and z (short strips over a large grid are more than 65535)
+    const int ty = std::min(a.n_tiles, 65535);
+    const dim3 grid((a.M + WM - 1) / WM, a.tiles ? ty : spans_of(a),
+                    a.tiles ? (a.n_tiles + ty - 1) / ty : strips_of(a));
     launch_pdl(f, grid, dim3(32, WM), shm, s, t);
 }
 

@@ -47,3 +47,30 @@ def test_a_grid_of_more_than_65535_short_strips(capi, track):
     for a, b in zip(*res):
         assert np.array_equal(a, b)
     assert res[0][0].max() > 0.0 and np.abs(res[0][2]).max() > 0.0
+
+
+def test_a_domain_of_more_than_65535_tiles(capi):
+    """Land cover with cells outside the domain: the step launches the tiles
+    that hold a cell of it, here 33 thousand strips of two spans.  The same
+    step, bit for bit, as with direct loads, which leave no tile out."""
+    ny, nx = 800_000, 129
+    z, n, h0 = _fields(ny, nx, 7)
+    cls = np.zeros((ny, nx), np.int32)
+    cls[::7, ::3] = 1
+    cls[400_000:400_100] = 3
+    classes = [c[:3] + (1 if i == 3 else 0,) for i, c in enumerate(synth.LAND_CLASSES)]
+    hy = synth.hyetograph_constant(60.0, 600.0)
+    res = []
+    for engine in (1, 0):
+        with capi.Grid(z, n) as g:
+            g.set_land_cover(cls, classes)
+            g.ensemble_init(1, np.ones(1, np.float32), np.ones(1, np.float32), hy, h0=h0)
+            rows = g.get_launch()[0]
+            assert 2 * ((ny - 100) // rows) > 65535
+            g.set_engine(engine)
+            g.step(2)
+            g.sync()
+            res.append(g.get_state(0))
+    for a, b in zip(*res):
+        assert np.array_equal(a, b)
+    assert res[0][0].max() > 0.0 and not res[0][0][400_000:400_100].any()
