@@ -53,7 +53,7 @@ struct StepArgs {
     struct MemberPlan* log;     // [M][dt_log_cap] plans of the steps taken (or null)
     float* ckpt;                // [n_ckpt][M][3][plane] checkpoint states (or null)
     int ckpt_every;             // a checkpoint after every ckpt_every steps of a member
-    int slots;                  // every state is kept: a step reads checkpoint slot i, writes slot i + 1
+    int slots;                  // every state is kept: a step goes from checkpoint slot to slot (kept_slot)
     // replay of a checkpointed segment (adjoint recomputation): slot i of
     // seg holds the state after step seg_first + i; this launch recomputes
     // step seg_first + replay_i of every member with seg_first + replay_i <
@@ -123,6 +123,16 @@ struct MemberPlan {
                               // slot the step reads)
     float q_in;               // inflow flux per unit width of this step (m^2/s), 0 without
 };
+
+// Where every state is kept, the checkpoint slot of a member's state after
+// `steps` steps, of slots 0 to last.  A window that turns out to need more
+// steps than the slots hold is run again, but it is followed to its end on its
+// own trajectory (its steps may raise the running maxima, or find a depth that
+// is not finite): those states take turns in the last two slots.
+__host__ __device__ inline int kept_slot(int64_t steps, int last)
+{
+    return steps <= last ? (int)steps : last - (int)((steps - last) & 1);
+}
 
 // Step length of one member (Eq. 4 with floor, cap and landing on the next
 // stop).

@@ -47,8 +47,7 @@ __global__ void gauge_slots_kernel(const float* __restrict__ slots, const Member
     if (t >= M * G) return;
     const int m = t / G, k = t % G;
     const int cell = cells[k];
-    const int64_t i = ms[m].steps < last ? ms[m].steps : last;
-    y[t] = slots[((size_t)i * M + m) * 3 * plane + (size_t)(cell / nx) * ld + cell % nx];
+    y[t] = slots[((size_t)kept_slot(ms[m].steps, last) * M + m) * 3 * plane + (size_t)(cell / nx) * ld + cell % nx];
 }
 
 // DA steps (II)-(IV) and the bookkeeping of step (V), one block.

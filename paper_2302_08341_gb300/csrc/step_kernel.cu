@@ -69,8 +69,8 @@ __global__ void plan_kernel(const StepArgs a)
     p.cur = in.cur;
     p.ckpt = -1;
     if (w.active) {
-        if (a.slots)  // (steps past the log's end stay in its last slots: the window is run again)
-            p.ckpt = (int)(in.steps < a.dt_log_cap ? in.steps : a.dt_log_cap - 1);
+        if (a.slots)
+            p.ckpt = kept_slot(in.steps, a.dt_log_cap);
         else if (a.ckpt && (in.steps + 1) % a.ckpt_every == 0 && in.steps + 1 <= a.dt_log_cap)
             p.ckpt = (int)((in.steps + 1) / a.ckpt_every);
     }

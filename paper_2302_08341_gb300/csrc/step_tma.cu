@@ -53,8 +53,8 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
     // the other state buffer, and a checkpoint slot every so many steps; or,
     // where every state is kept, from one slot to the next
     const bool slots = CK && a.slots;
-    float* __restrict__ dst = slots ? a.ckpt + ((size_t)(pl.ckpt + 1) * a.M + m) * mstride
-                                    : a.state + (size_t)((1 - pl.cur) * a.M + m) * mstride;
+    const int to = slots ? kept_slot((int64_t)pl.ckpt + 1, a.dt_log_cap) : 1 - pl.cur;
+    float* __restrict__ dst = (slots ? a.ckpt : a.state) + ((size_t)to * a.M + m) * mstride;
     float* ck = (CK && !slots && pl.ckpt >= 0) ? a.ckpt + ((size_t)pl.ckpt * a.M + m) * mstride : nullptr;
 
     FaceK k;

@@ -286,3 +286,36 @@ def test_kept_states_give_the_recomputed_gradients(capi, ny, nx, M, shape, land,
         res.append(got)
     for a, b in zip(*res):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("shape", [(8, 1), (16, 4), None])
+def test_a_window_run_twice_raises_the_maxima_of_its_own_states_only(capi, shape):
+    """Deep water under a rising storm with an inflow: the window outgrows the
+    first step log, while its states are kept from slot to slot (with a fixed
+    launch shape) or on the chip.  The maxima tracked meanwhile are those of
+    the states that explicit checkpoints pass through, bit for bit."""
+    ny, nx, M = 40, 140, 4
+    rng = np.random.default_rng(61)
+    terr = synth.make_terrain(ny, nx, seed=61, building_frac=0.0)
+    hy = (np.array([1.0, 40.0, 2000.0, 4000.0]) * 1e-3 / 3600.0).astype(np.float32)
+    rm, sc = synth.ensemble_prior(61, M)
+    start = (3.0 * rng.uniform(0.5, 1.0, (M, ny, nx))).astype(np.float32)
+    cells = rng.choice(ny * nx, 4, replace=False).astype(np.int32)
+    d = rng.uniform(1.5, 3.0, (3, 4))
+    p = capi.Params.default(rain_block=8.0)
+    res = []
+    for every in (0, 5):
+        with capi.Grid(terr.z, terr.n, p) as g:
+            g.ensemble_init(M, rm, sc, hy, h0=start)
+            g.set_inflow(5, 30, np.array([0.0, 20.0, 300.0, 900.0], np.float32))
+            g.track_max_depth(True)
+            if shape:
+                g.set_launch(*shape)
+            out = g.adjoint(cells, d, 10.0, ckpt_every=every)
+            # more steps than the first log holds (30 s at dt_cap = 1, and 2 x 3 + 8)
+            assert g.members()["steps"].min() > 30 + 14
+            vol = g.volumes()
+            res.append([out["loss"], out["grad_n"], vol["storage"], vol["rain"], vol["outflow"], vol["clamp"]] +
+                       [g.max_depth(m) for m in range(M)])
+    for a, b in zip(*res):
+        np.testing.assert_array_equal(a, b)
