@@ -66,11 +66,32 @@ bool keep_states(const flood_grid* g, size_t floats)
     return floats * sizeof(float) <= (free_b + g->ckpt_floats * sizeof(float)) / 3;
 }
 
+// The volume counters of an ensemble: rain and inflow per member, outflow and
+// clamp per slot, drained volume per slot (land cover).
+struct Volumes {
+    std::vector<double> rain, inflow, vacc, dacc;
+};
+
+int read_volumes(flood_grid* g, Volumes& v)
+{
+    const size_t M = g->M;
+    v.rain.resize(M);
+    v.vacc.resize(M * g->nslot * 2);
+    v.inflow.resize(g->inflow ? M : 0);
+    v.dacc.resize(g->dacc ? M * g->nslot : 0);
+    CK(g, cudaMemcpy(v.rain.data(), g->rain_acc, sizeof(double) * M, cudaMemcpyDeviceToHost));
+    CK(g, cudaMemcpy(v.vacc.data(), g->vacc, sizeof(double) * v.vacc.size(), cudaMemcpyDeviceToHost));
+    if (!v.inflow.empty())
+        CK(g, cudaMemcpy(v.inflow.data(), g->inflow_acc, sizeof(double) * M, cudaMemcpyDeviceToHost));
+    if (!v.dacc.empty())
+        CK(g, cudaMemcpy(v.dacc.data(), g->dacc, sizeof(double) * v.dacc.size(), cudaMemcpyDeviceToHost));
+    return FLOOD_OK;
+}
+
 // Put the state saved in ckpt slot 0 back into each member's current buffer
 // and restore the saved clocks and volume counters (a forward that overflowed
 // the step log is redone).
-int restore_start(flood_grid* g, const std::vector<MemberClock>& c0, const std::vector<double>& rain0,
-                  const std::vector<double>& vacc0, cudaStream_t s)
+int restore_start(flood_grid* g, const std::vector<MemberClock>& c0, const Volumes& v0, cudaStream_t s)
 {
     const int M = g->M;
     const size_t ms = 3 * g->plane;
@@ -86,8 +107,14 @@ int restore_start(flood_grid* g, const std::vector<MemberClock>& c0, const std::
     }
     CK(g, cudaMemcpyAsync(g->ms + (g->k % 3) * M, back.data(), sizeof(MemberClock) * M,
                           cudaMemcpyHostToDevice, s));
-    CK(g, cudaMemcpyAsync(g->rain_acc, rain0.data(), sizeof(double) * M, cudaMemcpyHostToDevice, s));
-    CK(g, cudaMemcpyAsync(g->vacc, vacc0.data(), sizeof(double) * vacc0.size(), cudaMemcpyHostToDevice, s));
+    auto put = [&](double* to, const std::vector<double>& v) {
+        return v.empty() ? cudaSuccess
+                         : cudaMemcpyAsync(to, v.data(), sizeof(double) * v.size(), cudaMemcpyHostToDevice, s);
+    };
+    CK(g, put(g->rain_acc, v0.rain));
+    CK(g, put(g->inflow_acc, v0.inflow));
+    CK(g, put(g->vacc, v0.vacc));
+    CK(g, put(g->dacc, v0.dacc));
     CK(g, cudaStreamSynchronize(s));
     return FLOOD_OK;
 }
@@ -123,9 +150,8 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             return flood::fail(g, FLOOD_ERR_ARG, "gauge cell index out of range");
 
     // saved start: clocks, volume counters (restored if the forward is redone)
-    std::vector<double> rain0(M), vacc0((size_t)M * g->nslot * 2);
-    CK(g, cudaMemcpy(rain0.data(), g->rain_acc, sizeof(double) * M, cudaMemcpyDeviceToHost));
-    CK(g, cudaMemcpy(vacc0.data(), g->vacc, sizeof(double) * vacc0.size(), cudaMemcpyDeviceToHost));
+    Volumes v0;
+    if ((rc = read_volumes(g, v0))) return rc;
 
     const double T = ns * L->sample_dt;
     const double dt_ref = g->p.dt_fixed > 0 ? g->p.dt_fixed : g->p.dt_cap;
@@ -221,7 +247,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         g->logging = g->slots = false;
         if (kmax <= cap) break;
         if (attempt >= 4) return flood::fail(g, FLOOD_ERR_STATE, "step log could not hold the window");
-        if ((rc = restore_start(g, c0, rain0, vacc0, s))) return rc;
+        if ((rc = restore_start(g, c0, v0, s))) return rc;
         cap = (int)std::min<int64_t>((int64_t)kmax * 2 + 8, INT32_MAX / 2);
     }
 

@@ -319,3 +319,44 @@ def test_a_window_run_twice_raises_the_maxima_of_its_own_states_only(capi, shape
                        [g.max_depth(m) for m in range(M)])
     for a, b in zip(*res):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("every", [0, 5])
+@pytest.mark.parametrize("shape", [(8, 1), None])
+def test_a_window_run_twice_counts_its_volumes_once(capi, shape, every):
+    """Deep water outgrows the first step log and the window is run again: the
+    rain, inflow, drained, outflow and clamp volumes are those of the same
+    window by ordinary steps, which land on the same observation times."""
+    ny, nx, M = 40, 140, 4
+    rng = np.random.default_rng(67)
+    terr = synth.make_terrain(ny, nx, seed=67, building_frac=0.0)
+    hy = (np.array([10.0, 40.0, 90.0, 60.0]) * 1e-3 / 3600.0).astype(np.float32)
+    rm, sc = synth.ensemble_prior(67, M)
+    start = (3.0 * rng.uniform(0.5, 1.0, (M, ny, nx))).astype(np.float32)
+    cells = rng.choice(ny * nx, 4, replace=False).astype(np.int32)
+    d = rng.uniform(1.5, 3.0, (3, 4))
+    p = capi.Params.default(rain_block=8.0)
+    res = []
+    for adjoint in (True, False):
+        with capi.Grid(terr.z, terr.n, p) as g:
+            g.set_land_cover(synth.land_cover(terr, seed=3, pond_side=(4, 9)), synth.LAND_CLASSES)
+            g.ensemble_init(M, rm, np.ones(M, np.float32), hy, h0=start)
+            g.set_land_params(*synth.land_prior(3, M))
+            g.set_inflow(5, 30, np.array([2.0, 20.0, 30.0, 9.0], np.float32))
+            if shape:
+                g.set_launch(*shape)
+            if adjoint:
+                g.adjoint(cells, d, 10.0, ckpt_every=every)
+            else:
+                for k in (1, 2, 3):
+                    g.advance_to(10.0 * k)
+            assert g.members()["steps"].min() > 30 + 14
+            v = g.volumes()
+            res.append([v["storage"], v["rain"], g.inflow_volume(), v["outflow"], v["clamp"], g.drained()])
+    # on the chip a launch's steps form one partial of the last three, and the
+    # launches start at the phase the first run left: the bound of
+    # test_gpu_resident.py for sums in other pieces
+    bound = [0.0] * 3 + [0.0 if shape else 2.0 ** -22] * 3
+    for a, b, tol in zip(*res, bound):
+        np.testing.assert_allclose(a, b, rtol=tol, atol=0)
+    assert min(res[0][2].min(), res[0][5].min()) > 0.0
