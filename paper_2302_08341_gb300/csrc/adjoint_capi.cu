@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <string>
 #include <vector>
 
 #include "adjoint.cuh"
@@ -119,6 +120,57 @@ int restore_start(flood_grid* g, const std::vector<MemberClock>& c0, const Volum
     return FLOOD_OK;
 }
 
+// Where the steps went from kept slot to slot, each member's last state back
+// into the ensemble's current buffer.
+int slots_to_state(flood_grid* g, cudaStream_t s)
+{
+    const int M = g->M;
+    const size_t ms = 3 * g->plane;
+    std::vector<MemberClock> c(M);
+    CK(g, cudaMemcpyAsync(c.data(), g->ms + (g->k % 3) * M, sizeof(MemberClock) * M, cudaMemcpyDeviceToHost, s));
+    CK(g, cudaStreamSynchronize(s));
+    for (int m = 0; m < M; ++m)
+        CK(g, cudaMemcpyAsync(g->state + (size_t)(c[m].cur * M + m) * ms,
+                              g->ckpt + ((size_t)flood::kept_slot(c[m].steps, g->log_cap) * M + m) * ms,
+                              sizeof(float) * ms, cudaMemcpyDeviceToDevice, s));
+    return FLOOD_OK;
+}
+
+// The window's forward: its steps are logged, and go from slot to slot where
+// `slots`.  However it ends, later steps do neither, and the ensemble holds
+// the state that its clocks stand at.
+struct Logging {
+    flood_grid* g;
+    cudaStream_t s;
+    Logging(flood_grid* g_, bool slots, cudaStream_t s_) : g(g_), s(s_)
+    {
+        g->logging = true;
+        g->slots = slots;
+    }
+    ~Logging()
+    {
+        if (!g->logging) return;
+        const std::string msg = g->msg;  // of the error that ends it
+        end();
+        g->msg = msg;
+    }
+    int end()
+    {
+        const int rc = g->slots ? slots_to_state(g, s) : FLOOD_OK;
+        g->logging = g->slots = false;
+        return rc;
+    }
+};
+
+struct Events {
+    cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
+    ~Events()
+    {
+        for (cudaEvent_t v : e)
+            if (v) cudaEventDestroy(v);
+    }
+};
+
 }  // namespace
 
 extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_every, float* grad_n,
@@ -164,10 +216,11 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     int K = 0;
     bool keep = false;  // every state of the window is kept: nothing is recomputed
     size_t n_ckpt = 0;
-    cudaEvent_t e0, e1, e2;
-    CK(g, cudaEventCreate(&e0));
-    CK(g, cudaEventCreate(&e1));
-    CK(g, cudaEventCreate(&e2));
+    Events ev;
+    for (cudaEvent_t& e : ev.e) CK(g, cudaEventCreate(&e));
+    // the gauges' cells, for the samples and the seeds
+    if ((rc = grow(g, &g->samp_cells, room.samp_cells, G))) return rc;
+    CK(g, cudaMemcpyAsync(g->samp_cells, cells.data(), sizeof(int32_t) * G, cudaMemcpyHostToDevice, s));
     for (int attempt = 0;; ++attempt) {
         keep = ckpt_every == 0 && keep_states(g, (size_t)(cap + 1) * M * ms);
         for (;;) {
@@ -183,11 +236,10 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         }
         // where every state is kept the TMA step goes from slot to slot (the
         // resident steps write each state to its slot as a checkpoint)
-        g->slots = keep && g->engine == 1 && g->maps_ok && g->wait_budget < 0 && !flood::steps_resident(g);
-        if (g->slots)
-            g->slots = flood::encode_map_3d(&g->ckpt_map, g->ckpt, g->ld, g->ny, (uint64_t)n_ckpt * M * 3,
-                                            sizeof(float) * g->ld, sizeof(float) * g->plane,
-                                            flood::tma_box_cols(), 1, 3) == 0;
+        const bool slots = keep && g->engine == 1 && g->maps_ok && g->wait_budget < 0 && !flood::steps_resident(g) &&
+                           flood::encode_map_3d(&g->ckpt_map, g->ckpt, g->ld, g->ny, (uint64_t)n_ckpt * M * 3,
+                                                sizeof(float) * g->ld, sizeof(float) * g->plane,
+                                                flood::tma_box_cols(), 1, 3) == 0;
         if ((rc = grow(g, &g->log, room.log, (size_t)M * cap))) return rc;
         if ((rc = grow(g, &g->samp_y, room.samp_y, (size_t)ns * M * G))) return rc;
         g->log_cap = cap;
@@ -202,22 +254,12 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         }
         CK(g, cudaMemcpyAsync(g->ms + (g->k % 3) * M, cz.data(), sizeof(MemberClock) * M,
                               cudaMemcpyHostToDevice, s));
-        g->logging = true;
-        CK(g, cudaEventRecord(e0, s));
+        Logging log(g, slots, s);
+        CK(g, cudaEventRecord(ev.e[0], s));
         int64_t kmax = 0;
         for (int sidx = 1; sidx <= ns; ++sidx) {
-            rc = flood_step(g, 0, t0 + sidx * L->sample_dt, stream);
-            if (rc) {
-                g->logging = g->slots = false;
-                return rc;
-            }
-            // the cells live in samp_cells (device) for both gauge sampling and seeding
-            if (sidx == 1) {
-                if ((rc = grow(g, &g->samp_cells, room.samp_cells, G))) return rc;
-                CK(g, cudaMemcpyAsync(g->samp_cells, cells.data(), sizeof(int32_t) * G,
-                                      cudaMemcpyHostToDevice, s));
-            }
-            if (g->slots)
+            if ((rc = flood_step(g, 0, t0 + sidx * L->sample_dt, stream))) return rc;
+            if (slots)
                 flood::launch_gauge_slots(g->ckpt, g->ms + (g->k % 3) * M, cap, g->samp_cells, G, M, g->ld, g->nx,
                                           g->plane, g->samp_y + (size_t)(sidx - 1) * M * G, s);
             else
@@ -225,26 +267,15 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
                                     g->plane, g->samp_y + (size_t)(sidx - 1) * M * G, s);
             g->launches++;
             std::vector<MemberClock> cc;
-            if ((rc = flood::read_clocks(g, cc, s))) {
-                g->logging = g->slots = false;
-                return rc;
-            }
+            if ((rc = flood::read_clocks(g, cc, s))) return rc;
             for (int m = 0; m < M; ++m) {
                 samp_step[(size_t)(sidx - 1) * M + m] = (int32_t)cc[m].steps;
                 K_m[m] = (int)std::min<int64_t>(cc[m].steps, INT32_MAX);
                 kmax = std::max<int64_t>(kmax, cc[m].steps);
             }
         }
-        if (g->slots && kmax <= cap) {  // the window's end is the ensemble's state
-            std::vector<MemberClock> cc;
-            if ((rc = flood::read_clocks(g, cc, s))) return rc;
-            for (int m = 0; m < M; ++m)
-                CK(g, cudaMemcpyAsync(g->state + (size_t)(cc[m].cur * M + m) * ms,
-                                      g->ckpt + ((size_t)K_m[m] * M + m) * ms, sizeof(float) * ms,
-                                      cudaMemcpyDeviceToDevice, s));
-        }
-        CK(g, cudaEventRecord(e1, s));
-        g->logging = g->slots = false;
+        if ((rc = log.end())) return rc;  // the window's end is the ensemble's state
+        CK(g, cudaEventRecord(ev.e[1], s));
         if (kmax <= cap) break;
         if (attempt >= 4) return flood::fail(g, FLOOD_ERR_STATE, "step log could not hold the window");
         if ((rc = restore_start(g, c0, v0, s))) return rc;
@@ -428,17 +459,14 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         }
         CK(g, cudaGetLastError());
     }
-    CK(g, cudaEventRecord(e2, s));
+    CK(g, cudaEventRecord(ev.e[2], s));
     CK(g, cudaStreamSynchronize(s));
     if ((rc = flood::check_err(g))) return rc;
     float fms = 0.0f, rms = 0.0f;
-    cudaEventElapsedTime(&fms, e0, e1);
-    cudaEventElapsedTime(&rms, e1, e2);
+    cudaEventElapsedTime(&fms, ev.e[0], ev.e[1]);
+    cudaEventElapsedTime(&rms, ev.e[1], ev.e[2]);
     g->adj_fwd_ms = fms;
     g->adj_rev_ms = rms;
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaEventDestroy(e2);
 
     if (grad_h0)
         for (int m = 0; m < M; ++m)

@@ -360,3 +360,34 @@ def test_a_window_run_twice_counts_its_volumes_once(capi, shape, every):
     for a, b, tol in zip(*res, bound):
         np.testing.assert_allclose(a, b, rtol=tol, atol=0)
     assert min(res[0][2].min(), res[0][5].min()) > 0.0
+
+
+@pytest.mark.parametrize("shape", [(8, 1), (16, 4), None])
+def test_an_error_within_a_window_leaves_the_states_it_came_to(capi, shape):
+    """A window that ends in an error (a depth that is not finite in one
+    member) returns with the ensemble at the state its clocks stand at, also
+    where every state is kept from slot to slot, and steps go on from there."""
+    ny, nx, M = 40, 140, 4
+    rng = np.random.default_rng(71)
+    terr = synth.make_terrain(ny, nx, seed=71, building_frac=0.0)
+    rm, sc = synth.ensemble_prior(71, M)
+    start = rng.uniform(0.1, 0.4, (M, ny, nx)).astype(np.float32)
+    start[1, 20, 70] = np.nan
+    cells = rng.choice(ny * nx, 4, replace=False).astype(np.int32)
+    res = []
+    for every in (0, 5):
+        with capi.Grid(terr.z, terr.n) as g:
+            g.ensemble_init(M, rm, sc, synth.hyetograph_constant(60.0, 600.0), h0=start)
+            if shape:
+                g.set_launch(*shape)
+            with pytest.raises(capi.FloodError) as e:
+                g.adjoint(cells, np.ones((3, 4)), 10.0, ckpt_every=every)
+            assert e.value.code == -5 and "non-finite" in str(e.value)
+            got = [g.members()["t"]] + [x for m in range(M) for x in g.get_state(m)]
+            g.step(3)
+            got += [g.members()["t"]] + [x for m in range(M) for x in g.get_state(m)]
+        assert got[0].min() > 0.0 and not np.array_equal(got[1], start[0])
+        res.append(got)
+    for a, b in zip(*res):
+        np.testing.assert_array_equal(a, b)
+    assert not np.array_equal(res[0][1], res[0][1 + 3 * M + 1])   # the state moved on
