@@ -206,8 +206,11 @@ typedef struct {
  * wet/dry test, outflow clip, negative-depth clamp).  Memory: a checkpoint
  * every ckpt_every steps plus ckpt_every + 1 replayed states, each 12 bytes per
  * cell per member; ckpt_every = 0: every state of the window where they take at
- * most a third of the free device memory (nothing is then replayed), else a
- * checkpoint about every sqrt(steps).  Results do not depend on it.
+ * most a third of the free device memory and a quarter of all of it (nothing is
+ * then replayed), else a checkpoint about every sqrt(steps).  Results do not
+ * depend on it.  Checkpoints stay with the ensemble; states that were kept go
+ * back to a pool of the process, which any allocation that needs the memory
+ * takes from (at most an eighth of the device's once a handle is destroyed).
  *   grad_n      [ny][nx] FP32  sum_i dL_i/dn_base (or NULL)
  *   grad_rain   [N] FP64       dL_i/d(rain multiplier of i) (or NULL)
  *   grad_scale  [N] FP64       dL_i/d(Manning scale of i) (or NULL)

@@ -9,7 +9,10 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "adjoint.cuh"
@@ -50,49 +53,108 @@ int reverse_rows(int ny, int nx, int M, int n_sm)
     return rh;
 }
 
-// Whether to keep every state of a window (`floats` of them in all) instead of
-// checkpoints to recompute from: the recomputation moves 26 bytes per
-// member-cell-step and takes a quarter of the gradient's time, the slots cost
-// nothing extra to write (24 members of 1000 x 1000, 60 steps, 20 GB: 28.9 ms
-// recomputing, 21.9 ms keeping).  Up to a third of the memory that is free
-// beside the slots already held.
-bool keep_states(const flood_grid* g, size_t floats)
-{
-    if (floats <= g->ckpt_floats) return true;
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return floats * sizeof(float) <= (free_b + g->ckpt_floats * sizeof(float)) / 3;
-}
-
-// The volume counters of an ensemble: rain and inflow per member, outflow and
-// clamp per slot, drained volume per slot (land cover).
-struct Volumes {
-    std::vector<double> rain, inflow, vacc, dacc;
+// The memory of kept states comes from a stream-ordered pool, one a device for
+// every ensemble of the process, and goes back to it with the call.  What the
+// pool holds unused the driver hands to any allocation of the process that
+// finds too little memory otherwise (a buffer of the ensemble's own would be
+// lost to the rest of the program, tens of GB of it), and the next window
+// finds it mapped: 20 GB in 4 us, 18.7 ms the first time.  It holds at most a
+// quarter of the device's memory, an eighth once an ensemble is destroyed.
+struct StatePool {
+    cudaMemPool_t pool = nullptr;  // (null: none can be had)
+    size_t total = 0;              // the device's memory
 };
 
-int read_volumes(flood_grid* g, Volumes& v)
+StatePool state_pool()
 {
-    const size_t M = g->M;
-    v.rain.resize(M);
-    v.vacc.resize(M * g->nslot * 2);
-    v.inflow.resize(g->inflow ? M : 0);
-    v.dacc.resize(g->dacc ? M * g->nslot : 0);
-    CK(g, cudaMemcpy(v.rain.data(), g->rain_acc, sizeof(double) * M, cudaMemcpyDeviceToHost));
-    CK(g, cudaMemcpy(v.vacc.data(), g->vacc, sizeof(double) * v.vacc.size(), cudaMemcpyDeviceToHost));
-    if (!v.inflow.empty())
-        CK(g, cudaMemcpy(v.inflow.data(), g->inflow_acc, sizeof(double) * M, cudaMemcpyDeviceToHost));
-    if (!v.dacc.empty())
-        CK(g, cudaMemcpy(v.dacc.data(), g->dacc, sizeof(double) * v.dacc.size(), cudaMemcpyDeviceToHost));
+    static std::mutex mu;
+    static std::map<int, StatePool> pools;
+    int dev = 0;
+    size_t free_b = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return {};
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = pools.find(dev);
+    if (it != pools.end()) return it->second;
+    StatePool p;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    uint64_t most = 0;
+    if (cudaMemGetInfo(&free_b, &p.total) == cudaSuccess && cudaMemPoolCreate(&p.pool, &props) == cudaSuccess) {
+        most = p.total / 4;
+        cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &most);
+    }
+    cudaGetLastError();
+    return pools[dev] = p;
+}
+
+// The kept states of one call.
+struct KeptStates {
+    flood_grid* g;
+    cudaStream_t s;
+    KeptStates(flood_grid* g_, cudaStream_t s_) : g(g_), s(s_) {}
+    ~KeptStates()
+    {
+        if (!g->kept) return;
+        release();
+        cudaStreamSynchronize(s);  // the memory is the pool's to give away once the free has run
+    }
+    void release()
+    {
+        if (g->kept) cudaFreeAsync(g->kept, s);
+        g->kept = nullptr;
+    }
+    // Whether to keep every state of a window (`floats` of them in all) instead
+    // of checkpoints to recompute from: the recomputation moves 26 bytes per
+    // member-cell-step and takes a quarter of the gradient's time, the slots
+    // cost nothing extra to write (24 members of 1000 x 1000, 60 steps, 20 GB:
+    // 28.9 ms recomputing, 21.9 ms keeping).  Memory that the pool holds
+    // already, or up to a third of what is free, and no more than it holds on to.
+    bool keep(size_t floats)
+    {
+        release();
+        const StatePool p = state_pool();
+        const size_t bytes = floats * sizeof(float);
+        size_t free_b = 0, total_b = 0;
+        uint64_t held = 0, used = 0;
+        if (p.pool && bytes <= p.total / 4 &&
+            cudaMemPoolGetAttribute(p.pool, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+            cudaMemPoolGetAttribute(p.pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+            (bytes <= held - used || (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+                                      bytes <= (free_b + (size_t)(held - used)) / 3))) {
+            void* mem = nullptr;
+            if (cudaMallocFromPoolAsync(&mem, bytes, p.pool, s) == cudaSuccess) g->kept = static_cast<float*>(mem);
+        }
+        cudaGetLastError();
+        g->kept_any |= g->kept != nullptr;
+        return g->kept != nullptr;
+    }
+};
+
+// The checkpoints of the window at hand: every state where they are kept.
+float* window_states(const flood_grid* g) { return g->kept ? g->kept : g->ckpt; }
+
+// The ensemble's volume counters (rain and inflow per member, outflow and clamp
+// per slot, drained volume per slot with land cover) to or from g->vol0.
+int copy_volumes(flood_grid* g, bool restore, cudaStream_t s)
+{
+    const size_t M = g->M, slots = M * g->nslot;
+    double* at = g->vol0;
+    const std::pair<double*, size_t> parts[] = {
+        {g->rain_acc, M}, {g->vacc, slots * 2}, {g->inflow_acc, M}, {g->dacc, g->dacc ? slots : 0}};
+    for (const auto& [p, n] : parts) {
+        if (n)
+            CK(g, cudaMemcpyAsync(restore ? p : at, restore ? at : p, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+        at += n;
+    }
     return FLOOD_OK;
 }
 
 // Put the state saved in ckpt slot 0 back into each member's current buffer
 // and restore the saved clocks and volume counters (a forward that overflowed
 // the step log is redone).
-int restore_start(flood_grid* g, const std::vector<MemberClock>& c0, const Volumes& v0, cudaStream_t s)
+int restore_start(flood_grid* g, const std::vector<MemberClock>& c0, cudaStream_t s)
 {
     const int M = g->M;
     const size_t ms = 3 * g->plane;
@@ -103,19 +165,12 @@ int restore_start(flood_grid* g, const std::vector<MemberClock>& c0, const Volum
     for (int m = 0; m < M; ++m) {
         back[m].cur = now[m].cur;
         back[m].steps = 0;
-        CK(g, cudaMemcpyAsync(g->state + (size_t)(now[m].cur * M + m) * ms, g->ckpt + (size_t)m * ms,
+        CK(g, cudaMemcpyAsync(g->state + (size_t)(now[m].cur * M + m) * ms, window_states(g) + (size_t)m * ms,
                               sizeof(float) * ms, cudaMemcpyDeviceToDevice, s));
     }
     CK(g, cudaMemcpyAsync(g->ms + (g->k % 3) * M, back.data(), sizeof(MemberClock) * M,
                           cudaMemcpyHostToDevice, s));
-    auto put = [&](double* to, const std::vector<double>& v) {
-        return v.empty() ? cudaSuccess
-                         : cudaMemcpyAsync(to, v.data(), sizeof(double) * v.size(), cudaMemcpyHostToDevice, s);
-    };
-    CK(g, put(g->rain_acc, v0.rain));
-    CK(g, put(g->inflow_acc, v0.inflow));
-    CK(g, put(g->vacc, v0.vacc));
-    CK(g, put(g->dacc, v0.dacc));
+    if ((rc = copy_volumes(g, true, s))) return rc;
     CK(g, cudaStreamSynchronize(s));
     return FLOOD_OK;
 }
@@ -131,7 +186,7 @@ int slots_to_state(flood_grid* g, cudaStream_t s)
     CK(g, cudaStreamSynchronize(s));
     for (int m = 0; m < M; ++m)
         CK(g, cudaMemcpyAsync(g->state + (size_t)(c[m].cur * M + m) * ms,
-                              g->ckpt + ((size_t)flood::kept_slot(c[m].steps, g->log_cap) * M + m) * ms,
+                              g->kept + ((size_t)flood::kept_slot(c[m].steps, g->log_cap) * M + m) * ms,
                               sizeof(float) * ms, cudaMemcpyDeviceToDevice, s));
     return FLOOD_OK;
 }
@@ -173,6 +228,16 @@ struct Events {
 
 }  // namespace
 
+namespace flood {
+
+void trim_state_pool()
+{
+    const StatePool p = state_pool();
+    if (p.pool) cudaMemPoolTrimTo(p.pool, p.total / 8);
+}
+
+}  // namespace flood
+
 extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_every, float* grad_n,
                              double* grad_rain, double* grad_scale, float* grad_h0, double* loss_out,
                              void* stream)
@@ -202,8 +267,9 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
             return flood::fail(g, FLOOD_ERR_ARG, "gauge cell index out of range");
 
     // saved start: clocks, volume counters (restored if the forward is redone)
-    Volumes v0;
-    if ((rc = read_volumes(g, v0))) return rc;
+    flood_grid::AdjointRoom& room = g->adj_room;
+    if ((rc = grow(g, &g->vol0, room.vol0, (size_t)M * (2 + 3 * g->nslot)))) return rc;
+    if ((rc = copy_volumes(g, false, s))) return rc;
 
     const double T = ns * L->sample_dt;
     const double dt_ref = g->p.dt_fixed > 0 ? g->p.dt_fixed : g->p.dt_cap;
@@ -212,9 +278,9 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     for (int m = 0; m < M; ++m) steps0[m] = c0[m].steps;
     std::vector<int> K_m(M);
     std::vector<int32_t> samp_step((size_t)ns * M);
-    flood_grid::AdjointRoom& room = g->adj_room;
     int K = 0;
     bool keep = false;  // every state of the window is kept: nothing is recomputed
+    KeptStates kept(g, s);
     size_t n_ckpt = 0;
     Events ev;
     for (cudaEvent_t& e : ev.e) CK(g, cudaEventCreate(&e));
@@ -222,22 +288,15 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     if ((rc = grow(g, &g->samp_cells, room.samp_cells, G))) return rc;
     CK(g, cudaMemcpyAsync(g->samp_cells, cells.data(), sizeof(int32_t) * G, cudaMemcpyHostToDevice, s));
     for (int attempt = 0;; ++attempt) {
-        keep = ckpt_every == 0 && keep_states(g, (size_t)(cap + 1) * M * ms);
-        for (;;) {
-            K = ckpt_every > 0 ? ckpt_every : keep ? 1 : std::max(1, (int)std::lround(std::sqrt((double)cap)));
-            n_ckpt = (size_t)cap / K + 1;
-            if (n_ckpt * M * ms <= g->ckpt_floats) break;
-            rc = grow(g, &g->ckpt, g->ckpt_floats, n_ckpt * M * ms);
-            if (!rc) break;
-            g->ckpt_floats = 0;
-            if (!keep || rc != FLOOD_ERR_OOM) return rc;
-            cudaGetLastError();
-            keep = false;  // another allocation took the room meanwhile
-        }
+        keep = ckpt_every == 0 && kept.keep((size_t)(cap + 1) * M * ms);
+        K = ckpt_every > 0 ? ckpt_every : keep ? 1 : std::max(1, (int)std::lround(std::sqrt((double)cap)));
+        n_ckpt = (size_t)cap / K + 1;
+        if (!keep && (rc = grow(g, &g->ckpt, g->ckpt_floats, n_ckpt * M * ms))) return rc;
+        float* const states = window_states(g);
         // where every state is kept the TMA step goes from slot to slot (the
         // resident steps write each state to its slot as a checkpoint)
         const bool slots = keep && g->engine == 1 && g->maps_ok && g->wait_budget < 0 && !flood::steps_resident(g) &&
-                           flood::encode_map_3d(&g->ckpt_map, g->ckpt, g->ld, g->ny, (uint64_t)n_ckpt * M * 3,
+                           flood::encode_map_3d(&g->ckpt_map, states, g->ld, g->ny, (uint64_t)n_ckpt * M * 3,
                                                 sizeof(float) * g->ld, sizeof(float) * g->plane,
                                                 flood::tma_box_cols(), 1, 3) == 0;
         if ((rc = grow(g, &g->log, room.log, (size_t)M * cap))) return rc;
@@ -248,7 +307,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         std::vector<MemberClock> cz;
         if ((rc = flood::read_clocks(g, cz, s))) return rc;
         for (int m = 0; m < M; ++m) {
-            CK(g, cudaMemcpyAsync(g->ckpt + (size_t)m * ms, g->state + (size_t)(cz[m].cur * M + m) * ms,
+            CK(g, cudaMemcpyAsync(states + (size_t)m * ms, g->state + (size_t)(cz[m].cur * M + m) * ms,
                                   sizeof(float) * ms, cudaMemcpyDeviceToDevice, s));
             cz[m].steps = 0;
         }
@@ -260,7 +319,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         for (int sidx = 1; sidx <= ns; ++sidx) {
             if ((rc = flood_step(g, 0, t0 + sidx * L->sample_dt, stream))) return rc;
             if (slots)
-                flood::launch_gauge_slots(g->ckpt, g->ms + (g->k % 3) * M, cap, g->samp_cells, G, M, g->ld, g->nx,
+                flood::launch_gauge_slots(states, g->ms + (g->k % 3) * M, cap, g->samp_cells, G, M, g->ld, g->nx,
                                           g->plane, g->samp_y + (size_t)(sidx - 1) * M * G, s);
             else
                 flood::launch_gauge(g->state, g->ms + (g->k % 3) * M, g->samp_cells, G, M, g->ld, g->nx,
@@ -278,7 +337,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
         CK(g, cudaEventRecord(ev.e[1], s));
         if (kmax <= cap) break;
         if (attempt >= 4) return flood::fail(g, FLOOD_ERR_STATE, "step log could not hold the window");
-        if ((rc = restore_start(g, c0, v0, s))) return rc;
+        if ((rc = restore_start(g, c0, s))) return rc;
         cap = (int)std::min<int64_t>((int64_t)kmax * 2 + 8, INT32_MAX / 2);
     }
 
@@ -304,7 +363,7 @@ extern "C" int flood_adjoint(flood_grid* g, const flood_loss_spec* L, int ckpt_e
     if (!keep && (size_t)(K + 1) * M * ms > g->seg_floats) {
         if ((rc = grow(g, &g->seg, g->seg_floats, (size_t)(K + 1) * M * ms))) return rc;
     }
-    float* const seg = keep ? g->ckpt : g->seg;
+    float* const seg = keep ? g->kept : g->seg;
     if ((rc = grow(g, &g->lam, room.lam, 2 * (size_t)M * ms))) return rc;
     const int rrows = g->launch_fixed ? g->rows_per_strip : reverse_rows(g->ny, g->nx, M, g->n_sm);
     const int nslot = flood::step_nslot(g->ny, g->nx, rrows);

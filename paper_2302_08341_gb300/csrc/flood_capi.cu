@@ -67,7 +67,7 @@ void free_ensemble(flood_grid* g)
     dfree(g->part); dfree(g->storage); dfree(g->cells); dfree(g->d); dfree(g->sigma);
     dfree(g->plan); dfree(g->log); dfree(g->ckpt); dfree(g->seg); dfree(g->lam);
     dfree(g->gnm); dfree(g->gn_out); dfree(g->gpart); dfree(g->seg_end); dfree(g->samp_step);
-    dfree(g->samp_y); dfree(g->samp_d); dfree(g->samp_cells); dfree(g->closs);
+    dfree(g->samp_y); dfree(g->samp_d); dfree(g->samp_cells); dfree(g->vol0); dfree(g->closs);
     dfree(g->hmax_field); dfree(g->lc_n); dfree(g->lc_drain); dfree(g->dacc);
     dfree(g->rs_words);
     g->rs_words = nullptr; g->rs_xch = nullptr; g->rs_seq = nullptr;
@@ -80,7 +80,7 @@ void free_ensemble(flood_grid* g)
     g->plan = nullptr; g->log = nullptr; g->ckpt = nullptr; g->seg = nullptr;
     g->lam = nullptr; g->gnm = nullptr; g->gn_out = nullptr; g->gpart = nullptr;
     g->seg_end = nullptr; g->samp_step = nullptr; g->samp_y = nullptr; g->samp_d = nullptr;
-    g->samp_cells = nullptr; g->log_cap = 0; g->ckpt_floats = 0; g->seg_floats = 0;
+    g->samp_cells = nullptr; g->vol0 = nullptr; g->log_cap = 0; g->ckpt_floats = 0; g->seg_floats = 0;
     g->adj_room = flood_grid::AdjointRoom{};
     g->logging = false;
     g->state = nullptr; g->rain_mult = nullptr; g->scale = nullptr; g->hyeto = nullptr;
@@ -116,7 +116,7 @@ StepArgs step_args(const flood_grid* g, double t_end)
     a.plan = g->plan;
     a.log = g->logging ? g->log : nullptr;
     a.dt_log_cap = g->log_cap;
-    a.ckpt = g->logging ? g->ckpt : nullptr;
+    a.ckpt = !g->logging ? nullptr : g->kept ? g->kept : g->ckpt;
     a.ckpt_every = g->ckpt_every > 0 ? g->ckpt_every : 1;
     a.slots = g->logging && g->slots ? 1 : 0;
     a.err = g->err;
@@ -628,6 +628,7 @@ int flood_destroy(flood_grid* g)
     dfree(g->tiles);
     dfree(g->prod_u);
     dfree(g->zc);
+    if (g->kept_any) flood::trim_state_pool();
     delete g;
     return FLOOD_OK;
 }

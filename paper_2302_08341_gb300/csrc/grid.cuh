@@ -94,6 +94,8 @@ struct flood_grid {
     float* ckpt = nullptr;        // [n_ckpt][M][3][plane]
     size_t ckpt_floats = 0;
     int ckpt_every = 0;
+    float* kept = nullptr;        // [cap + 1][M][3][plane] every state of a window, during its adjoint
+    bool kept_any = false;        // some adjoint kept its states
     bool slots = false;           // the logged forward steps from checkpoint slot to slot
     CUtensorMap ckpt_map;         // the checkpoint slots, for such steps
     float* seg = nullptr;         // [slots][M][3][plane]
@@ -107,8 +109,9 @@ struct flood_grid {
     float* samp_y = nullptr;      // [ns][M][G]
     double* samp_d = nullptr;     // [ns][G]
     int32_t* samp_cells = nullptr;
+    double* vol0 = nullptr;       // the volume counters at the window's start
     struct AdjointRoom {          // values each of the adjoint's buffers holds
-        size_t log = 0, samp_y = 0, samp_cells = 0, lam = 0, gpart = 0, seg_end = 0, samp_step = 0,
+        size_t vol0 = 0, log = 0, samp_y = 0, samp_cells = 0, lam = 0, gpart = 0, seg_end = 0, samp_step = 0,
                samp_d = 0, gnm = 0, gn_out = 0, gdpart = 0;
     } adj_room;
     double adj_fwd_ms = 0.0, adj_rev_ms = 0.0;
@@ -171,6 +174,7 @@ int dalloc(flood_grid* g, T** p, size_t count)
 StepArgs step_args(const flood_grid* g, double t_end);
 int auto_rows(flood_grid* g);   // the automatic strip height, with or without tracked maxima
 int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s);
+void trim_state_pool();         // memory kept for the adjoints' states (adjoint_capi.cu)
 int read_clocks(flood_grid* g, std::vector<MemberClock>& out, cudaStream_t s);
 // Whether the next steps run on the chip (step_resident.cu).
 bool steps_resident(const flood_grid* g);

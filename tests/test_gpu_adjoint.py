@@ -391,3 +391,41 @@ def test_an_error_within_a_window_leaves_the_states_it_came_to(capi, shape):
     for a, b in zip(*res):
         np.testing.assert_array_equal(a, b)
     assert not np.array_equal(res[0][1], res[0][1 + 3 * M + 1])   # the state moved on
+
+
+def test_kept_states_leave_the_memory_to_other_allocations(capi):
+    """The states that ckpt_every = 0 keeps (4 GB here) are not held against
+    the rest of the program: after the call an allocation of nearly all that
+    was free before it succeeds, and the next call gives the same gradients."""
+    import ctypes
+    import torch
+    ny, nx, M = 600, 640, 8
+    terr = synth.make_terrain(ny, nx, seed=73, building_frac=0.0)
+    rm, sc = synth.ensemble_prior(73, M)
+    cells = synth.gauge_cells(terr, 4, seed=73)
+    d = np.full((1, 4), 0.1)
+    state = 12.0 * ny * nx * M                # bytes of one state of the ensemble
+    with capi.Grid(terr.z, terr.n) as g:
+        def adjoint():
+            g.ensemble_init(M, rm, sc, synth.hyetograph_constant(60.0, 600.0))
+            n0 = g.launch_count
+            out = g.adjoint(cells, d, 100.0, grad_h0=False)
+            return out, g.launch_count - n0
+        g.ensemble_init(M, rm, sc, synth.hyetograph_constant(60.0, 600.0))
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        a, launches = adjoint()
+        assert launches < 3 * 100 + 50        # plan, step and reverse: no replay, so the states were kept
+        # what stays with the ensemble: two sensitivities, a gradient field a member, the small arrays
+        ask = int(free - 3.0 * state - 256e6)
+        assert ask > free - 100 * state + 1e9
+        torch.cuda.empty_cache()
+        rt = ctypes.CDLL("libcudart.so.13")
+        p = ctypes.c_void_p()
+        rt.cudaMalloc.argtypes = [ctypes.POINTER(ctypes.c_void_p), ctypes.c_size_t]
+        rt.cudaFree.argtypes = [ctypes.c_void_p]
+        assert rt.cudaMalloc(ctypes.byref(p), ask) == 0
+        assert rt.cudaFree(p) == 0
+        b, _ = adjoint()
+    for k in ("loss", "grad_n", "grad_rain", "grad_scale"):
+        np.testing.assert_array_equal(a[k], b[k])
