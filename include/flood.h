@@ -507,12 +507,15 @@ int flood_set_graphs(flood_grid* g, int on);
  * replayed (either pointer may be NULL).  Errors: FLOOD_ERR_ARG. */
 int flood_graph_stats(flood_grid* g, int64_t* captures, int64_t* replays);
 
-/* Autotuner: time every step-kernel configuration (engine x rows per strip
- * {32, 64, 128} x members per CTA {8, 4, 2, 1}; 8 and 2 with the plain TMA
- * step only) for steps_per_trial steps on the
- * live ensemble, keep the fastest, and restore the ensemble (state, clocks,
- * volume counters) to where it was.  Writes the choice and its time per step
- * (ms); any output may be NULL.  Synchronous. */
+/* Autotuner: time the automatic shape (flood_set_launch 0, 0) and every
+ * step-kernel configuration of engine x rows per strip {32, 64, 128} x members
+ * per CTA {8, 4, 2, 1} (8 and 2 with the plain TMA step only), the best of five
+ * trials of steps_per_trial steps on the live ensemble each, keep the fastest
+ * (the earlier of two within 3 %, the automatic one first), and restore the
+ * ensemble (state, clocks, volume counters) to where it was.  Writes the choice
+ * and its time per step (ms); any output may be NULL.  Where the automatic
+ * shape keeps the steps on the chip, which has no strips, the shape written is
+ * the best of the others.  Synchronous. */
 int flood_autotune(flood_grid* g, int steps_per_trial, int* best_rows, int* best_mpc,
                    int* best_engine, double* best_ms, void* stream);
 

@@ -328,6 +328,35 @@ def test_autotune_leaves_the_ensemble_untouched(capi):
     assert np.array_equal(res[0][2]["steps"], res[1][2]["steps"])
 
 
+def test_autotune_keeps_no_slower_shape_than_the_automatic_one(capi):
+    """The automatic strip height lies between the listed ones and competes
+    with them: at 1000 x 1000 x 16 the best listed shape is 13 % slower.  The
+    tuned steps take at most 6 % more (the tuner's tie of 3 %, and as much for
+    the timing here)."""
+    import torch
+    terr = synth.make_terrain(1000, 1000, seed=16)
+    rm, sc = synth.ensemble_prior(16, 16)
+    with capi.Grid(terr.z, terr.n) as g:
+        g.ensemble_init(16, rm, sc, synth.hyetograph_constant(150.0, 600.0))
+        g.advance_to(60.0)
+
+        def us():
+            best = np.inf
+            for _ in range(6):
+                e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                e0.record()
+                g.step(12)
+                e1.record()
+                e1.synchronize()
+                best = min(best, e0.elapsed_time(e1) * 1e3 / 12)
+            return best
+
+        automatic = us()
+        rows, mpc, engine, _ = g.autotune(steps_per_trial=6)
+        assert (rows, mpc) == g.get_launch() and engine == 1
+        assert us() <= 1.06 * automatic
+
+
 @pytest.mark.parametrize("ny,nx", [(37, 129), (70, 300), (5, 7)])
 def test_wet_dry_threshold_one_step_on_dyadic_state(capi, ny, nx):
     """h_eps = 1e-3 m (links whose flow depth is at most 1 mm carry no flow):
