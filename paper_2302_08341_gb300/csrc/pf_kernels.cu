@@ -338,9 +338,11 @@ cudaError_t launch_pf(const PfArgs& a, cudaStream_t s)
     // the shared memory of more members is refused here, before anything is
     // launched that would read what the filter did not write
     if (a.M > kPfMaxMembers) return cudaErrorInvalidValue;
-    static const bool attr = cudaFuncSetAttribute(pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)pf_smem(kPfMaxMembers)) == cudaSuccess;
-    (void)attr;
+    if (pf_smem(a.M) > 32 * 1024) {  // each time: the attribute is the current device's
+        const cudaError_t e = cudaFuncSetAttribute(pf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)pf_smem(kPfMaxMembers));
+        if (e != cudaSuccess) return e;
+    }
     pf_kernel<<<1, kPfThreads, pf_smem(a.M), s>>>(a);
     return cudaGetLastError();
 }
