@@ -26,9 +26,9 @@ __global__ void batch_plan_kernel(const BatchArgs a, int n_scen)
         return sd.t_end < t_stop ? sd.t_end : t_stop;
     };
     // ahead of the wait, as plan_kernel does
-    PlanQuad<BatchArgs> w{a, lane, end(), sd.hyeto, nullptr, sd.nb, 0, 0, sd.rain_mult};
-    const uint32_t early = __ldcg(&a.ms_in[i].hmax_bits);
-    w.at(__ldcg(&a.ms_in[i].t));
+    PlanQuad<BatchArgs> w{a, lane, quad_first(end()), sd.hyeto, nullptr, sd.nb, 0, 0, sd.rain_mult};
+    const uint32_t early = quad_first(__ldcg(&a.ms_in[i].hmax_bits));
+    w.at(quad_first(__ldcg(&a.ms_in[i].t)));
     w.step(__uint_as_float(early));
     double v = (double)w.p.dr * a.cell_area;
     pdl_wait();

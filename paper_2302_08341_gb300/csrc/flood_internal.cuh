@@ -214,6 +214,15 @@ inline float capped_below(double alpha_dx, double g, double dt_cap)
 // A: StepArgs or BatchArgs.  The four lanes hold the same.
 constexpr int kPlanMembers = 8;  // of a warp
 
+// What the first of a plan's four lanes holds.  A word read ahead of the wait
+// may change meanwhile (the step before raises the maximum depth), so the lanes
+// take one reading of it: they decide and shuffle together afterwards.
+template <class T>
+__device__ __forceinline__ T quad_first(T v)
+{
+    return __shfl_sync(0xffffffffu, v, 0, 4);
+}
+
 template <class A>
 struct PlanQuad {
     const A& a;

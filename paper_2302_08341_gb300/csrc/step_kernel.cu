@@ -42,9 +42,9 @@ __global__ void plan_kernel(const StepArgs a)
     // is there since the step before was planned); whether they stayed is seen
     // after the wait
     PlanQuad<StepArgs> w{a, lane, a.t_end, a.hyeto, a.inflow, a.nb, a.inflow_blocks, a.in_r1 - a.in_r0,
-                         __ldcg(a.rain_mult + m)};
-    const uint32_t early = __ldcg(&a.ms_in[m].hmax_bits);
-    w.at(__ldcg(&a.ms_in[m].t));
+                         quad_first(__ldcg(a.rain_mult + m))};
+    const uint32_t early = quad_first(__ldcg(&a.ms_in[m].hmax_bits));
+    w.at(quad_first(__ldcg(&a.ms_in[m].t)));
     w.step(__uint_as_float(early));
     const double rows = (double)(a.in_r1 - a.in_r0);
     // the rain and inflow volumes, a lane each
