@@ -135,8 +135,7 @@ __global__ void __launch_bounds__(32 * W, 20 / W) batch_tma_kernel(const BatchAr
     const int lane = threadIdx.x;
     const int w = threadIdx.y;
     const int tid = blockIdx.x * W + w;
-    pdl_wait();
-    pdl_launch();  // after the wait: the next plan may then read the clocks this step's plan left
+    pdl_wait_launch();  // the next plan may then read the clocks this step's plan left
     if (tid >= a.ntasks) return;  // whole warps; no block-wide barriers below
     const WarpTask tk = a.tasks[tid];
     const int i = tk.scen;

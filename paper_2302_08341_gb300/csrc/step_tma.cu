@@ -31,8 +31,7 @@ __global__ void __launch_bounds__(32 * WM, tma_warps_per_sm(TRACK_MAX) / WM)
     const int w = threadIdx.y;
     const int m = blockIdx.x * WM + w;
     int span = blockIdx.y, strip = blockIdx.z;
-    pdl_wait();
-    pdl_launch();  // after the wait: the next plan may then read the clocks this step's plan left
+    pdl_wait_launch();  // the next plan may then read the clocks this step's plan left
     if (a.tiles) {  // only the tiles that hold a cell of the domain are launched
         const int64_t i = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
         if (i >= a.n_tiles) return;
