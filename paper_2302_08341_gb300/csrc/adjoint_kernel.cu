@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
     const bool act = c < nx;
     const int r0 = blockIdx.z * a.rows_per_strip;
     const int r1 = min(r0 + a.rows_per_strip, ny);
-    const float* __restrict__ lin = a.lam + ((size_t)a.lam_in * a.M + m) * mstride;
+    const float* const lin = a.lam + ((size_t)a.lam_in * a.M + m) * mstride;
     float* __restrict__ lout = a.lam + ((size_t)(1 - a.lam_in) * a.M + m) * mstride;
 
     const int j = a.seg_end[m] - 1 - a.rev_i;
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
             for (int r = r0; r < r1; ++r)
                 for (int k = 0; k < 3; ++k) {
                     const size_t o = k * plane + (size_t)r * ld + c;
-                    *reinterpret_cast<float4*>(lout + o) = ldg4(lin + o);
+                    *reinterpret_cast<float4*>(lout + o) = *reinterpret_cast<const float4*>(lin + o);
                 }
         return;
     }
@@ -79,11 +79,14 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
     const float s_half = 0.5f * s;
     const bool interior = c0 + kSpan < nx;  // no east edge in this span
 
-    const float* __restrict__ st = a.seg + ((size_t)(j - a.seg_first) * a.M + m) * mstride;
-    const float* __restrict__ sh = st;
-    const float* __restrict__ sqx = st + plane;
-    const float* __restrict__ sqy = st + 2 * plane;
-    const float* __restrict__ h1p = st + (size_t)a.M * mstride;  // depth after the step
+    // lambda and the states are the kernels' before this one, which may still run
+    // when this one takes its places: plain loads.  (The read-only path is for
+    // what stays as it is from a kernel's start to its end: bed, roughness.)
+    const float* const st = a.seg + ((size_t)(j - a.seg_first) * a.M + m) * mstride;
+    const float* const sh = st;
+    const float* const sqx = st + plane;
+    const float* const sqy = st + 2 * plane;
+    const float* const h1p = st + (size_t)a.M * mstride;  // depth after the step
     const float* __restrict__ z = a.z;
     const float* __restrict__ n = a.n + (size_t)m * a.n_mstride;
     float* __restrict__ gn = a.gn ? a.gn + (size_t)m * plane : nullptr;
@@ -96,7 +99,7 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
     };
     // a row's values (lambda~: zero where the step clamped)
     auto load_row = [&](size_t o) -> AdjRow {
-        return AdjRow{ldg_quad(sh + o), ldg_quad(z + o), ldg_quad(n + o), masked(ldg_quad(h1p + o), ldg_quad(lin + o))};
+        return AdjRow{ld_quad(sh + o), ldg_quad(z + o), ldg_quad(n + o), masked(ld_quad(h1p + o), ld_quad(lin + o))};
     };
     const AdjRow none{quad_of(0.0f), quad_of(0.0f), quad_of(0.0f), quad_of(0.0f)};
     AdjRow C = none;
@@ -106,7 +109,7 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
         C = load_row(o);
         if (r0 > 0) {  // the strip's north links, recomputed
             const size_t u = o - ld;
-            north_carry<LIM>(load_row(u), ldg_quad(sqy + u), ldg_quad(lin + 2 * plane + u), C, c, nx, k2, T, k, carH,
+            north_carry<LIM>(load_row(u), ld_quad(sqy + u), ld_quad(lin + 2 * plane + u), C, c, nx, k2, T, k, carH,
                              carN);
         }
     }
@@ -122,24 +125,24 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
         Quad qxo = quad_of(0.0f), qyo = qxo, lqx = qxo, lqy = qxo;
         if (act) {
             if (has_s) S = load_row(o + ld);
-            qxo = ldg_quad(sqx + o);
-            qyo = ldg_quad(sqy + o);
-            lqx = ldg_quad(lin + plane + o);
-            lqy = ldg_quad(lin + 2 * plane + o);
+            qxo = ld_quad(sqx + o);
+            qyo = ld_quad(sqy + o);
+            lqx = ld_quad(lin + plane + o);
+            lqy = ld_quad(lin + 2 * plane + o);
         }
         AdjSide E{__shfl_down_sync(0xffffffffu, C.h.a.x, 1), __shfl_down_sync(0xffffffffu, C.z.a.x, 1),
                   __shfl_down_sync(0xffffffffu, C.n.a.x, 1), __shfl_down_sync(0xffffffffu, C.l.a.x, 1), 0.0f, 0.0f};
         if (east_halo) {
             const size_t e = o + 4;
-            E.h = __ldg(sh + e); E.z = __ldg(z + e); E.n = __ldg(n + e);
-            E.l = masked(__ldg(h1p + e), __ldg(lin + e));
+            E.h = sh[e]; E.z = __ldg(z + e); E.n = __ldg(n + e);
+            E.l = masked(h1p[e], lin[e]);
         }
         AdjSide W{0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
         if (c0 > 0) {  // one cell for the whole warp
             const size_t w = (size_t)r * ld + c0 - 1;
-            W.h = __ldg(sh + w); W.z = __ldg(z + w); W.n = __ldg(n + w);
-            W.qx = __ldg(sqx + w); W.lqx = __ldg(lin + plane + w);
-            W.l = masked(__ldg(h1p + w), __ldg(lin + w));
+            W.h = sh[w]; W.z = __ldg(z + w); W.n = __ldg(n + w);
+            W.qx = sqx[w]; W.lqx = lin[plane + w];
+            W.l = masked(h1p[w], lin[w]);
         }
         Quad lh, lx, ly, gnr;
         float gr_row, gs_row;
@@ -151,7 +154,7 @@ __global__ void __launch_bounds__(32 * WM * WC, RW ? 3 : 4) adjoint_kernel(const
                 rwv = ldg_quad(a.rw + o);
                 const float4 d = ldg4(a.dflag + o);
                 dfv[0] = d.x; dfv[1] = d.y; dfv[2] = d.z; dfv[3] = d.w;
-                haC = ldg_quad(h1p + o);
+                haC = ld_quad(h1p + o);
             }
             kahan_add(gd_s, gd_c, drain_row(C.l, haC, dfv));
         }

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
     const bool act = c < nx;
     const int r0 = blockIdx.z * a.rows_per_strip;
     const int r1 = min(r0 + a.rows_per_strip, ny);
-    const float* __restrict__ lin = a.lam + ((size_t)a.lam_in * a.M + m) * mstride;
+    const float* const lin = a.lam + ((size_t)a.lam_in * a.M + m) * mstride;
     float* __restrict__ lout = a.lam + ((size_t)(1 - a.lam_in) * a.M + m) * mstride;
 
     const int j = a.seg_end[m] - 1 - a.rev_i;
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(32 * WM, WM == 4 ? 3 : 12) adjoint_tma_kernel(
             for (int r = r0; r < r1; ++r)
                 for (int q = 0; q < 3; ++q) {
                     const size_t o = q * plane + (size_t)r * ld + c;
-                    *reinterpret_cast<float4*>(lout + o) = ldg4(lin + o);
+                    *reinterpret_cast<float4*>(lout + o) = *reinterpret_cast<const float4*>(lin + o);
                 }
         return;
     }
