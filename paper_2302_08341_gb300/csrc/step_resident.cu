@@ -184,8 +184,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
     }
     MemberPlan mp{};             // the last plan
     mp.dt = -1.0;
-    Sum2 vout, vclamp;
-    float drn_s = 0.0f, drn_c = 0.0f;
+    Sum2 vout, vclamp, vdrn;     // over all steps of the launch: two words each
     bool bad = false;
     unsigned long long* const words[2] = {t.words + (size_t)m * t.bands,
                                           t.words + ((size_t)a.M + m) * t.bands};
@@ -377,7 +376,7 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
                     quad_at(v, i) = (hp > 0.0f && sink == hp) ? -0.0f : __fsub_rn(hp, sink);
                     row_sink = __fadd_rn(row_sink, sink);
                 }
-                kahan_add(drn_s, drn_c, row_sink);
+                vdrn.add(row_sink);
             }
             if (c + 4 > nx) {
 #pragma unroll
@@ -503,18 +502,13 @@ __global__ void __launch_bounds__(kThreads, 1) step_resident_kernel(const __grid
         if (a.inflow) a.inflow_acc[m] = inflow_acc;
         t.seq[m] = seq0 + (uint32_t)t.n_steps + 1u;
     }
-    Sum2 drained;
-    if (LC) {
-        drained.add(drn_s);
-        drained.lo = __fsub_rn(drained.lo, drn_c);
-        drained.warp_sum();
-    }
+    if (LC) vdrn.warp_sum();
     vout.warp_sum();
     vclamp.warp_sum();
     if (lane == 0) {
         s_red[0][warp] = make_float2(vout.hi, vout.lo);
         s_red[1][warp] = make_float2(vclamp.hi, vclamp.lo);
-        s_red[2][warp] = make_float2(drained.hi, drained.lo);
+        s_red[2][warp] = make_float2(vdrn.hi, vdrn.lo);
     }
     __syncthreads();
     if (tid < 3) {
