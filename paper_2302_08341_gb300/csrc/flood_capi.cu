@@ -70,7 +70,7 @@ void free_ensemble(flood_grid* g)
     dfree(g->samp_y); dfree(g->samp_d); dfree(g->samp_cells); dfree(g->vol0); dfree(g->closs);
     dfree(g->hmax_field); dfree(g->lc_n); dfree(g->lc_drain); dfree(g->dacc);
     dfree(g->rs_words);
-    g->rs_words = nullptr; g->rs_xch = nullptr; g->rs_seq = nullptr;
+    g->rs_words = nullptr; g->rs_xch = nullptr; g->rs_seq = nullptr; g->rs_refused = false;
     dfree(g->inflow_acc); dfree(g->lc_adj); dfree(g->lc_cgrad); dfree(g->gdpart); dfree(g->lc_dgrad);
     g->inflow_acc = nullptr; g->lc_adj = nullptr; g->lc_cgrad = nullptr; g->gdpart = nullptr;
     g->lc_dgrad = nullptr;
@@ -240,7 +240,7 @@ static int launch_one(flood_grid* g, double t_end, cudaStream_t s)
 // for that times or limits single step kernels.
 static bool resident_now(const flood_grid* g, ResidentShape* sh)
 {
-    if (!g->rs_words || g->engine != 1 || !g->maps_ok || g->profile || g->launch_fixed || g->wait_budget >= 0)
+    if (!g->rs_words || g->rs_refused || g->engine != 1 || !g->maps_ok || g->profile || g->launch_fixed || g->wait_budget >= 0)
         return false;
     *sh = resident_shape(g->ny, g->nx, g->M, g->n_sm, g->smem_max, g->track_max, g->lc_on);
     return sh->bands > 0;
@@ -274,8 +274,9 @@ static int resident_buffers(flood_grid* g, cudaStream_t s)
     return FLOOD_OK;
 }
 
-// n steps of every member in one launch.
-static int launch_resident_run(flood_grid* g, const ResidentShape& sh, int n, double t_end, cudaStream_t s)
+// n steps of every member in one launch.  False where the launch is refused (a
+// context that may not use all of the SMs, say): the ensemble marches from then on.
+static bool launch_resident_run(flood_grid* g, const ResidentShape& sh, int n, double t_end, cudaStream_t s)
 {
     ResidentArgs t{};
     t.a = step_args(g, t_end);
@@ -287,10 +288,14 @@ static int launch_resident_run(flood_grid* g, const ResidentShape& sh, int n, do
     t.bands = sh.bands;
     t.rows = sh.rows;
     t.n_steps = n;
-    CK(g, launch_resident(t, sh, s));
+    if (launch_resident(t, sh, s) != cudaSuccess) {
+        cudaGetLastError();
+        g->rs_refused = true;
+        return false;
+    }
     g->k += n;
     g->launches++;
-    return FLOOD_OK;
+    return true;
 }
 
 // Steps per captured run: a multiple of the member-clock ring's period (3),
@@ -349,8 +354,9 @@ static int ensure_graph(flood_grid* g, double t_end)
     CK(g, cudaStreamBeginCapture(g->cap_stream, cudaStreamCaptureModeRelaxed));
     int rc = FLOOD_OK;
     ResidentShape sh;
+    bool refused = false;
     if (resident_now(g, &sh))
-        rc = launch_resident_run(g, sh, kGraphSteps, t_end, g->cap_stream);
+        refused = !launch_resident_run(g, sh, kGraphSteps, t_end, g->cap_stream);
     else
         for (int i = 0; i < kGraphSteps && rc == FLOOD_OK; ++i) rc = launch_one(g, t_end, g->cap_stream);
     cudaGraph_t graph = nullptr;
@@ -359,6 +365,10 @@ static int ensure_graph(flood_grid* g, double t_end)
     g->k = k0;
     g->launches = l0;
     cudaGetLastError();  // a failed capture is reported below, not by the next check
+    if (refused) {  // the same run marching
+        if (graph) cudaGraphDestroy(graph);
+        return ensure_graph(g, t_end);
+    }
     if (rc != FLOOD_OK || ec != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
         return rc != FLOOD_OK ? rc
@@ -382,11 +392,10 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
     g->epoch++;
     int64_t i = 0;
     ResidentShape sh;
-    const bool res = resident_now(g, &sh);
     // up to `n` steps, however they run
     auto some = [&](int n) -> int {
         i += n;
-        if (res) return launch_resident_run(g, sh, n, t_end, s);
+        if (resident_now(g, &sh) && launch_resident_run(g, sh, n, t_end, s)) return FLOOD_OK;
         for (int q = 0; q < n; ++q) {
             const int rc = launch_one(g, t_end, s);
             if (rc) return rc;
@@ -398,7 +407,7 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
     // phase 0 and the remainder launch plainly.  Resident steps run in the
     // same pieces with and without graphs
     const bool graphs = g->graphs && !g->profile && !g->logging;
-    if ((graphs || res) && count >= kGraphSteps + 2) {
+    if ((graphs || resident_now(g, &sh)) && count >= kGraphSteps + 2) {
         if (g->k % 3 != 0) {
             const int rc = some((int)(3 - g->k % 3));
             if (rc) return rc;
@@ -410,7 +419,7 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
         // a resident launch costs about 5 us beside its steps (256 x 256 x 1,
         // 300 steps: runs of 24 833 us, of up to 240 753 us); longer ones
         // would hold the SMs for milliseconds
-        while (res && count - i >= 11 * kGraphSteps) {
+        while (resident_now(g, &sh) && count - i >= 11 * kGraphSteps) {
             const int rc = some(10 * kGraphSteps);
             if (rc) return rc;
         }
@@ -428,7 +437,7 @@ int launch_steps(flood_grid* g, int64_t count, double t_end, cudaStream_t s)
         }
     }
     while (i < count) {
-        const int rc = some(res ? (int)(count - i) : 1);
+        const int rc = some(resident_now(g, &sh) ? (int)(count - i) : 1);
         if (rc) return rc;
     }
     CK(g, cudaGetLastError());

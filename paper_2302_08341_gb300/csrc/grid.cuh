@@ -49,6 +49,7 @@ struct flood_grid {
     unsigned long long* rs_words = nullptr;  // one block: band words, exchange rows, step numbers
     unsigned long long* rs_xch = nullptr;
     uint32_t* rs_seq = nullptr;
+    bool rs_refused = false;      // their launch was refused: this ensemble marches
     // particle filter
     int G = 0, G_cap = 0;
     int32_t* cells = nullptr;     // [G_cap]

@@ -1,6 +1,10 @@
 """GPU steps that stay on the chip, further: that they are the ones that ran,
 options beside those of test_gpu_resident.py, and the volumes they sum over
 many steps at once."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -41,3 +45,43 @@ def test_drained_volume_of_many_steps_in_one_launch(capi, shape):
         assert np.array_equal(a, b)
     assert res[1][0].min() > 0.0
     assert np.all(np.abs(res[0][0] - res[1][0]) <= 2.0 ** -34 * res[1][0])
+
+
+_REFUSED = """
+import sys
+sys.modules["torch"] = None
+import numpy as np
+from paper_2302_08341_gb300 import capi, synth
+terr = synth.make_terrain(64, 131, seed=98)
+rm, sc = synth.ensemble_prior(98, 7)
+res = []
+for march, graphs in ((True, False), (False, False), (False, True)):
+    with capi.Grid(terr.z, terr.n) as g:
+        g.ensemble_init(7, rm, sc, synth.hyetograph_constant(60.0, 600.0))
+        g.set_graphs(graphs)
+        if march:
+            g.set_launch(8, 1)
+        n0 = g.launch_count
+        g.step(60)
+        g.advance_to(90.0)
+        assert g.launch_count - n0 >= 2 * 90, "the steps did not march"
+        res.append([np.stack(g.get_state(m)) for m in range(7)])
+for r in res[1:]:
+    for a, b in zip(res[0], r):
+        assert np.array_equal(a, b)
+print("done")
+"""
+
+
+def test_a_refused_cooperative_launch_falls_back_to_the_march(capi, tmp_path):
+    """The runtime's cooperative launch replaced by one that returns its error
+    (cudaErrorCooperativeLaunchTooLarge): the steps march, plainly and from a
+    graph, with the same results."""
+    shim = tmp_path / "refuse.c"
+    shim.write_text("int cudaLaunchCooperativeKernel() { return 720; }\n")
+    lib = tmp_path / "refuse.so"
+    subprocess.run(["gcc", "-shared", "-fPIC", "-o", str(lib), str(shim)], check=True)
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _REFUSED], cwd=root, capture_output=True, text=True, timeout=120,
+                       env=dict(os.environ, LD_PRELOAD=str(lib)))
+    assert r.returncode == 0 and "done" in r.stdout, r.stderr
