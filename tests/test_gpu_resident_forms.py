@@ -47,6 +47,75 @@ def test_drained_volume_of_many_steps_in_one_launch(capi, shape):
     assert np.all(np.abs(res[0][0] - res[1][0]) <= 2.0 ** -34 * res[1][0])
 
 
+def _forms(capi, shape, march, params, land, track, stream=None):
+    import torch
+    ny, nx, M = shape
+    rng = np.random.default_rng(101)
+    terr = synth.make_terrain(ny, nx, seed=101)
+    rm, sc = synth.ensemble_prior(101, M)
+    h0 = rng.uniform(0.0, 1.5, (M, ny, nx)).astype(np.float32)
+    h0[:, ::3, ::2] = 0.0
+    with capi.Grid(terr.z, terr.n, capi.Params.default(**params)) as g:
+        if land:
+            cls = rng.integers(0, 4, (ny, nx))
+            cls[: max(1, ny // 5)] = 3                          # outside the domain, and scattered cells
+            g.set_land_cover(cls, synth.LAND_CLASSES)
+        with torch.cuda.stream(stream) if stream else torch.cuda.stream(torch.cuda.current_stream()):
+            g.ensemble_init(M, rm, sc, synth.hyetograph_triangular(60.0, 30.0, 60.0), h0=h0)
+            if land:
+                g.set_land_params(*synth.land_prior(101, M))
+            if track:
+                g.track_max_depth(True)
+            if march:
+                g.set_launch(8, 1)
+            n0 = g.launch_count
+            g.step(31)
+            launches = g.launch_count - n0
+            g.advance_to(90.0)
+            g.sync()
+            out = [x for m in range(M) for x in g.get_state(m)]
+            if track:
+                out += [g.max_depth(m) for m in range(M)]
+            y = g.gauge_sample(np.array([0, ny * nx // 2, ny * nx - 1], np.int32))
+        mem = g.members()
+        out += [y, mem["t"], mem["steps"], mem["hmax"], g.volumes()["storage"], g.volumes()["rain"]]
+        # resident: 31 steps are at most a launch to the ring's first slot, one of 24 and the rest
+        assert launches == 62 if march else launches <= 3
+        return out
+
+
+@pytest.mark.parametrize("shape", [(1, 9, 3), (64, 131, 7), (40, 129, 76), (305, 310, 1)])
+@pytest.mark.parametrize("options", [dict(params=dict(limiter=0)), dict(params=dict(east_outflow=0)),
+                                     dict(params=dict(east_outflow=0, south_outflow=1, limiter=0)),
+                                     dict(params=dict(), land=True),
+                                     dict(params=dict(south_outflow=1, limiter=0), land=True, track=True)])
+def test_resident_steps_ran_and_equal_the_march(capi, shape, options):
+    """The limiter off, closed and open edges, land cover with cells and whole
+    rows outside the domain: states, clocks, maxima, gauges, storage and rain
+    bit for bit, and the launches counted are those of resident steps."""
+    if options.get("land") and shape[0] < 5:
+        pytest.skip("no row would be inside the domain")
+    o = dict(dict(land=False, track=False), **options)
+    a = _forms(capi, shape, False, **o)
+    b = _forms(capi, shape, True, **o)
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("march", [False, True])
+def test_every_call_on_a_side_stream(capi, march):
+    """An ensemble made, stepped and read on a non-blocking stream while the
+    default stream is busy: as on the default stream."""
+    import torch
+    shape, o = (64, 131, 7), dict(params=dict(), land=True, track=True)
+    ref = _forms(capi, shape, march, **o)
+    side = torch.cuda.Stream()
+    torch.cuda._sleep(200_000_000)
+    got = _forms(capi, shape, march, stream=side, **o)
+    for x, y in zip(ref, got):
+        assert np.array_equal(x, y)
+
+
 _REFUSED = """
 import sys
 sys.modules["torch"] = None
