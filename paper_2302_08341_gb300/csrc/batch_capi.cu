@@ -122,7 +122,8 @@ int build_tasks(flood_batch* b)
     if (!b->launch_fixed) {  // as the ensemble's automatic strip height
         int64_t rows = 0;
         for (int e = 0; e < b->S; ++e) rows += (int64_t)b->ny[e] * ((b->nx[e] + kSpan - 1) / kSpan);
-        b->rows_per_strip = flood::strip_rows(rows, b->n_sm, false);
+        const bool lc = std::any_of(b->lc.begin(), b->lc.end(), [](int v) { return v != 0; });
+        b->rows_per_strip = flood::strip_rows(rows, b->n_sm, false, lc, lc ? 5 : 16);
     }
     b->tasks.clear();
     b->slot0.assign(b->S, 0);

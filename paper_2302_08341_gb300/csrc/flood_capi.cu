@@ -502,12 +502,12 @@ namespace {
 
 // The automatic strip height of the TMA step (strip_rows).  The strips of a
 // span lie along grid.z, which holds 65535.
-int choose_rows_per_strip(int ny, int nx, int M, int n_sm, bool track)
+int choose_rows_per_strip(int ny, int nx, int M, int n_sm, bool track, bool lc)
 {
     const int64_t spans = (int64_t)M * ((nx + 127) / 128);
     // strips do not cross members or spans: round the strips per span down
-    int rh = flood::strip_rows(spans * ny, n_sm, track);
-    while (rh < (track ? 9 : 12) && spans * ((ny + rh - 1) / rh) > (int64_t)n_sm * (track ? 16 : 20)) ++rh;
+    int rh = flood::strip_rows(spans * ny, n_sm, track, lc, lc && !track ? 5 : 0);
+    while (rh < flood::strip_few(track, lc) && spans * ((ny + rh - 1) / rh) > (int64_t)n_sm * (track ? 16 : 20)) ++rh;
     return std::min(std::max(rh, (ny + 65534) / 65535), 4096);
 }
 
@@ -529,7 +529,7 @@ namespace flood {
 int auto_rows(flood_grid* g)
 {
     if (g->launch_fixed || !g->M) return FLOOD_OK;
-    const int rh = choose_rows_per_strip(g->ny, g->nx, g->M, g->n_sm, g->track_max);
+    const int rh = choose_rows_per_strip(g->ny, g->nx, g->M, g->n_sm, g->track_max, g->lc_on);
     const int rc = ensure_vacc(g, step_nslot(g->ny, g->nx, rh));
     if (rc == FLOOD_OK) g->rows_per_strip = rh;
     return rc;
@@ -658,14 +658,16 @@ int flood_ensemble_init(flood_grid* g, int M, const float* h0, int h0_per_member
     g->M = M;
     g->nb = n_blocks;
     if (!g->launch_fixed) {
-        g->rows_per_strip = choose_rows_per_strip(g->ny, g->nx, M, g->n_sm, false);
+        g->rows_per_strip = choose_rows_per_strip(g->ny, g->nx, M, g->n_sm, false, g->lc_on);
         g->members_per_cta = choose_members_per_cta(M);
     }
     // (a band of resident steps takes a slot too, where there are any: a volume
     // report copies and adds up every slot, 3000 members of 64 x 64 in 172 us,
     // with a slot for each SM 661)
-    g->nslot = std::max({flood::step_nslot(g->ny, g->nx, g->rows_per_strip),
-                         flood::step_nslot(g->ny, g->nx, choose_rows_per_strip(g->ny, g->nx, M, g->n_sm, true)),
+    int shortest = g->rows_per_strip;
+    for (int v = 0; v < 4; ++v)  // with and without tracked maxima and land cover
+        shortest = std::min(shortest, choose_rows_per_strip(g->ny, g->nx, M, g->n_sm, v & 1, v & 2));
+    g->nslot = std::max({flood::step_nslot(g->ny, g->nx, shortest),
                          flood::resident_shape(g->ny, g->nx, M, g->n_sm, g->smem_max, false, false).bands});
     g->part_cap = (g->ny + 15) / 16;
     const size_t pf_doubles = (size_t)M + 1 + 2 + 2 * (size_t)M;  // w_post, neff, the flags, idx to copy_src

@@ -531,7 +531,10 @@ int encode_map_3d_u8(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d
                      uint32_t b2);
 int step_nslot(int ny, int nx, int rows_per_strip);
 // Rows per strip for a step over `warp_rows` rows of 128-column spans (of all
-// members) on a GPU that holds `warps` of the kernel's warps at a time.
-int strip_rows(int64_t warp_rows, int n_sm, bool track);
+// members), with or without tracked maxima and land cover; tall: the rounds of
+// 24-row strips from which those are taken (0: never).
+int strip_rows(int64_t warp_rows, int n_sm, bool track, bool lc, int tall);
+// The height where strips take several rounds.
+int strip_few(bool track, bool lc);
 
 }  // namespace flood

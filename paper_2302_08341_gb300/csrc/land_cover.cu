@@ -402,7 +402,7 @@ extern "C" int flood_set_land_cover(flood_grid* g, const uint8_t* cls, int n_cla
     g->lc_on = true;
     g->epoch++;
     if (g->M && (rc = flood::land_ensemble_init(g))) return rc;
-    return FLOOD_OK;
+    return flood::auto_rows(g);
 }
 
 extern "C" int flood_set_land_params(flood_grid* g, const float* n_class, const float* drain_rate)

@@ -186,20 +186,27 @@ int step_nslot(int ny, int nx, int rows_per_strip)
 //  - all strips resident at once with at most 12 rows: the shortest such
 //    strips (1024 x 1024 x 1: 3 rows 14, 8 rows 16.5; 2000 x 2000 x 1: 12 rows
 //    32, 4 rows 34; 600 x 707 x 8: 12 rows 28, 8 rows (1.2 rounds) 33);
-//  - a few rounds of strips: 12 rows (1000 x 1000 x 16: 12 rows 83, 32 rows 96,
-//    4 rows 100; 2000 x 2000 x 8: 145, 148, 179); where the maxima are tracked
-//    and an SM holds 16 warps, 9 (777 x 1013 x 12: 59.8, 12 rows 62.2; 1000 x
-//    1000 x 24: 129.5, 132.5);
-//  - from about five rounds of 24 rows on, 24 (2000 x 2000 x 96: 24 rows 1420,
-//    64 rows 1533, 12 rows 1486; 1200 x 1310 x 32 with land cover: 201, 217 (48
-//    rows), 206; neighbouring strips' halo rows then still meet in L2).
-int strip_rows(int64_t warp_rows, int n_sm, bool track)
+//  - more: 12 rows, of eleven sizes from 2.6 to 42 rounds of 24-row strips the
+//    best at eight and within 1 % at the others (1000 x 1000 x 24: 9 rows 109.6,
+//    12 108.4, 24 113.2; 2000 x 2000 x 16: 259, 255, 262; 2000 x 2000 x 96: 1440,
+//    1393, 1418); with tracked maxima, where an SM holds 16 warps, 9, the best
+//    of all eleven (1000 x 1000 x 24: 128, 132, 140; 2000 x 2000 x 32: 627, 638,
+//    673); with both tracked maxima and land cover 12 (133, 132, 139; 619, 597, 625);
+//  - 24 where the caller's rows make that many rounds of them (tall; 0: never).
+//    Ensembles with land cover from five on (1000 x 1000 x 24, 2.6 rounds: 12
+//    rows 115.9, 24 117.4; 1200 x 1310 x 32, 5.8: 226, 223; 2000 x 2000 x 32, 14:
+//    512, 491); batches, whose strips share no bed, with land cover from five on
+//    (64 scenarios, 5.1: 249.6, 250.5; 24 x 2, 10.6: 442, 424), without from
+//    sixteen (5.1: 249, 252; 10.6: 440, 443; 64 x 4, 20.5: 786, 767).
+int strip_few(bool track, bool lc) { return track && !lc ? 9 : 12; }
+
+int strip_rows(int64_t warp_rows, int n_sm, bool track, bool lc, int tall)
 {
     const int64_t warps = (int64_t)n_sm * (track ? 16 : 20);
     const int64_t one = (warp_rows + warps - 1) / warps;  // rows a warp when all are resident
-    const int few = track ? 9 : 12;
+    const int few = strip_few(track, lc);
     if (one <= few) return (int)(one < 1 ? 1 : one);
-    return warp_rows >= warps * 24 * 5 ? 24 : few;
+    return tall && warp_rows >= warps * 24 * tall ? 24 : few;
 }
 
 // members_per_cta: warps of one CTA hold this many members of the same span
