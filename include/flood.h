@@ -122,8 +122,12 @@ int flood_ensemble_init(flood_grid* g, int n_members, const float* h0, int h0_pe
  *   t_end >= 0  advance every member to t_end (members already there stay
  *               put).  n_steps <= 0: no limit on steps, > 0: at most n_steps
  *               steps.  Synchronises `stream` to follow the members' clocks.
- * Each step is a plan kernel then a step kernel on `stream`; with
- * flood_set_graphs, runs of 24 steps are replayed from a CUDA graph instead.
+ * Each step is a plan kernel then a step kernel on `stream`; where the members'
+ * states fit in the SMs' shared memory, up to 240 steps are one cooperative
+ * launch instead (not with a shape set by flood_set_launch, another engine,
+ * flood_profile or a wait budget).  With flood_set_graphs, runs of 24 steps are
+ * replayed from a CUDA graph.  The results are the same bit for bit, but for
+ * the last digits of the outflow, clamp and drained volumes.
  * Errors: FLOOD_ERR_STATE before flood_ensemble_init, FLOOD_ERR_NAN if a
  * depth became non-finite (detected at the synchronisation points),
  * FLOOD_ERR_CUDA.

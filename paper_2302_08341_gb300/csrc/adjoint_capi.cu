@@ -1,11 +1,12 @@
-// flood_adjoint: gradients of a gauge-misfit loss by reverse mode with
-// checkpointing (extension beyond the paper).  Forward: the ensemble advances
-// through the observation times exactly as flood_step would, logging each
-// member's step lengths and storing its state every ckpt_every steps.
-// Reverse: segment by segment from the last, the segment's states are
-// recomputed bit for bit from its checkpoint (replay kernel), then the
-// adjoint kernel runs backwards through them, seeded with the loss
-// sensitivities at the observation times.
+// flood_adjoint: gradients of a gauge-misfit loss by reverse mode (extension
+// beyond the paper).  Forward: the ensemble advances through the observation
+// times exactly as flood_step would, logging each member's step lengths and
+// keeping every state where memory allows (the steps then go from slot to slot
+// of the kept states), else storing its state every ckpt_every steps.  Reverse:
+// the adjoint kernel runs backwards through the states, seeded with the loss
+// sensitivities at the observation times; from checkpoints segment by segment
+// from the last, the segment's states recomputed bit for bit before (replay
+// kernel).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -86,7 +87,7 @@ StatePool state_pool()
         cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &most);
     }
     cudaGetLastError();
-    return pools[dev] = p;
+    return p.pool ? pools[dev] = p : p;  // (a refusal may pass: asked again next time)
 }
 
 // The kept states of one call.

@@ -44,9 +44,10 @@ namespace flood {
 namespace {
 
 constexpr int kThreads = 512;
-// Clock cycles a band may wait for another (about 2 s): the launch is
-// cooperative, but a kernel of another stream can hold an SM for a while
-// before the last band gets its place.
+// Clock cycles a band may wait for another (about 2 s; a step takes
+// microseconds).  The launch is cooperative, so no band starts before all have
+// their places: a kernel of another stream that held an SM's shared memory for
+// 3 s held the launch up for as long, and no wait ran out.
 constexpr long long kBandWaitBudget = 4000000000LL;
 constexpr int kWarps = kThreads / 32;
 constexpr int kWords = 5;      // 152 bands: a member's most

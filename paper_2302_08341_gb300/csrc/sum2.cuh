@@ -3,7 +3,8 @@
 
 namespace flood {
 
-// A sum kept in two FP32 words (hi + lo, about 2^-46 relative).  The FP64 pipe
+// A sum kept in two FP32 words (hi + lo, about 2^-46 relative): Knuth's
+// error-free addition, the errors added up beside the sum.  The FP64 pipe
 // takes 64 cycles a warp instruction and a division fifteen of them, so what
 // every warp sums stays off it and one lane widens the total at the end: a
 // warp's five-round FP64 sum over its lanes cost a strip some 2400 cycles.

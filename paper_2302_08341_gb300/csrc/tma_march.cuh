@@ -24,9 +24,9 @@
 // bed and roughness are read again from its stage rather than carried over,
 // so the row loop needs no unrolling to stay free of moves; the row is
 // compiled apart for spans without the grid's last column and for its last
-// row: 350 instructions a row.  2000 x 2000 cells x 96 members: 1.63 -> 1.42 ms
-// per step, where memory binds (96 % of the measured copy rate); 1000 x 1000 x
-// 16: 105 -> 83 us.
+// row: 350 instructions a row.  2000 x 2000 cells x 96 members: 1.63 -> 1.39 ms
+// per step, where memory binds (7.2 TB/s at 26 bytes a cell, of which some 23
+// reach DRAM); 1000 x 1000 x 16: 105 -> 79 us.
 // Two spans a warp (one wait and one link west for 256 cells, 12 warps per SM
 // instead of 20) measured the same or slower at every size but one.
 #pragma once
@@ -249,8 +249,11 @@ __device__ __forceinline__ bool tma_march(const CUtensorMap* state_map, const CU
         if (TRACK_MAX) hmo = ld_quad(R + kTmaHmOff / 4 + 4 * lane);
         // with tracked maxima (16 warps an SM and registers to spare) the row
         // goes into registers whole and its stage takes a later row before the
-        // arithmetic (777 x 1013 x 12, 80 steps: 5.55 -> 5.39 ms); with 20 warps
-        // that costs more than it hides (1000 x 1000 x 16: 5.76 -> 6.22 ms)
+        // arithmetic: over twenty sizes 0.1 to 2.4 % less a step (us: 777 x 1013 x
+        // 12 60.3 -> 59.6, 1200 x 1310 x 32 259.1 -> 253.0, 2000 x 2000 x 24 480.5
+        // -> 480.1; with land cover 1000 x 1000 x 24 136.3 -> 133.2, 1500 x 1500 x
+        // 40 441.3 -> 432.0); with 20 warps that costs more than it hides (1000 x
+        // 1000 x 16, 68 steps: 5.76 -> 6.22 ms)
         if (TRACK_MAX) release(r, sC);
         const Quad uC = bounds(hC);
         Quad qE, qS, nS;
