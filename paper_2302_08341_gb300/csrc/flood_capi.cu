@@ -240,8 +240,8 @@ static int launch_one(flood_grid* g, double t_end, cudaStream_t s)
 // for that times or limits single step kernels.
 static bool resident_now(const flood_grid* g, ResidentShape* sh)
 {
-    if (!g->rs_words || g->rs_refused || g->engine != 1 || !g->maps_ok || g->profile || g->launch_fixed || g->wait_budget >= 0)
-        return false;
+    if (!g->rs_words || g->rs_refused || g->engine != 1 || !g->maps_ok) return false;
+    if (g->profile || g->launch_fixed || g->wait_budget >= 0) return false;
     *sh = resident_shape(g->ny, g->nx, g->M, g->n_sm, g->smem_max, g->track_max, g->lc_on);
     return sh->bands > 0;
 }
